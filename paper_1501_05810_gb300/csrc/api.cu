@@ -70,14 +70,15 @@ static bool alloc_contact_arrays(nbgs_scene* s, int64_t cap)
     if (!ok) return false;
     s->srec = dev_alloc(s, c * rec_bytes(s));
     s->sp = dev_alloc(s, c * vec4_bytes(s));
-    return s->srec && s->sp;
+    s->spre = dev_alloc(s, c * (s->fp32 ? sizeof(SweepPre<float>) : sizeof(SweepPre<double>)));
+    return s->srec && s->sp && s->spre;
 }
 
 static void free_contact_arrays(nbgs_scene* s)
 {
     void* ps[] = {s->cj1, s->cj2, s->cgeo, s->clev, s->cimp, s->cworld, s->prev_j2, s->prev_P, s->adj, s->cstate,
                   s->cprio, s->wl[0], s->wl[1], s->colour_key, s->colour_key2, s->perm, s->perm_in, s->srec, s->sp,
-                  s->cpack};
+                  s->spre, s->cpack};
     for (void* p : ps) dev_free(s, p);
 }
 

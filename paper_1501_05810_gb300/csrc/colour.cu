@@ -21,7 +21,7 @@
 #include <algorithm>
 #include <utility>
 
-#include "nbgs_internal.cuh"
+#include "relax.cuh"
 
 namespace nbgs {
 
@@ -474,6 +474,26 @@ __global__ void k_colour_offsets(const uint32_t* __restrict__ col_count, uint32_
     }
 }
 
+// One end of a contact's dependency word from the colours of its body's
+// contacts (mask, 256 bits): the colour below c and whether c is the highest.
+__device__ __forceinline__ uint32_t dep_end(const uint32_t* __restrict__ mask, uint32_t c)
+{
+    const uint4* q = reinterpret_cast<const uint4*>(mask);
+    const uint4 lo = q[0], hi = q[1];
+    const uint32_t m[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    const uint32_t wd = c >> 5, bit = c & 31u;
+    uint32_t pred = 0u;
+    bool last = true;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) {
+        const uint32_t below = k < wd ? m[k] : (k == wd ? m[k] & ((1u << bit) - 1u) : 0u);
+        const uint32_t above = k > wd ? m[k] : (k == wd ? (m[k] >> bit) >> 1 : 0u);
+        if (below) pred = 32u * k + 32u - (uint32_t)__clz((int)below);   // colour + 1
+        if (above) last = false;
+    }
+    return pred | (last ? kDepLastA : 0u) | kDepListA;
+}
+
 // Slot of every canonical contact in colour order: the inverse of perm.
 __global__ void k_invert(DCount Cc, const uint32_t* __restrict__ perm, uint32_t* __restrict__ inv)
 {
@@ -493,8 +513,10 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
                               const double2* __restrict__ clev, double dt, double beta, double mu_all, SceneView V,
                               int warm,
                               const uint32_t* __restrict__ prev_row_off, const uint32_t* __restrict__ prev_j2,
-                              const double4_32a* __restrict__ prev_P, int64_t prev_cap, SweepRec<R>* __restrict__ rec,
-                              R4<R>* __restrict__ p)
+                              const double4_32a* __restrict__ prev_P, int64_t prev_cap,
+                              const uint32_t* __restrict__ cstate, const uint4* __restrict__ cpack,
+                              const uint32_t* __restrict__ mask, const R4<R>* __restrict__ vel,
+                              SweepRec<R>* __restrict__ rec, R4<R>* __restrict__ p, SweepPre<R>* __restrict__ pre)
 {
     const int64_t C = Cc.get();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
@@ -516,13 +538,37 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
             r.ids_bias = make_double2(__longlong_as_double((long long)(((uint64_t)rb << 32) | ra)), bias);
             r.lev = make_double2(l.x, l.y);
             r.nxy = make_double2(g.x, g.y);
-            r.nz_ = make_double2(g.z, 0.0);
+            // the factor of the tangent basis (tangent_basis)
+            r.nz_ = make_double2(g.z, -1.0 / (copysign(1.0, g.z) + g.z));
         }
         rec[s] = r;
+        if (mask) {
+            const bool dyn_b = b < (uint64_t)n;
+            const R ima = vel[2 * (int64_t)a].w, iIa = vel[2 * (int64_t)a + 1].w;
+            const R imb = dyn_b ? vel[2 * (int64_t)b].w : R(0), iIb = dyn_b ? vel[2 * (int64_t)b + 1].w : R(0);
+            SweepPre<R> x;
+            // the levers as the records hold them
+            const R la = (R)l.x, lb = (R)l.y, nz = (R)g.z;
+            const R wn = ima + imb, wt = wn + iIa * la * la + iIb * lb * lb;
+            x.m.x = ima;
+            x.m.y = imb;
+            x.m.z = la * iIa;
+            x.m.w = lb * iIb;
+            if constexpr (sizeof(R) == 4) x.w = make_float4(wt, 1.f / wn, 1.f / wt, -1.f / (copysignf(1.f, nz) + nz));
+            else x.w = make_double4_32a(wn, wt, 1.0 / wn, 1.0 / wt);
+            pre[s] = x;
+        }
         // the previous world impulse in the new contact frame, projected onto
         // the friction cone; in the sweep precision (FP64 arithmetic is scarce
         // on this GPU, and an FP32 sweep starts from an FP32 impulse anyway)
-        R pn = R(0), pt = R(0), po = R(0), found = R(0);
+        R pn = R(0), pt = R(0), po = R(0);
+        uint32_t dep = 0u;   // mask: the colours of every body's contacts (no subdomains)
+        if (mask) {
+            const uint32_t col = cstate[c] & 0xFFu;
+            const uint4 q = cpack[c];
+            if (q.x != kNoList) dep |= dep_end(mask + 8 * (int64_t)q.x, col);
+            if (q.y != kNoList) dep |= dep_end(mask + 8 * (int64_t)q.y, col) << 11;
+        }
         if (warm) {
             const uint32_t e = prev_row_off[a + 1];
             for (uint32_t t = prev_row_off[a]; t < e && t < prev_cap; ++t) {
@@ -530,7 +576,7 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
                 const double4_32a P = prev_P[t];
                 const R mu = (R)(V.batch ? V.mu[V.scene_of[a]] : mu_all);
                 const R nx = (R)g.x, ny = (R)g.y, nz = (R)g.z, Px = (R)P.x, Py = (R)P.y, Pz = (R)P.z;
-                found = R(1);
+                dep |= kDepFound;   // read by the network warm start
                 R tx, ty, tz, ox, oy, oz;
                 tangent_basis<R>(nx, ny, nz, tx, ty, tz, ox, oy, oz);
                 pn = nx * Px + ny * Py + nz * Pz;
@@ -553,7 +599,7 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
         q.x = pn;
         q.y = pt;
         q.z = po;
-        q.w = found;   // 1: the contact existed in the previous step (read by the network warm start)
+        dep_store(dep, q.w);
         p[s] = q;
     }
 }
@@ -702,14 +748,17 @@ nbgs_status run_colour(nbgs_scene* s)
                                                    s->clev, s->prm.dt,
                                                    s->prm.beta, s->prm.mu, scene_view(s), warm, s->prev_row_off,
                                                    s->prev_j2,
-                                                   s->prev_P, s->ccap, (SweepRec<float>*)s->srec, (float4*)s->sp);
+                                                   s->prev_P, s->ccap, s->cstate, s->cpack, sub ? nullptr : s->cmask,
+                                                   (const float4*)s->vel, (SweepRec<float>*)s->srec, (float4*)s->sp,
+                                                   (SweepPre<float>*)s->spre);
         else
             k_build_sweep<double><<<gb, T, 0, st>>>(Cn, n, s->perm_in, s->cj1, s->cj2, sub ? s->inst : nullptr, s->cgeo,
                                                     s->clev, s->prm.dt,
                                                     s->prm.beta, s->prm.mu, scene_view(s), warm, s->prev_row_off,
                                                     s->prev_j2,
-                                                    s->prev_P, s->ccap, (SweepRec<double>*)s->srec,
-                                                    (double4_32a*)s->sp);
+                                                    s->prev_P, s->ccap, s->cstate, s->cpack, sub ? nullptr : s->cmask,
+                                                    (const double4_32a*)s->vel, (SweepRec<double>*)s->srec,
+                                                    (double4_32a*)s->sp, (SweepPre<double>*)s->spre);
         if (s->timing) s->phase_launches[1] += 3;
         s->n_colours = -1;  // known on the device; read lazily
     } else {

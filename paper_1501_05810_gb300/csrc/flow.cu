@@ -1,0 +1,496 @@
+// flow.cu -- the NBGS solve as a dataflow over body versions.
+//
+// The sweeps relax the contacts colour by colour; the order that matters is
+// only that every body sees its contacts in colour order.  So a contact does
+// not wait for a colour to end anywhere: every body's velocity record carries
+// a version, each contact waits until both of its bodies show the version its
+// predecessor leaves, and stores the two records back with the next one.  The
+// result is that of the sweeps in colour order, bit for bit.
+//
+// Versions.  A contact of colour c relaxed in pass k (pass 0 applies the
+// initial impulses of a warm start, the sweeps follow) leaves (k << 9) | (c +
+// 1) on its bodies, and ((k + 1) << 9) on a body whose last contact it is; it
+// expects (k << 9) | (colour of the body's contact before it + 1), or (k <<
+// 9) on a body whose first contact it is.  The 9-bit fields come from the
+// bodies' colour masks (dep word in .w of the impulse, colour.cu).
+//
+// Memory.  The state and its version travel in one 128-bit word, loaded and
+// stored as .b128 with relaxed gpu scope: such an access is single-copy
+// atomic, so a word that shows the expected version holds that version's
+// values, with no fence, flag or barrier.  A body takes two words in FP32
+// (v, tag), (w, tag), and four in FP64 (each a double, half of a third one
+// and the tag).  1/m and 1/I sit in a read-only array beside them.  In FP32 a
+// pair of lanes moves the two halves of one body (a whole 32-byte sector per
+// pair) and exchanges them by shuffles.
+//
+// Schedule.  A colour is cut into tiles of up to 32 contacts; the tiles of
+// all colours, in colour order, are dealt to the warps in turn, the same in
+// every pass, so that a contact's impulse stays with one lane.  A warp goes
+// through its tiles in (pass, colour) order and a tile waits only for tiles
+// that come earlier in that order, so with every warp resident (a cooperative
+// launch) the earliest unfinished tile can always run.  Every wait is bounded.
+#include <algorithm>
+#include <mutex>
+#include <utility>
+#include <vector>
+
+#include "units.cuh"
+
+namespace nbgs {
+
+namespace {
+
+template <class R> struct Mass2;
+template <> struct Mass2<float> { using T = float2; };
+template <> struct Mass2<double> { using T = double2; };
+
+template <class R> struct FlowArgs {
+    int64_t n;
+    uint4* tv;                        // versioned velocities, Words<R>::N per body
+    const typename Mass2<R>::T* mass;  // (1/m, 1/I), kept for the way back
+    const SweepRec<R>* rec;
+    const SweepPre<R>* pre;
+    __device__ __forceinline__ uint32_t body_a(uint32_t s) const
+    {
+        return sizeof(R) == 4 ? __float_as_uint(reinterpret_cast<const SweepRec<float>*>(rec)[s].a.x)
+                              : reinterpret_cast<const uint32_t*>(rec + s)[0];
+    }
+    R4<R>* p;                         // impulses and dep words, colour order
+    const uint32_t* col_off;
+    DevInfo* info;
+    R mu, omega;
+    double gdt_norm;
+    int max_sweeps;
+    double tol;
+    int warm;
+    int tile;                         // contacts per tile: a power of two, at most 32
+    SceneView V;                      // batched scenes
+    int64_t nscene;
+    unsigned long long* scene_rk;
+    uint32_t* scene_done;
+    double* scene_res;
+};
+
+// Gravity, versions 0 and the mass array.
+template <class R>
+__global__ void k_flow_init(int64_t n, const R4<R>* __restrict__ vel, R gx, R gy, R gz, uint4* __restrict__ tv,
+                            typename Mass2<R>::T* __restrict__ mass)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        R4<R> v, w;
+        ld_body(vel + 2 * i, v, w);
+        typename Mass2<R>::T m;
+        m.x = v.w;
+        m.y = w.w;
+        mass[i] = m;
+        if (v.w > R(0)) {
+            v.x += gx;
+            v.y += gy;
+            v.z += gz;
+        }
+        pack_body(tv + Words<R>::N * i, 0u, v, w);
+    }
+}
+
+// The solved velocities back into the body records, and the solve's outcome.
+template <class R, bool Batch>
+__global__ void k_flow_out(FlowArgs<R> A, R4<R>* __restrict__ vel)
+{
+    const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, gstride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = gtid; i < A.n; i += gstride) {
+        R4<R> v, w;
+        uint32_t tags[4];
+        load_body(A.tv + Words<R>::N * i, v, w, tags);
+        const typename Mass2<R>::T m = A.mass[i];
+        v.w = m.x;
+        w.w = m.y;
+        st_body(vel + 2 * i, v, w);
+    }
+    const int k = (int)A.info->sweeps_done;
+    if (Batch) {   // scenes still short of their tolerance ran every sweep
+        for (int64_t sc = gtid; sc < A.nscene; sc += gstride) {
+            if (A.scene_done[sc] == 0) {
+                A.scene_done[sc] = (uint32_t)k;
+                A.scene_res[sc] =
+                    k > 0 ? __longlong_as_double((long long)A.scene_rk[scene_slot(k - 1) * A.nscene + sc]) : 0.0;
+            }
+        }
+    }
+    if (gtid == 0) {
+        const double vref = v_ref_of(A.info, A.gdt_norm);
+        A.info->residual =
+            k > 0 ? __longlong_as_double((long long)A.info->rk_bits[rk_slot(k - 1)]) / (Batch ? 1.0 : vref) : 0.0;
+        A.info->v_ref = vref;
+    }
+}
+
+// Threads of a block and blocks per SM the kernels are compiled for.
+template <class R, int L> struct FlowShape {
+    static constexpr int threads = 256, blocks = sizeof(R) == 4 ? 2 : 1;
+};
+template <> struct FlowShape<float, 1> {
+    static constexpr int threads = 128, blocks = 6;
+};
+
+template <class R, int L, bool Batch>
+__global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::blocks)) k_solve_flow(FlowArgs<R> A)
+{
+    __shared__ uint32_t s_tile[kMaxColours + 1];   // first tile of every colour
+    __shared__ uint32_t s_off[kMaxColours + 1];
+    __shared__ int s_vote;
+    const int ncol = min((int)A.info->n_colours, kMaxColours);
+    const unsigned nb = gridDim.x;
+    const int lane = threadIdx.x & 31;
+    const uint32_t tw = (uint32_t)A.tile;
+    for (int c = threadIdx.x; c <= ncol; c += blockDim.x) s_off[c] = A.col_off[c];
+    __syncthreads();
+    if (threadIdx.x < 32) {   // tiles before every colour
+        uint32_t carry = 0;
+        for (int c0 = 0; c0 < ncol; c0 += 32) {
+            const int c = c0 + lane;
+            uint32_t v = c < ncol ? (s_off[c + 1] - s_off[c] + tw - 1) / tw : 0u;
+            const uint32_t own = v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += y;
+            }
+            if (c < ncol) s_tile[c] = carry + v - own;
+            carry += __shfl_sync(0xffffffffu, v, 31);
+        }
+        if (lane == 0) s_tile[ncol] = carry;
+    }
+    __syncthreads();
+    const uint32_t ntile = s_tile[ncol];
+    // warp w of the grid: warps 0 of all blocks first, so that few tiles spread over the SMs
+    const uint32_t W = nb * (blockDim.x >> 5), w0 = (threadIdx.x >> 5) * nb + blockIdx.x;
+    const bool work = w0 < ntile;
+    const double vref = v_ref_of(A.info, A.gdt_norm);
+    const double vnorm = Batch ? 1.0 : vref;   // batched residuals arrive already divided by v_ref_s
+    const int warm = A.warm ? 1 : 0;
+    const int npass = A.max_sweeps + warm;
+    bool ok = true;
+
+    // lanes 2i and 2i + 1 of a lane per FP32 contact take contacts i and i +
+    // 16 of a tile of 32: each access of a pair of lanes then covers
+    // consecutive contacts, whose bodies tend to share lines
+    const uint32_t unit = sizeof(R) == 4 && L == 1 ? (uint32_t)(lane >> 1) + 16u * (lane & 1) : (uint32_t)(lane / L);
+    // a position in the tile order: tile T of colour c, the colour's tiles end
+    // at tend; unit u's contact of it is slot base + T tw + u, if below send
+    struct Pos {
+        uint32_t T, tend, base, send;
+        int c;
+    };
+    auto seek = [&](Pos& q, uint32_t T, int c) {
+        while (T >= s_tile[c + 1]) ++c;
+        q.T = T;
+        q.c = c;
+        q.tend = s_tile[c + 1];
+        q.send = s_off[c + 1];
+        q.base = s_off[c] - s_tile[c] * tw;
+    };
+    Unit<R, L> K;
+    uint32_t s = 0;
+    bool on = false;
+    Pos at = {0u, 0u, 0u, 0u, 0};
+    SweepRec<R> nrec;
+    SweepPre<R> npre;
+    R4<R> npp;
+    auto read = [&](uint32_t sl) {
+        nrec = ld_rec(A.rec + sl);
+        npre = ld_pre(A.pre + sl);
+        npp = A.p[sl];
+    };
+    // the records of the warp's next tile: into registers, or, in the variant
+    // whose many warps leave none to spare, into L1 (loads nobody waits for)
+    constexpr bool Touch = sizeof(R) == 4 && L == 1;
+    auto fetch = [&](const Pos& q, uint32_t& sl, bool& live) {
+        sl = q.base + q.T * tw + unit;
+        live = unit < tw && sl < q.send;
+        if (!live) return;
+        if constexpr (Touch) {
+            uint32_t x;
+            asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(A.rec + sl));
+            asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(A.pre + sl));
+            asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(A.p + sl));
+        } else {
+            read(sl);
+        }
+    };
+    // the contact fetched (slot s) becomes the unit's current one
+    auto take = [&]() {
+        if (on) {
+            if (Touch) read(s);
+            K.take(nrec, npre, npp, (uint32_t)A.n);
+        }
+        // idle units read along with the first one, which every tile has
+        const uint32_t q0 = __shfl_sync(kFull, K.qa, 0);
+        if (!on) K.idle(q0);
+    };
+    if (work) {
+        seek(at, w0, 0);
+        fetch(at, s, on);
+        take();
+    }
+    int k = 0;
+    for (int pass = 0; pass < npass; ++pass) {
+        const bool apply = pass < warm;
+        k = pass - warm;
+        if (!apply) {
+            if (blockIdx.x == 0 && threadIdx.x == 0 && k + 1 >= kHistKept) A.info->rk_bits[rk_slot(k + 1)] = 0ull;
+            if (Batch)   // the slot of sweep k + 1 is neither read nor written during sweep k
+                for (int64_t sc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; sc < A.nscene;
+                     sc += (int64_t)gridDim.x * blockDim.x)
+                    A.scene_rk[scene_slot(k + 1) * A.nscene + sc] = 0ull;
+        }
+        R rmax = R(0);
+        const uint32_t base = (uint32_t)pass << 9;
+        for (bool more = work; more && ok;) {
+            K.load(A.tv);
+            // while the bodies' words are on their way: the warp's next tile
+            // (the first one again at the end of a pass), whose records
+            // depend on no other warp
+            const bool wrap = at.T + W >= ntile;
+            const uint32_t Tn = wrap ? w0 : at.T + W;
+            const bool same = Tn == at.T;
+            uint32_t sn = s;
+            bool non = on;
+            const uint32_t c1 = (uint32_t)at.c + 1u;
+            if (!same) {
+                if (wrap || Tn >= at.tend) seek(at, Tn, wrap ? 0 : at.c);
+                at.T = Tn;
+                fetch(at, sn, non);
+            }
+            const uint32_t dep = on ? dep_bits(K.pp.w) : 0u;
+            bool live = on;
+            R mu = A.mu;
+            double vref_s = 1.0;
+            uint32_t scene = 0;
+            if (Batch && on) {
+                scene = A.V.scene_of[A.body_a(s)];
+                if (!apply && k > 0) {   // this scene met its tolerance in an earlier sweep: it is done
+                    const double prev =
+                        __longlong_as_double((long long)A.scene_rk[scene_slot(k - 1) * A.nscene + scene]);
+                    if (prev <= A.tol) live = false;
+                }
+                mu = (R)A.V.mu[scene];
+                vref_s = A.V.vref[scene];
+            }
+            const bool va = live && (dep & kDepListA) != 0u, vb = live && K.hasb && (dep & kDepListB) != 0u;
+            const uint32_t ma = va ? ~0u : 0u, mb = vb ? ~0u : 0u;
+            const uint32_t ea = base | (dep & 0x1FFu), eb = base | ((dep >> 11) & 0x1FFu);
+            const uint32_t after = base | c1, next = base + 512u;
+            const uint32_t oa = (dep & kDepLastA) ? next : after, ob = (dep & kDepLastB) ? next : after;
+            if (!__all_sync(kFull, K.ready(ma, mb, ea, eb))) {
+                const long long t0 = clock64();
+                int polls = 0;
+                for (;;) {
+                    K.load(A.tv);
+                    if (__all_sync(kFull, K.ready(ma, mb, ea, eb))) break;
+                    if ((++polls & 255) == 0) {   // bounded like every other wait
+                        bool give_up = (((volatile uint32_t*)&A.info->err)[0] & kErrTimeout) != 0u;
+                        if (clock64() - t0 > (1LL << 31)) {
+                            if (lane == 0) atomicOr(&A.info->err, kErrTimeout);
+                            give_up = true;
+                        }
+                        if (__any_sync(kFull, give_up)) {
+                            ok = false;
+                            break;
+                        }
+                    }
+                }
+                if (!ok) break;
+            }
+            if (apply) {
+                K.template relax<true>(live, mu, A.omega);
+                K.store(A.tv, va, vb, oa, ob);
+            } else {
+                K.template relax<false>(live, mu, A.omega);
+                K.store(A.tv, va, vb, oa, ob);
+                if (live) K.save(A.p + s);
+                R r2 = K.residual();
+                if (Batch && live) {   // per-scene R_k; the read filter only saves atomics
+                    const double rn = (double)sqrt(r2) / vref_s;
+                    unsigned long long* dst = A.scene_rk + scene_slot(k) * A.nscene + scene;
+                    const unsigned long long bits = (unsigned long long)__double_as_longlong(rn);
+                    if (lane % L == 0 && bits > *(volatile unsigned long long*)dst) atomicMax(dst, bits);
+                    r2 = (R)rn;
+                }
+                rmax = live && above(r2, rmax) ? r2 : rmax;
+            }
+            __syncwarp();   // the lanes of a unit read back what one of them saved
+            more = !wrap;
+            if (!same) {
+                s = sn;
+                on = non;
+                take();
+            }
+        }
+        if (apply) continue;
+        if (!Batch) rmax = sqrt(rmax);
+        // R_k is recorded by every warp; a test of it needs the whole block, and
+        // every block near the rotating residual slots or for batched scenes
+        const bool vote = !Batch && ncol > 0 && A.tol > 0.0 && k + 2 < kHistKept;
+        const bool sync = ncol > 0 && !vote && (A.tol > 0.0 || Batch || k + 2 >= kHistKept);
+        if (!vote && !sync) {
+            if (!ok) break;
+            if (work) {
+                for (int o = 16; o > 0; o >>= 1) rmax = fmax(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+                if (lane == 0) {
+                    double x = (double)rmax;
+                    if (!(x <= 1e300)) x = __longlong_as_double(0x7FF0000000000000LL);
+                    atomicMax(&A.info->rk_bits[rk_slot(k)], (unsigned long long)__double_as_longlong(x));
+                }
+            }
+            continue;
+        }
+        if (!__syncthreads_and(ok)) {
+            ok = false;
+            break;
+        }
+        const double rb = block_max_to<R>(rmax, &A.info->rk_bits[rk_slot(k)]);
+        if (vote) {
+            const int v = tol_vote(A.info, k, rb, vnorm, A.tol, nb, &s_vote);
+            if (v < 0) ok = false;
+            if (v <= 0) break;
+            continue;
+        }
+        if (!grid_barrier(A.info, nb)) {
+            ok = false;
+            break;
+        }
+        if (Batch && A.tol > 0.0) {   // scenes that met their tolerance in this sweep
+            for (int64_t sc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; sc < A.nscene;
+                 sc += (int64_t)gridDim.x * blockDim.x) {
+                const double rs = __longlong_as_double(
+                    (long long)((volatile unsigned long long*)A.scene_rk)[scene_slot(k) * A.nscene + sc]);
+                if (A.scene_done[sc] == 0 && rs <= A.tol) {
+                    A.scene_done[sc] = (uint32_t)(k + 1);
+                    A.scene_res[sc] = rs;
+                }
+            }
+        }
+        const double Rk = __longlong_as_double((long long)((volatile unsigned long long*)A.info->rk_bits)[rk_slot(k)]) / vnorm;
+        if (A.tol > 0.0 && Rk <= A.tol) break;
+    }
+    // sweeps run: k + 1 after a break at sweep k, and max_sweeps at the end
+    if (blockIdx.x == 0 && threadIdx.x == 0 && ok)
+        A.info->sweeps_done = (uint32_t)(A.max_sweeps == 0 ? 0 : min(k + 1, A.max_sweeps));
+}
+
+// Resident blocks per SM of a flow kernel at a block size, looked up once.
+int flow_occ(const void* fn, int threads)
+{
+    static std::mutex mu;
+    static std::vector<std::pair<std::pair<const void*, int>, int>> known;
+    std::lock_guard<std::mutex> lock(mu);
+    for (const auto& kv : known)
+        if (kv.first.first == fn && kv.first.second == threads) return kv.second;
+    int o = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, threads, 0);
+    cudaGetLastError();
+    known.push_back({{fn, threads}, o});
+    return o;
+}
+
+// Which kernel, and how many warps, for a scene of n bodies.
+//
+// A pile has 2 to 3 contacts per body (6 at most) in 13 to 18 colours.  Up to
+// some 10^5 bodies a sweep takes as long as its longest chain of contacts, so
+// the contact itself has to be quick (more lanes) and a warp beyond the tiles
+// of a colour only polls; above, it takes as long as the memory system needs
+// for the contacts in flight, so they have to be many.  50 sweeps of a pile,
+// ms, one GB300:
+//   bodies                        30k    120k    250k    500k      1M
+//   FP32, 2 lanes, 1 block/SM    0.86    1.21    2.06    4.95    9.70
+//   FP32, 2 lanes, 2 blocks/SM   0.91    1.16    1.48    2.93    5.55
+//   FP32, 1 lane,  6 blocks/SM   1.24    1.64    1.85    2.57    4.15
+//   bodies                         1k     12k     30k     60k    120k
+//   FP64, 4 lanes, 8 warps/SM    1.44    1.74    2.23    3.67    7.09
+//   FP64, 1 lane,  4 warps/SM    3.14    4.20    4.43    4.43    5.31
+//   FP64, 1 lane,  8 warps/SM    3.14    4.91    5.55    5.73    5.83
+struct FlowPlan {
+    const void* fn;
+    int tile, warps, blocks_per_sm;   // contacts per tile, warps per block
+};
+
+template <class R>
+FlowPlan flow_plan(int64_t n, bool batch);
+
+template <>
+FlowPlan flow_plan<float>(int64_t n, bool batch)
+{
+    if (n < 350000)
+        return {batch ? (const void*)k_solve_flow<float, 2, true> : (const void*)k_solve_flow<float, 2, false>, 16, 8,
+                n < 90000 ? 1 : 2};
+    return {batch ? (const void*)k_solve_flow<float, 1, true> : (const void*)k_solve_flow<float, 1, false>, 32, 4, 6};
+}
+
+template <>
+FlowPlan flow_plan<double>(int64_t n, bool batch)
+{
+    if (n < 64000)
+        return {batch ? (const void*)k_solve_flow<double, 4, true> : (const void*)k_solve_flow<double, 4, false>, 8, 8, 1};
+    return {batch ? (const void*)k_solve_flow<double, 1, true> : (const void*)k_solve_flow<double, 1, false>, 32,
+            n < 250000 ? 4 : 8, 1};
+}
+
+}  // namespace
+
+// The whole solve: gravity and versions, the passes, the body records.
+template <class R>
+nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm)
+{
+    cudaStream_t st = s->stream;
+    const int64_t n = s->n;
+    FlowArgs<R> A;
+    A.n = n;
+    // the state-transfer staging buffer (13 doubles per body) holds the
+    // versioned records and the masses during a solve
+    A.tv = (uint4*)s->stage;
+    typename Mass2<R>::T* mass = (typename Mass2<R>::T*)(A.tv + (size_t)Words<R>::N * std::max<int64_t>(n, 1));
+    A.mass = mass;
+    A.rec = (const SweepRec<R>*)s->srec;
+    A.pre = (const SweepPre<R>*)s->spre;
+    A.p = (R4<R>*)s->sp;
+    A.col_off = s->col_off;
+    A.info = s->info;
+    A.mu = (R)s->prm.mu;
+    A.omega = (R)s->prm.omega;
+    const double* g = s->prm.gravity;
+    A.gdt_norm = sqrt((g[0] * g[0] + g[1] * g[1]) + g[2] * g[2]) * s->prm.dt;
+    A.max_sweeps = max_sweeps;
+    A.tol = tol;
+    A.warm = warm;
+    A.V = scene_view(s);
+    A.nscene = s->n_scenes;
+    A.scene_rk = s->scene_rk;
+    A.scene_done = s->scene_done;
+    A.scene_res = s->scene_res;
+    const FlowPlan P = flow_plan<R>(s->n, s->batch);
+    A.tile = P.tile;
+    const void* fn = P.fn;
+    const int threads = 32 * P.warps;
+    int nblocks = std::min(flow_occ(fn, threads), P.blocks_per_sm) * s->num_sms;
+    if (s->coop_blocks < s->max_coop_blocks) nblocks = std::min(nblocks, s->coop_blocks);   // set by nbgs_autotune
+    if (nblocks < 1) return fail(s, NBGS_ECUDA, "solve: sweep kernel does not fit");
+    const int T = 256, gb = grid_for(std::max<int64_t>(n, 1), T, 8, s->num_sms);
+    k_flow_init<R><<<gb, T, 0, st>>>(n, (const R4<R>*)s->vel, (R)(s->prm.dt * g[0]), (R)(s->prm.dt * g[1]),
+                                     (R)(s->prm.dt * g[2]), A.tv, mass);
+    void* args[] = {&A};
+    if (s->timing) cudaEventRecord(s->ev[8], st);
+    const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nblocks), dim3(threads), args, 0, st);
+    if (s->timing) {
+        cudaEventRecord(s->ev[9], st);
+        s->phase_launches[2] += 3;
+        s->sweep_launches += 1;
+    }
+    if (e != cudaSuccess) return cuda_check(s, e, "solve: cooperative launch");
+    if (s->batch) k_flow_out<R, true><<<gb, T, 0, st>>>(A, (R4<R>*)s->vel);
+    else k_flow_out<R, false><<<gb, T, 0, st>>>(A, (R4<R>*)s->vel);
+    return cuda_check(s, cudaGetLastError(), "solve");
+}
+
+template nbgs_status run_flow<float>(nbgs_scene*, int, double, int);
+template nbgs_status run_flow<double>(nbgs_scene*, int, double, int);
+
+}  // namespace nbgs

@@ -272,7 +272,7 @@ template <class R> struct WarmArgs {
 
 // Features of sweep slot s (see the top of this file) and what applying the
 // network's output needs: the frame angle (cth, sth), w_n, v_ref, mu and the
-// previous-step impulse (p0.w != 0: the contact existed in the last step).
+// previous-step impulse (kDepFound in p0.w: the contact existed in the last step).
 template <class R> struct ContactFeatures {
     float f[kIn];
     double cth, sth, wn, vr, mu;
@@ -390,7 +390,7 @@ static __device__ __noinline__ void warm_tiles(const WarmArgs<R>& A, TcMlpSmem* 
         } else {
 #pragma unroll
             for (int k = 0; k < kIn; ++k) F.f[k] = 0.f;
-            F.p0.w = R(1);
+            dep_store(kDepFound, F.p0.w);
         }
         if (!S || !ok) continue;   // both uniform over the CTA
         float out[kOutN];
@@ -399,7 +399,7 @@ static __device__ __noinline__ void warm_tiles(const WarmArgs<R>& A, TcMlpSmem* 
             if (threadIdx.x == 0) atomicOr(&A.info->err, kErrTimeout);
             continue;
         }
-        if (live && F.p0.w == R(0)) {
+        if (live && !(dep_bits(F.p0.w) & kDepFound)) {
             const double k = F.vr / F.wn;   // skip connection: previous impulse + network correction
             const double y1 = ((double)out[0] + F.f[3]) * k;
             const double y2 = ((double)out[1] + F.f[4]) * k;
@@ -417,7 +417,7 @@ static __device__ __noinline__ void warm_tiles(const WarmArgs<R>& A, TcMlpSmem* 
                 q.x = (R)pn;
                 q.y = (R)pt;
                 q.z = (R)po;
-                q.w = R(0);
+                q.w = F.p0.w;
                 A.p[s] = q;
             }
         }

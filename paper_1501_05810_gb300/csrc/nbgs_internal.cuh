@@ -203,6 +203,32 @@ template <> struct __align__(16) SweepRec<double> {
     double2 nz_;       // (nz, unused)
 };
 
+// What the dataflow sweeps need of a contact besides its record: the masses of
+// its bodies and the quotients that do not change during a solve (k = l / I;
+// w_n = 1/m_a + 1/m_b, w_t and their reciprocals; f = -1 / (sign(n_z) + n_z)
+// of the tangent basis; in FP64 f sits in nz_.y of the record).
+template <class R> struct SweepPre;
+template <> struct __align__(32) SweepPre<float> {
+    float4 m;       // 1/m_a, 1/m_b, la/I_a, lb/I_b
+    float4 w;       // w_t, 1/w_n, 1/w_t, f
+};
+template <> struct __align__(32) SweepPre<double> {
+    double4_32a m;  // 1/m_a, 1/m_b, la/I_a, lb/I_b
+    double4_32a w;  // w_n, w_t, 1/w_n, 1/w_t
+};
+
+// Dependency word of a contact (bits of .w of its sweep impulse): per end,
+// the colour + 1 of the contact before it in its body's colour order (9 bits,
+// 0: it is the first), whether it is the body's last, and whether the body
+// takes impulses at all; bit 31: the contact existed in the previous step.
+constexpr uint32_t kDepLastA = 1u << 9, kDepListA = 1u << 10, kDepLastB = 1u << 20, kDepListB = 1u << 21;
+constexpr uint32_t kDepFound = 1u << 31;
+
+__device__ __forceinline__ uint32_t dep_bits(float w) { return __float_as_uint(w); }
+__device__ __forceinline__ uint32_t dep_bits(double w) { return (uint32_t)__double2loint(w); }
+__device__ __forceinline__ void dep_store(uint32_t d, float& w) { w = __uint_as_float(d); }
+__device__ __forceinline__ void dep_store(uint32_t d, double& w) { w = __longlong_as_double((long long)d); }
+
 // 256-bit global accesses: a body's (v, 1/m) and (w, 1/I) pair and an FP32
 // sweep record each move as one request instead of two (FP64: two instead
 // of four).  The body accesses keep their order with every other memory
@@ -496,6 +522,7 @@ struct nbgs_scene {
     // sweep
     void* srec = nullptr;
     void* sp = nullptr;
+    void* spre = nullptr;          // SweepPre per contact, colour order
     // device info
     nbgs::DevInfo* info = nullptr;
     nbgs::DevInfo* hinfo = nullptr;   // pinned host copy
@@ -539,6 +566,8 @@ void dev_free(nbgs_scene* s, void* p);
 nbgs_status run_detect(nbgs_scene* s);
 nbgs_status run_colour(nbgs_scene* s);
 nbgs_status run_solve(nbgs_scene* s, int max_sweeps, double tol);
+template <class R>
+nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm);   // flow.cu: the dataflow sweeps
 nbgs_status run_integrate(nbgs_scene* s);
 nbgs_status run_final_residuals(nbgs_scene* s, nbgs_residuals* out);
 nbgs_status run_set_impulses(nbgs_scene* s, const double* impulse);

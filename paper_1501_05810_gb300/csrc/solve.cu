@@ -22,7 +22,7 @@
 #include <utility>
 #include <vector>
 
-#include "mlp_tc.cuh"
+#include "relax.cuh"
 
 namespace nbgs {
 
@@ -57,72 +57,7 @@ template <class R> struct SolveArgs {
     const uint32_t* rlist;     // shared bodies grouped by the block that reduces them (local scheduling)
     const uint32_t* rstart;    // B + 1: each block's range of rlist
     const int2* dep_r;         // B: window of each block's reduction phase
-    int mlp;                   // the network's warm start of new contacts runs in the kernel's prologue
-    WarmArgs<R> W;             // its arguments
 };
-
-// Rotating per-scene residual slot of sweep k (three, so that clearing the
-// slot of sweep k + 1 while sweep k runs touches nothing still read).
-__host__ __device__ __forceinline__ int scene_slot(int k) { return k % 3; }
-
-template <class R>
-__device__ __forceinline__ void decode(const SweepRec<R>& r, uint32_t& a, uint32_t& b, R& la, R& lb, R& nx, R& ny, R& nz,
-                                       R& bias);
-
-template <>
-__device__ __forceinline__ void decode<float>(const SweepRec<float>& r, uint32_t& a, uint32_t& b, float& la, float& lb,
-                                              float& nx, float& ny, float& nz, float& bias)
-{
-    a = __float_as_uint(r.a.x);
-    b = __float_as_uint(r.a.y);
-    la = r.a.z;
-    lb = r.a.w;
-    nx = r.b.x;
-    ny = r.b.y;
-    nz = r.b.z;
-    bias = r.b.w;
-}
-
-template <>
-__device__ __forceinline__ void decode<double>(const SweepRec<double>& r, uint32_t& a, uint32_t& b, double& la,
-                                               double& lb, double& nx, double& ny, double& nz, double& bias)
-{
-    const uint64_t ids = (uint64_t)__double_as_longlong(r.ids_bias.x);
-    a = (uint32_t)(ids & 0xFFFFFFFFu);
-    b = (uint32_t)(ids >> 32);
-    bias = r.ids_bias.y;
-    la = r.lev.x;
-    lb = r.lev.y;
-    nx = r.nxy.x;
-    ny = r.nxy.y;
-    nz = r.nz_.x;
-}
-
-// State of the two bodies of a contact, gathered before anything is stored.
-template <class R> struct Bodies {
-    R4<R> va, wa, vb, wb;
-};
-
-// Sweep records do not change during a solve.
-__device__ __forceinline__ SweepRec<float> ld_rec(const SweepRec<float>* p)
-{
-    SweepRec<float> r;
-    asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=f"(r.a.x), "=f"(r.a.y), "=f"(r.a.z), "=f"(r.a.w), "=f"(r.b.x), "=f"(r.b.y), "=f"(r.b.z), "=f"(r.b.w)
-        : "l"(p));
-    return r;
-}
-__device__ __forceinline__ SweepRec<double> ld_rec(const SweepRec<double>* p)
-{
-    SweepRec<double> r;
-    asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
-        : "=d"(r.ids_bias.x), "=d"(r.ids_bias.y), "=d"(r.lev.x), "=d"(r.lev.y)
-        : "l"(p));
-    asm("ld.global.nc.v4.f64 {%0,%1,%2,%3}, [%4];"
-        : "=d"(r.nxy.x), "=d"(r.nxy.y), "=d"(r.nz_.x), "=d"(r.nz_.y)
-        : "l"(reinterpret_cast<const char*>(p) + 32));
-    return r;
-}
 
 template <class R>
 __device__ __forceinline__ void gather(const SolveArgs<R>& A, const SweepRec<R>& rr, Bodies<R>& B)
@@ -163,85 +98,17 @@ __device__ __forceinline__ R relax_gathered(const SolveArgs<R>& A, int64_t s, co
         mu = (R)A.V.mu[scene];
         vref_s = A.V.vref[scene];
     }
-    R4<R> va = B.va, wa = B.wa, vb = B.vb, wb = B.wb;
-    const bool dyn_b = ib < (uint64_t)A.nslot;
-    const R ima = va.w, iIa = wa.w, imb = vb.w, iIb = wb.w;
-    R tx, ty, tz, ox, oy, oz;
-    tangent_basis<R>(nx, ny, nz, tx, ty, tz, ox, oy, oz);
-    const R wn = ima + imb;
-    if (!(wn > R(0))) return R(0);  // both masses infinite: nothing can move
-    const R wt = wn + iIa * la * la + iIb * lb * lb;
-    R dn, dt_, do_;
-    if (apply_only) {
-        dn = pp.x;
-        dt_ = pp.y;
-        do_ = pp.z;
-    } else {
-        // u = v_a - la (w_a x n) - v_b - lb (w_b x n)
-        const R cax = wa.y * nz - wa.z * ny, cay = wa.z * nx - wa.x * nz, caz = wa.x * ny - wa.y * nx;
-        const R cbx = wb.y * nz - wb.z * ny, cby = wb.z * nx - wb.x * nz, cbz = wb.x * ny - wb.y * nx;
-        const R ux = (va.x - la * cax) - (vb.x + lb * cbx);
-        const R uy = (va.y - la * cay) - (vb.y + lb * cby);
-        const R uz = (va.z - la * caz) - (vb.z + lb * cbz);
-        const R un = nx * ux + ny * uy + nz * uz;
-        const R ut = tx * ux + ty * uy + tz * uz;
-        const R uo = ox * ux + oy * uy + oz * uz;
-        const R bn = un - wn * pp.x + bias;
-        const R bt = ut - wt * pp.y;
-        const R bo = uo - wt * pp.z;
-        R yn = -bn / wn;
-        yn = yn > R(0) ? yn : R(0);
-        R yt = -bt / wt, yo = -bo / wt;
-        const R lim = mu * yn;
-        const R len2 = yt * yt + yo * yo;
-        if (len2 > lim * lim) {
-            if (len2 > R(0)) {
-                const R sc = lim / sqrt(len2);
-                yt *= sc;
-                yo *= sc;
-            } else {
-                yt = yo = R(0);
-            }
-        }
-        const R om = A.omega, om1 = R(1) - A.omega;
-        const R pn = om * yn + om1 * pp.x, pt = om * yt + om1 * pp.y, po = om * yo + om1 * pp.z;
-        dn = pn - pp.x;
-        dt_ = pt - pp.y;
-        do_ = po - pp.z;
-        R4<R> q;
-        q.x = pn;
-        q.y = pt;
-        q.z = po;
+    R4<R> q = pp;
+    bool moves;
+    const R r2 = relax_bodies<R, apply_only>(rr, mu, A.omega, q, B, moves);
+    if (!moves) return R(0);
+    if (!apply_only) {
         q.w = R(0);
         A.p[s] = q;
     }
-    // world impulse change P = dn n + dt t + do o; torque arm n x P
-    const R Px = dn * nx + dt_ * tx + do_ * ox;
-    const R Py = dn * ny + dt_ * ty + do_ * oy;
-    const R Pz = dn * nz + dt_ * tz + do_ * oz;
-    const R qx = ny * Pz - nz * Py, qy = nz * Px - nx * Pz, qz = nx * Py - ny * Px;
-    if (ima > R(0) || iIa > R(0)) {
-        va.x += ima * Px;
-        va.y += ima * Py;
-        va.z += ima * Pz;
-        const R ka = la * iIa;
-        wa.x -= ka * qx;
-        wa.y -= ka * qy;
-        wa.z -= ka * qz;
-        st_body(A.vel + 2 * (int64_t)ia, va, wa);
-    }
-    if (dyn_b && (imb > R(0) || iIb > R(0))) {
-        vb.x -= imb * Px;
-        vb.y -= imb * Py;
-        vb.z -= imb * Pz;
-        const R kb = lb * iIb;
-        wb.x -= kb * qx;
-        wb.y -= kb * qy;
-        wb.z -= kb * qz;
-        st_body(A.vel + 2 * (int64_t)ib, vb, wb);
-    }
-    const R r1 = wn * dn, r2 = wt * dt_, r3 = wt * do_;
-    const R r = sqrt(r1 * r1 + r2 * r2 + r3 * r3);
+    if (B.va.w > R(0) || B.wa.w > R(0)) st_body(A.vel + 2 * (int64_t)ia, B.va, B.wa);
+    if (ib < (uint64_t)A.nslot && (B.vb.w > R(0) || B.wb.w > R(0))) st_body(A.vel + 2 * (int64_t)ib, B.vb, B.wb);
+    const R r = sqrt(r2);
     if (Batch && !apply_only) {
         // per-scene R_k; the read filter only saves atomics
         const double rn = (double)r / vref_s;
@@ -356,30 +223,6 @@ __device__ __forceinline__ void inst_reduce_pass(const SolveArgs<R>& A, int64_t 
     for (int64_t t = gtid; t < ns; t += gstride) inst_reduce_body<R>(A, A.shared[t]);
 }
 
-template <class R>
-__device__ __forceinline__ double block_max_to(R v, unsigned long long* dst)
-{
-    __shared__ double sm[32];
-    double x = (double)v;
-    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_down_sync(0xffffffffu, x, o));
-    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = x;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) x = fmax(x, sm[k]);
-        if (!(x <= 1e300)) x = __longlong_as_double(0x7FF0000000000000LL);  // NaN/Inf -> +Inf
-        atomicMax(dst, (unsigned long long)__double_as_longlong(x));
-    }
-    __syncthreads();
-    return x;
-}
-
-__device__ __forceinline__ double v_ref_of(const DevInfo* info, double gdt_norm)
-{
-    double v = __longlong_as_double((long long)info->vmax_bits);
-    v = fmax(v, gdt_norm);
-    return fmax(v, 1e-12);
-}
-
 // ---------------------------------------------------------------------------
 // Whole solve in one cooperative launch: gravity, warm-start impulses and the
 // sweeps.  Block b owns the same contiguous chunk of every colour in every
@@ -400,49 +243,6 @@ template <class R> struct Stage {
 // [ceil(b C / B), ceil((b + 1) C / B)): a contiguous range of the colour
 // (the colour sort is stable), balanced by contact count and local in body
 // index, so that a chunk's bodies are touched only by nearby blocks.
-// --- TMA bulk copies (global -> shared) completed on an mbarrier -----------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(bar)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-    return ok != 0;
-}
-
-// Bounded wait for the stage of the given parity; false (timeout bit set)
-// after ~2^31 SM clocks.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, DevInfo* info)
-{
-    const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
-        if (clock64() - t0 > (1LL << 31)) {
-            atomicOr(&info->err, kErrTimeout);
-            return false;
-        }
-    }
-    return true;
-}
-
 // Thread 0 starts the copy of this block's chunk of colour c (its first CAP
 // contacts) into the stage; returns the number of staged contacts.
 template <class R>
@@ -677,45 +477,7 @@ __device__ __forceinline__ R process_gathered(const SolveArgs<R>& A, int64_t b0,
     return rmax;
 }
 
-// The tolerance test of sweep k without a grid barrier.  R_k <= tol holds
-// exactly when every block's own maximum (divided by the same v_ref) is at
-// or below tol, so a block above it announces that and goes on at once; a
-// block at or below it counts itself and waits until either some block has
-// announced (the sweeps go on) or every block has counted itself (the solve
-// stops after sweep k).  Every block reaches the end of sweep k, so the
-// wait ends; bounded like every other.  Returns 1 to go on, 0 to stop, -1
-// when the wait ran out.
-__device__ __forceinline__ int tol_vote(DevInfo* info, int k, double rb, double vnorm, double tol, unsigned nb,
-                                        int* s_vote)
-{
-    if (threadIdx.x == 0) {
-        uint32_t* flag = info->votes + 2 * k;
-        int v = 1;
-        if (!(rb / vnorm <= tol)) {
-            atomicExch(flag, 1u);
-        } else {
-            atomicAdd(flag + 1, 1u);
-            const long long t0 = clock64();
-            for (;;) {
-                if (((volatile uint32_t*)flag)[0] != 0u) break;
-                if (((volatile uint32_t*)flag)[1] == nb) {
-                    v = 0;
-                    break;
-                }
-                if ((((volatile uint32_t*)&info->err)[0] & kErrTimeout) || clock64() - t0 > (1LL << 31)) {
-                    atomicOr(&info->err, kErrTimeout);
-                    v = -1;
-                    break;
-                }
-            }
-        }
-        *s_vote = v;
-    }
-    __syncthreads();
-    return *s_vote;
-}
-
-template <class R, bool Batch, bool Warp, bool Sub, int K = 1, bool Mlp = false>
+template <class R, bool Batch, bool Warp, bool Sub, int K = 1>
 __global__ void __launch_bounds__(kPersistThreads, (PersistMinBlocks<R, Batch, K>::value)) k_solve_persistent(SolveArgs<R> A)
 {
     extern __shared__ __align__(128) unsigned char stage_mem[];
@@ -734,13 +496,6 @@ __global__ void __launch_bounds__(kPersistThreads, (PersistMinBlocks<R, Batch, K
     const bool stage = K == 1 && !Warp && (A.flags & NBGS_SWEEP_TMA_STAGE) != 0;
     const bool local = (A.flags & NBGS_SWEEP_GLOBAL_SYNC) == 0;
     if (threadIdx.x == 0) mbar_init(&bar);
-    if constexpr (Mlp) {
-        // the network's warm start (tensor cores, 128 contacts per tile, the
-        // dynamic shared memory as its operand space), every impulse written
-        // before any block applies them
-        warm_tiles<R>(A.W, reinterpret_cast<TcMlpSmem*>(stage_mem));
-        if (!grid_barrier(A.info, nb)) return;
-    }
     gravity_pass<R>(A, gtid, gstride);
     if (!grid_barrier(A.info, nb)) return;
     if (Sub) {
@@ -1279,7 +1034,6 @@ static SolveArgs<R> make_args(nbgs_scene* s, int max_sweeps, double tol)
     A.rlist = s->rlist;
     A.rstart = s->rstart;
     A.dep_r = s->dep_r;
-    A.mlp = 0;
     return A;
 }
 
@@ -1297,7 +1051,7 @@ static int persist_occ(const void* fn)
     for (const auto& kv : known)
         if (kv.first == fn) return kv.second;
     int o = 0;
-    const int dyn = (int)std::max<size_t>(Stage<R>::BYTES, sizeof(TcMlpSmem));   // TMA stage or network operands
+    const int dyn = (int)Stage<R>::BYTES;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, kPersistThreads, dyn);
     cudaGetLastError();
@@ -1324,25 +1078,17 @@ static nbgs_status solve_impl(nbgs_scene* s, int max_sweeps, double tol)
         if (s->timing) s->phase_launches[2] += 1;
     }
     if (s->prm.warm_start == NBGS_WARM_MLP) {
-        const bool warp_sched = (s->prm.sweep_flags & NBGS_SWEEP_WARP_SYNC) && !(s->prm.sweep_flags & NBGS_SWEEP_GLOBAL_SYNC);
-        if (s->prm.solver == NBGS_SOLVER_PERSISTENT && !s->composite && s->n_contacts > 0 && !A.sub && !warp_sched) {
-            // fused into the persistent kernel's prologue
-            if (!s->mlp_theta) return fail(s, NBGS_EINVAL, "MLP warm start: no network loaded (nbgs_mlp_load)");
-            A.mlp = 1;
-            A.W = warm_args<R>(s, 1, nullptr);
-            A.W.C = s->n_contacts;
-        } else {
-            nbgs_status rc = run_mlp_prologue(s, 1, nullptr);
-            if (rc != NBGS_OK) return rc;
-        }
+        nbgs_status rc = run_mlp_prologue(s, 1, nullptr);
+        if (rc != NBGS_OK) return rc;
     }
+    // no scheduling flag: the dataflow sweeps
+    if (s->prm.solver == NBGS_SOLVER_PERSISTENT && s->prm.sweep_flags == 0 && !A.sub)
+        return run_flow<R>(s, max_sweeps, tol, A.warm);
     if (s->prm.solver == NBGS_SOLVER_PERSISTENT) {
         // scheduling units: blocks, or warps with NBGS_SWEEP_WARP_SYNC
         const bool warp = (s->prm.sweep_flags & NBGS_SWEEP_WARP_SYNC) && !(s->prm.sweep_flags & NBGS_SWEEP_GLOBAL_SYNC);
         const int gk = gather_k(s->prm.sweep_flags);
-        const void* fn = A.mlp ? (s->batch ? (const void*)k_solve_persistent<R, true, false, false, 1, true>
-                                           : (const void*)k_solve_persistent<R, false, false, false, 1, true>)
-                         : s->batch ? (warp      ? (const void*)k_solve_persistent<R, true, true, false>
+        const void* fn = s->batch ? (warp      ? (const void*)k_solve_persistent<R, true, true, false>
                                      : gk == 2 ? (const void*)k_solve_persistent<R, true, false, false, 2>
                                                : (const void*)k_solve_persistent<R, true, false, false>)
                          : A.sub  ? (warp ? (const void*)k_solve_persistent<R, false, true, true>
@@ -1391,8 +1137,7 @@ static nbgs_status solve_impl(nbgs_scene* s, int max_sweeps, double tol)
         }
         void* args[] = {&A};
         if (s->timing) cudaEventRecord(s->ev[8], st);
-        size_t dyn = (s->prm.sweep_flags & NBGS_SWEEP_TMA_STAGE) ? Stage<R>::BYTES : 0;
-        if (A.mlp) dyn = std::max(dyn, sizeof(TcMlpSmem));
+        const size_t dyn = (s->prm.sweep_flags & NBGS_SWEEP_TMA_STAGE) ? Stage<R>::BYTES : 0;
         cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nblocks), dim3(s->coop_threads), args, dyn, st);
         if (s->timing) {
             cudaEventRecord(s->ev[9], st);
@@ -1586,7 +1331,7 @@ static void persist_occupancy(int threads, int& occ, int& occ_b)
     const void* batched[] = {(const void*)k_solve_persistent<R, true, false, false>,
                              (const void*)k_solve_persistent<R, true, true, false>};
     occ = occ_b = 1 << 30;
-    const int dyn = (int)std::max<size_t>(Stage<R>::BYTES, sizeof(TcMlpSmem));   // TMA stage or network operands
+    const int dyn = (int)Stage<R>::BYTES;
     for (const void* f : single) {
         int o = 0;
         cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);

@@ -1,0 +1,72 @@
+"""The dataflow sweeps against the other schedules of the same sweeps: the
+kernels chosen by size (lanes per contact, warps), tiles that are not full,
+bodies that take no impulses, the tolerance test, warm starts and omega."""
+import numpy as np
+import pytest
+
+from paper_1501_05810_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+GLOBAL_SYNC = 1
+
+
+def _scene(shape, precision, **kw):
+    sc = scenes.hcp_packing(*shape, dt=5e-4, mu=0.5, precision=precision, warm_start="prev", **kw)
+    rng = np.random.default_rng(sum(shape))
+    n = len(sc["radius"])
+    sc["radius"] = sc["radius"] * (1.0 - 1e-3 * rng.random(n))
+    sc["pos"][:, :2] += 0.25
+    sc["vel"] = rng.normal(0.0, 0.01, (n, 3))
+    sc["angvel"] = rng.normal(0.0, 0.01, (n, 3))
+    return sc
+
+
+def _run(sc, flags, tol, sweeps, fixed):
+    from paper_1501_05810_gb300 import nbgs
+    s = dict(sc)
+    s["params"] = dict(sc["params"], sweep_flags=flags)
+    g = nbgs.Scene(s)
+    if fixed:   # every fifth body has no linear, every seventh no angular mobility; some have neither
+        n = g.n
+        m = 4.0 / 3.0 * np.pi * sc["radius"] ** 3
+        im, iI = 1.0 / m, 2.5 / (m * sc["radius"] ** 2)
+        i = np.arange(n)
+        im[i % 5 == 0] = 0.0
+        iI[(i % 7 == 0) | (i % 10 == 0)] = 0.0
+        g.set_mass_properties(im, iI)
+    out = []
+    for _ in range(2):   # a cold and a warm-started step
+        st = g.step(sweeps, tol)
+        b = g.get_bodies()
+        out.append((st, g.residual_history(), b, g.get_contacts()))
+    g.close()
+    return out
+
+
+@pytest.mark.parametrize("shape,precision,tol,omega,fixed", [
+    ((5, 6, 2), "fp32", 0.0, 1.0, False), ((5, 6, 4), "fp32", 1e-3, 1.0, True), ((9, 10, 9), "fp32", 0.0, 0.8, True),
+    ((44, 46, 44), "fp32", 0.0, 1.0, False), ((45, 46, 46), "fp32", 0.0, 1.0, False),
+    ((70, 72, 70), "fp32", 0.0, 1.0, True), ((5, 6, 2), "fp64", 0.0, 1.0, True), ((7, 8, 6), "fp64", 1e-6, 0.9, True),
+    ((40, 40, 39), "fp64", 0.0, 1.0, False), ((40, 42, 40), "fp64", 0.0, 1.0, True)])
+def test_flow_equals_grid_synchronised_sweeps(shape, precision, tol, omega, fixed):
+    sc = _scene(shape, precision, omega=omega)
+    sweeps = 12
+    flow, ref = _run(sc, 0, tol, sweeps, fixed), _run(sc, GLOBAL_SYNC, tol, sweeps, fixed)
+    for (sa, ha, ba, ca), (sb, hb, bb, cb) in zip(flow, ref):
+        assert sa["n_contacts"] == sb["n_contacts"] and sa["n_colours"] == sb["n_colours"]
+        assert sa["sweeps_done"] == sb["sweeps_done"]
+        for k in ("j1", "j2", "colour"):
+            assert np.array_equal(ca[k], cb[k])
+        if precision == "fp32":   # the same roundings in every kernel
+            for k in ("pos", "quat", "vel", "angvel"):
+                assert np.array_equal(ba[k], bb[k]), k
+            assert np.array_equal(ca["impulse"], cb["impulse"])
+            assert np.array_equal(ha, hb) and sa["residual"] == sb["residual"]
+        else:
+            # a few roundings of 1.1e-16 per relaxation, some 12 x 12 relaxations per body and step, two
+            # steps, passed on with a gain of at most 10
+            bound = 1.1e-16 * 4 * 144 * 2 * 10
+            for k in ("vel", "angvel"):
+                assert np.abs(ba[k] - bb[k]).max() <= bound * np.abs(bb[k]).max()
+            assert np.abs(ca["impulse"] - cb["impulse"]).max() <= bound * np.abs(cb["impulse"]).max()
