@@ -43,8 +43,6 @@ __device__ __forceinline__ uint64_t local_key(uint32_t a, uint32_t b, const Scen
     return ((uint64_t)(a - off) << 32) | lb;
 }
 
-constexpr uint32_t kNoList = 0xFFFFFFFFu;   // a contact end without an incidence list (wall, infinite mass)
-
 // Priorities from the contacts' keys; body degrees from the incidence ends
 // ib1, ib2 (the contact's bodies: the contact ends themselves for spheres,
 // the members' bodies for composites; >= n marks a wall).
@@ -472,26 +470,6 @@ __global__ void k_colour_offsets(const uint32_t* __restrict__ col_count, uint32_
         }
         col_off[kMaxColours] = acc;
     }
-}
-
-// One end of a contact's dependency word from the colours of its body's
-// contacts (mask, 256 bits): the colour below c and whether c is the highest.
-__device__ __forceinline__ uint32_t dep_end(const uint32_t* __restrict__ mask, uint32_t c)
-{
-    const uint4* q = reinterpret_cast<const uint4*>(mask);
-    const uint4 lo = q[0], hi = q[1];
-    const uint32_t m[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-    const uint32_t wd = c >> 5, bit = c & 31u;
-    uint32_t pred = 0u;
-    bool last = true;
-#pragma unroll
-    for (uint32_t k = 0; k < 8; ++k) {
-        const uint32_t below = k < wd ? m[k] : (k == wd ? m[k] & ((1u << bit) - 1u) : 0u);
-        const uint32_t above = k > wd ? m[k] : (k == wd ? (m[k] >> bit) >> 1 : 0u);
-        if (below) pred = 32u * k + 32u - (uint32_t)__clz((int)below);   // colour + 1
-        if (above) last = false;
-    }
-    return pred | (last ? kDepLastA : 0u) | kDepListA;
 }
 
 // Slot of every canonical contact in colour order: the inverse of perm.

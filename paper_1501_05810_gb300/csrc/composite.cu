@@ -14,12 +14,12 @@
 // dynamics through the members and the inertia).
 //
 // Layouts: bvel R4[4 nb] = (v, 1/m), (w, 0), (Ixx, Iyy, Izz, Ixy),
-// (Ixz, Iyz, 0, 0) of the world inverse inertia; sweep record CompRec<R>
+// (Ixz, Iyz, 1/m, 0) of the world inverse inertia; sweep record CompRec<R>
 // (colour order) = (ids, bias), (n, Wnn), (l_a, Wtt), (l_b, Woo),
 // (Wnt, Wno, Wto, -).
 #include <cmath>
 
-#include "nbgs_internal.cuh"
+#include "units.cuh"
 
 namespace nbgs {
 
@@ -301,6 +301,90 @@ __device__ void one_contact_general(const Sym3<R>& W, R mu, const R b[3], R p[3]
     p[2] = po;
 }
 
+// The same solve by G lanes (a unit, aligned in the warp) on the same
+// inputs; every lane of the warp takes part, live: its unit's result is
+// wanted.  The 64 samples of the sliding condition are spread over the lanes
+// (lane j: k = j, j + G, ...; tab[k] = (cos, sin)), each root is refined by a
+// lane of its own, and the candidates are taken in the serial solver's order:
+// the result is the serial one.
+template <class R, int G>
+__device__ __forceinline__ void one_contact_on(const Sym3<R>& W, R mu, const R b[3], bool live, const R4<R>* tab, R p[3])
+{
+    static_assert(G == 4 || G == 8, "a root per lane");
+    constexpr int N = 64 / G;
+    p[0] = p[1] = p[2] = R(0);
+    const bool push = live && !(b[0] >= R(0));
+    // sticking: Cramer's rule
+    const R c00 = W.tt * W.oo - W.to * W.to;
+    const R c01 = W.to * W.no - W.nt * W.oo;
+    const R c02 = W.nt * W.to - W.tt * W.no;
+    const R det = W.nn * c00 + W.nt * c01 + W.no * c02;
+    const R i01 = W.no * W.to - W.nt * W.oo, i02 = W.nt * W.to - W.no * W.tt;
+    const R i11 = W.nn * W.oo - W.no * W.no, i12 = W.no * W.nt - W.nn * W.to;
+    const R i22 = W.nn * W.tt - W.nt * W.nt;
+    const R ps0 = -(c00 * b[0] + i01 * b[1] + i02 * b[2]) / det;
+    const R ps1 = -(c01 * b[0] + i11 * b[1] + i12 * b[2]) / det;
+    const R ps2 = -(c02 * b[0] + i12 * b[1] + i22 * b[2]) / det;
+    const bool stick = ps0 > R(0) && sqrt(ps1 * ps1 + ps2 * ps2) <= mu * ps0;
+    if (push && stick) {
+        p[0] = ps0;
+        p[1] = ps1;
+        p[2] = ps2;
+    }
+    const bool slide = push && !stick;
+    if (!__any_sync(kFull, slide)) return;
+    const R co[5] = {b[0] * W.nt - b[1] * W.nn, b[2] * W.nn - b[0] * W.no,
+                     mu * (b[0] * (W.tt - W.oo) - b[1] * W.nt + b[2] * W.no), mu * (b[0] * W.to - b[1] * W.no),
+                     mu * (b[2] * W.nt - b[0] * W.to)};
+    const uint32_t lane = threadIdx.x & 31u, j = lane % G, first = lane - j;
+    R g[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const R4<R> cs = tab[G * i + j];
+        g[i] = slide_g(co, cs.x, cs.y);
+    }
+    uint64_t marks = 0ull;   // bit k: a bracket between samples k and k + 1
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const R glo = g[i];
+        // sample k + 1: the next lane's, lane 0's next one after the last lane
+        const R ghi = __shfl_sync(kFull, j == 0u ? g[(i + 1) % N] : g[i], (int)(first + (j + 1u) % G));
+        const bool mark = glo == R(0) || ((glo < R(0)) != (ghi < R(0)) && ghi != R(0));
+        marks |= (uint64_t)((__ballot_sync(kFull, mark) >> first) & ((1u << G) - 1u)) << (G * i);
+    }
+    const R dth = (R)6.283185307179586 / (R)64;
+    const int nbr = __popcll(marks);
+    // lane r of the unit takes the r-th bracket (more than four: rounding
+    // near a double root; the serial solver goes on from there)
+    bool found = false;
+    R best = R(0), q[3] = {R(0), R(0), R(0)};
+    if (slide && (int)j < nbr && nbr <= 4) {
+        uint64_t m = marks;
+        for (uint32_t r = 0; r < j; ++r) m &= m - 1ull;
+        const int k = __ffsll((long long)m) - 1, kn = (k + 1) & 63;
+        const R4<R> c0 = tab[k], c1 = tab[kn];
+        const R glo = slide_g(co, c0.x, c0.y), ghi = slide_g(co, c1.x, c1.y);
+        slide_candidate(W, mu, b, slide_root(co, k, glo, ghi, dth), found, best, q);
+    }
+    bool any = false;
+    R e = R(0);
+    for (int r = 0; r < 4; ++r) {   // the first of least energy
+        const bool fr = __shfl_sync(kFull, found ? 1 : 0, r, G) != 0;
+        const R er = __shfl_sync(kFull, best, r, G);
+        const R q0 = __shfl_sync(kFull, q[0], r, G), q1 = __shfl_sync(kFull, q[1], r, G),
+                q2 = __shfl_sync(kFull, q[2], r, G);
+        if (slide && fr && (!any || er < e)) {
+            any = true;
+            e = er;
+            p[0] = q0;
+            p[1] = q1;
+            p[2] = q2;
+        }
+    }
+    // no qualifying root (the diagonal form), or too many brackets
+    if (slide && (!any || nbr > 4)) one_contact_general<R>(W, mu, b, p);
+}
+
 // --- per-step kernels -----------------------------------------------------
 __global__ void k_comp_ends(int64_t C, int64_t nm, int64_t nb, const uint32_t* __restrict__ cj1,
                             const uint32_t* __restrict__ cj2, const uint32_t* __restrict__ mbody,
@@ -332,20 +416,11 @@ __global__ void k_comp_iinv(int64_t nb, const double4_32a* __restrict__ bquat, c
         a.w = (R)I6[3];
         b.x = (R)I6[4];
         b.y = (R)I6[5];
-        b.z = R(0);
+        b.z = bvel[4 * i].w;   // 1/m once more, beside what does not change during a solve
         b.w = R(0);
         bvel[4 * i + 2] = a;
         bvel[4 * i + 3] = b;
     }
-}
-
-// A canonical contact position per body for the dependency windows: the
-// first contact of its first member (any fixed position serves).
-__global__ void k_comp_anchor(int64_t nb, const uint32_t* __restrict__ bfirst, const uint32_t* __restrict__ row_off,
-                              uint32_t* __restrict__ anchor)
-{
-    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nb; b += (int64_t)gridDim.x * blockDim.x)
-        anchor[b] = row_off[bfirst[b]];
 }
 
 // Sweep record of slot s (contact perm[s]) and its initial impulse.
@@ -360,8 +435,9 @@ __global__ void k_comp_records(int64_t C, int64_t nm, const uint32_t* __restrict
                                const double* __restrict__ binvm, const double4_32a* __restrict__ cgeo,
                                const double2* __restrict__ clev, double dt, double beta, double mu, int warm,
                                const uint32_t* __restrict__ prev_row_off, const uint32_t* __restrict__ prev_j2,
-                               const double4_32a* __restrict__ prev_P, CompRec<R>* __restrict__ rec,
-                               R4<R>* __restrict__ p)
+                               const double4_32a* __restrict__ prev_P, const uint32_t* __restrict__ cstate,
+                               const uint4* __restrict__ cpack, const uint32_t* __restrict__ mask,
+                               CompRec<R>* __restrict__ rec, R4<R>* __restrict__ p)
 {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < C; s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t c = perm[s];
@@ -442,13 +518,12 @@ __global__ void k_comp_records(int64_t C, int64_t nm, const uint32_t* __restrict
         rr.e.w = R(0);
         rec[s] = rr;
         // warm start: the previous world impulse in the new frame, in the cone
-        R pn = R(0), pt = R(0), po = R(0), found = R(0);
+        R pn = R(0), pt = R(0), po = R(0);
         if (warm) {
             const uint32_t e = prev_row_off[ma + 1];
             for (uint32_t k = prev_row_off[ma]; k < e; ++k) {
                 if (prev_j2[k] != mbm) continue;
                 const double4_32a P = prev_P[k];
-                found = R(1);
                 pn = (R)(n[0] * P.x + n[1] * P.y + n[2] * P.z);
                 if (!(pn > R(0))) pn = R(0);
                 pt = (R)(t[0] * P.x + t[1] * P.y + t[2] * P.z);
@@ -469,7 +544,12 @@ __global__ void k_comp_records(int64_t C, int64_t nm, const uint32_t* __restrict
         q.x = pn;
         q.y = pt;
         q.z = po;
-        q.w = found;
+        const uint32_t col = cstate[c] & 0xFFu;
+        const uint4 ends = cpack[c];
+        uint32_t dep = 0u;
+        if (ends.x != kNoList) dep |= dep_end(mask + 8 * (int64_t)ends.x, col);
+        if (ends.y != kNoList) dep |= dep_end(mask + 8 * (int64_t)ends.y, col) << 11;
+        dep_store(dep, q.w);
         p[s] = q;
     }
 }
@@ -479,11 +559,14 @@ __global__ void k_comp_records(int64_t C, int64_t nm, const uint32_t* __restrict
 template <class R>
 __global__ void k_comp_velinit(int64_t nb, const double4_32a* __restrict__ bquat, const double* __restrict__ bI0,
                                const double* __restrict__ bIinv, const double* __restrict__ binvm, double3 gdt,
-                               double dt, R4<R>* __restrict__ bvel)
+                               double dt, R4<R>* __restrict__ bvel, uint4* __restrict__ tv)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nb; i += (int64_t)gridDim.x * blockDim.x) {
-        if (!(binvm[i] > 0.0)) continue;
         R4<R> v = bvel[4 * i], w = bvel[4 * i + 1];
+        if (!(binvm[i] > 0.0)) {
+            if (tv) pack_body(tv + Words<R>::N * i, 0u, v, w);
+            continue;
+        }
         double Rm[3][3], I[3][3];
         quat_rows(bquat[i], Rm);
         to_world(Rm, bI0 + 9 * i, I);
@@ -501,14 +584,13 @@ __global__ void k_comp_velinit(int64_t nb, const double4_32a* __restrict__ bquat
         v.z = (R)((double)v.z + gdt.z);
         bvel[4 * i] = v;
         bvel[4 * i + 1] = w;
+        if (tv) pack_body(tv + Words<R>::N * i, 0u, v, w);
     }
 }
 
 template <class R> struct CompArgs {
-    int local;                 // dependency windows (else a grid barrier after every colour)
-    int* prog;                 // per block: last sweep phase completed
-    const int2* dep;           // per (colour, block): ring window of blocks sharing bodies with the chunk
-    const uint32_t* cstart;    // per colour, B + 1 chunk boundaries
+    uint4* tv;                 // versioned velocities (the dataflow sweeps)
+    int tile;                  // contacts per tile
     int64_t C, nb;
     const CompRec<R>* rec;
     R4<R>* p;
@@ -522,13 +604,15 @@ template <class R> struct CompArgs {
     int warm;
 };
 
-// Relax one composite contact (apply_only: add the stored impulse), its
-// record and impulse already loaded.
-template <class R, bool apply_only>
-__device__ __forceinline__ R relax_comp_loaded(const CompArgs<R>& A, int64_t s, const CompRec<R>& rr, const R4<R>& pp)
+// State of the two bodies of a contact: (v, 1/m), w and the six entries of the
+// world inverse inertia.
+template <class R> struct CompBodies {
+    R4<R> va, wa, ia1, ia2, vb, wb, ib1, ib2;
+};
+
+template <class R>
+__device__ __forceinline__ void comp_ids(const CompRec<R>& rr, uint32_t& ia, uint32_t& ib, R& bias)
 {
-    uint32_t ia, ib;
-    R bias;
     if constexpr (sizeof(R) == 4) {
         ia = __float_as_uint(rr.a.x);
         ib = __float_as_uint(rr.a.y);
@@ -539,25 +623,26 @@ __device__ __forceinline__ R relax_comp_loaded(const CompArgs<R>& A, int64_t s, 
         ib = (uint32_t)(ids >> 32);
         bias = rr.a.y;
     }
-    const bool hasB = ib < (uint64_t)A.nb;
+}
+
+// Relax one composite contact (apply_only: add the stored impulse) on loaded
+// bodies: the velocities in B and the impulse pp (xyz) are updated.  G lanes
+// run it together (one_contact_on).  False in `moves`: nothing can move.
+template <class R, bool apply_only, int G>
+__device__ __forceinline__ R relax_comp_bodies(R mu, R omega, const CompRec<R>& rr, bool hasB, R4<R>& pp,
+                                               CompBodies<R>& B, const R4<R>* tab, bool live, bool& moves)
+{
+    uint32_t ia, ib;
+    R bias;
+    comp_ids<R>(rr, ia, ib, bias);
     const Sym3<R> W = {rr.b.w, rr.c.w, rr.d.w, rr.e.x, rr.e.y, rr.e.z};
-    if (!(W.nn > R(0))) return R(0);
+    moves = live && W.nn > R(0);
+    if (G == 1 && !moves) return R(0);
     const R n[3] = {rr.b.x, rr.b.y, rr.b.z};
     const R lA[3] = {rr.c.x, rr.c.y, rr.c.z}, lB[3] = {rr.d.x, rr.d.y, rr.d.z};
     R t[3], o[3];
     tangent_basis<R>(n[0], n[1], n[2], t[0], t[1], t[2], o[0], o[1], o[2]);
-    // a body's state is 4 vectors: v, w and the 6 entries of its world inverse
-    // inertia, read as two 256-bit accesses
-    R4<R> va, wa, ia1, ia2;
-    ld_body(A.bv + 4 * (int64_t)ia, va, wa);
-    ld_body(A.bv + 4 * (int64_t)ia + 2, ia1, ia2);
-    R4<R> vb, wb, ib1, ib2;
-    vb.x = vb.y = vb.z = vb.w = R(0);
-    wb = ib1 = ib2 = vb;
-    if (hasB) {
-        ld_body(A.bv + 4 * (int64_t)ib, vb, wb);
-        ld_body(A.bv + 4 * (int64_t)ib + 2, ib1, ib2);
-    }
+    R4<R>&va = B.va, &wa = B.wa, &vb = B.vb, &wb = B.wb;
     R d[3];
     if (apply_only) {
         d[0] = pp.x;
@@ -578,22 +663,27 @@ __device__ __forceinline__ R relax_comp_loaded(const CompArgs<R>& A, int64_t s, 
         b[1] = ut - (W.nt * pp.x + W.tt * pp.y + W.to * pp.z);
         b[2] = uo - (W.no * pp.x + W.to * pp.y + W.oo * pp.z);
         R y[3];
-        one_contact_general<R>(W, A.mu, b, y);
-        const R om = A.omega, om1 = R(1) - A.omega;
+        if constexpr (G == 1) one_contact_general<R>(W, mu, b, y);
+        else one_contact_on<R, G>(W, mu, b, moves, tab, y);
+        const R om = omega, om1 = R(1) - omega;
         R4<R> q;
         q.x = om * y[0] + om1 * pp.x;
         q.y = om * y[1] + om1 * pp.y;
         q.z = om * y[2] + om1 * pp.z;
-        q.w = R(0);
         d[0] = q.x - pp.x;
         d[1] = q.y - pp.y;
         d[2] = q.z - pp.z;
-        A.p[s] = q;
+        if (moves) {
+            pp.x = q.x;
+            pp.y = q.y;
+            pp.z = q.z;
+        }
     }
+    if (!moves) return R(0);
     const R P[3] = {d[0] * n[0] + d[1] * t[0] + d[2] * o[0], d[0] * n[1] + d[1] * t[1] + d[2] * o[1],
                     d[0] * n[2] + d[1] * t[2] + d[2] * o[2]};
     if (va.w > R(0)) {
-        const R I6[6] = {ia1.x, ia1.y, ia1.z, ia1.w, ia2.x, ia2.y};
+        const R I6[6] = {B.ia1.x, B.ia1.y, B.ia1.z, B.ia1.w, B.ia2.x, B.ia2.y};
         R tq[3], dw[3];
         cross(lA, P, tq);
         sym_mul(I6, tq, dw);
@@ -603,10 +693,9 @@ __device__ __forceinline__ R relax_comp_loaded(const CompArgs<R>& A, int64_t s, 
         wa.x += dw[0];
         wa.y += dw[1];
         wa.z += dw[2];
-        st_body(A.bv + 4 * (int64_t)ia, va, wa);
     }
     if (hasB && vb.w > R(0)) {
-        const R I6[6] = {ib1.x, ib1.y, ib1.z, ib1.w, ib2.x, ib2.y};
+        const R I6[6] = {B.ib1.x, B.ib1.y, B.ib1.z, B.ib1.w, B.ib2.x, B.ib2.y};
         R tq[3], dw[3];
         cross(lB, P, tq);
         sym_mul(I6, tq, dw);
@@ -616,12 +705,41 @@ __device__ __forceinline__ R relax_comp_loaded(const CompArgs<R>& A, int64_t s, 
         wb.x -= dw[0];
         wb.y -= dw[1];
         wb.z -= dw[2];
-        st_body(A.bv + 4 * (int64_t)ib, vb, wb);
     }
     const R r0 = W.nn * d[0] + W.nt * d[1] + W.no * d[2];
     const R r1 = W.nt * d[0] + W.tt * d[1] + W.to * d[2];
     const R r2 = W.no * d[0] + W.to * d[1] + W.oo * d[2];
     return sqrt(r0 * r0 + r1 * r1 + r2 * r2);
+}
+
+// The same with the bodies read from and written to their records (a colour's
+// contacts share no finite body).
+template <class R, bool apply_only>
+__device__ __forceinline__ R relax_comp_loaded(const CompArgs<R>& A, int64_t s, const CompRec<R>& rr, const R4<R>& p0)
+{
+    uint32_t ia, ib;
+    R bias;
+    comp_ids<R>(rr, ia, ib, bias);
+    const bool hasB = ib < (uint64_t)A.nb;
+    // a body's state is 4 vectors: v, w and the 6 entries of its world inverse
+    // inertia, read as two 256-bit accesses
+    CompBodies<R> B;
+    ld_body(A.bv + 4 * (int64_t)ia, B.va, B.wa);
+    ld_body(A.bv + 4 * (int64_t)ia + 2, B.ia1, B.ia2);
+    B.vb.x = B.vb.y = B.vb.z = B.vb.w = R(0);
+    B.wb = B.ib1 = B.ib2 = B.vb;
+    if (hasB) {
+        ld_body(A.bv + 4 * (int64_t)ib, B.vb, B.wb);
+        ld_body(A.bv + 4 * (int64_t)ib + 2, B.ib1, B.ib2);
+    }
+    R4<R> pp = p0;
+    bool moves;
+    const R r = relax_comp_bodies<R, apply_only, 1>(A.mu, A.omega, rr, hasB, pp, B, nullptr, true, moves);
+    if (!moves) return R(0);
+    if (!apply_only) A.p[s] = pp;
+    if (B.va.w > R(0)) st_body(A.bv + 4 * (int64_t)ia, B.va, B.wa);
+    if (hasB && B.vb.w > R(0)) st_body(A.bv + 4 * (int64_t)ib, B.vb, B.wb);
+    return r;
 }
 
 template <class R, bool apply_only>
@@ -648,9 +766,9 @@ __device__ __forceinline__ void block_max_atomic(double x, unsigned long long* d
 
 constexpr int kCompThreads = 256;
 
-// The whole composite solve in one cooperative launch: the initial impulses
-// colour by colour, then the sweeps, a grid barrier after every colour (each
-// colour's contacts touch disjoint finite bodies) and R_k after every sweep.
+// The composite solve with NBGS_SWEEP_GLOBAL_SYNC: the initial impulses colour
+// by colour, then the sweeps, a grid barrier after every colour (each colour's
+// contacts touch disjoint finite bodies) and R_k after every sweep.
 template <class R>
 __global__ void __launch_bounds__(kCompThreads) k_solve_comp(CompArgs<R> A)
 {
@@ -666,71 +784,210 @@ __global__ void __launch_bounds__(kCompThreads) k_solve_comp(CompArgs<R> A)
             if (!grid_barrier(A.info, nb)) return;
         }
     }
-    __shared__ int s_ok;
     int k = 0;
     double Rk = 0.0;
-    bool synced = true;
     for (; k < A.max_sweeps; ++k) {
         if (blockIdx.x == 0 && threadIdx.x == 0 && k + 1 >= kHistKept) A.info->rk_bits[rk_slot(k + 1)] = 0ull;
         R rmax = R(0);
         for (int c = 0; c < ncol; ++c) {
-            if (A.local) {
-                // this block's chunk of the colour, after the blocks sharing
-                // its bodies have finished the phase before
-                const int g = k * ncol + c;
-                int64_t b0, b1;
-                colour_chunk(A.cstart, c, b0, b1);
-                // the first record and impulse of this thread do not depend on
-                // the neighbours: loaded before the wait
-                const int64_t s0 = b0 + threadIdx.x;
-                CompRec<R> rr;
-                R4<R> pp;
-                if (s0 < b1) {
-                    rr = A.rec[s0];
-                    pp = A.p[s0];
-                }
-                if (b1 > b0 && !wait_deps(A.prog, A.dep[c * (int)nb + blockIdx.x], g, A.info, &s_ok)) return;
-                for (int64_t s = s0; s < b1; s += blockDim.x) {
-                    if (s != s0) {
-                        rr = A.rec[s];
-                        pp = A.p[s];
-                    }
-                    const R r = relax_comp_loaded<R, false>(A, s, rr, pp);
-                    rmax = r > rmax ? r : rmax;
-                }
-                if (c == ncol - 1) block_max_atomic((double)rmax, &A.info->rk_bits[rk_slot(k)]);
-                publish(A.prog, g);
-            } else {
-                for (int64_t s = A.col_off[c] + gtid; s < A.col_off[c + 1]; s += gstride) {
-                    const R r = relax_comp<R, false>(A, s);
-                    rmax = r > rmax ? r : rmax;
-                }
-                if (c == ncol - 1) block_max_atomic((double)rmax, &A.info->rk_bits[rk_slot(k)]);
-                if (!grid_barrier(A.info, nb)) return;
+            for (int64_t s = A.col_off[c] + gtid; s < A.col_off[c + 1]; s += gstride) {
+                const R r = relax_comp<R, false>(A, s);
+                rmax = r > rmax ? r : rmax;
             }
-        }
-        synced = !A.local;
-        // R_k needs every block: a grid barrier per sweep when the tolerance
-        // is tested (and near the rotating residual slots)
-        if (A.local && ncol > 0 && (A.tol > 0.0 || k + 2 >= kHistKept)) {
+            if (c == ncol - 1) block_max_atomic((double)rmax, &A.info->rk_bits[rk_slot(k)]);
             if (!grid_barrier(A.info, nb)) return;
-            synced = true;
         }
-        if (synced) {
-            Rk = __longlong_as_double((long long)((volatile unsigned long long*)A.info->rk_bits)[rk_slot(k)]) / vref;
-            if (A.tol > 0.0 && ncol > 0 && Rk <= A.tol) {
-                ++k;
-                break;
-            }
+
+        Rk = __longlong_as_double((long long)((volatile unsigned long long*)A.info->rk_bits)[rk_slot(k)]) / vref;
+        if (A.tol > 0.0 && ncol > 0 && Rk <= A.tol) {
+            ++k;
+            break;
         }
-    }
-    if (!synced && k > 0) {
-        if (!grid_barrier(A.info, nb)) return;
-        Rk = __longlong_as_double((long long)((volatile unsigned long long*)A.info->rk_bits)[rk_slot(k - 1)]) / vref;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         A.info->sweeps_done = (uint32_t)k;
         A.info->residual = Rk;
+        A.info->v_ref = vref;
+    }
+}
+
+// The composite sweeps as a dataflow over body versions (flow.cu has the
+// scheme): G lanes per contact, 32 / G contacts per tile, the tiles of all
+// colours dealt to the warps in turn.  The inverse inertia and 1/m of a body
+// do not change during a solve and are read beside its versioned velocities.
+template <class R, int G>
+__global__ void __launch_bounds__(kCompThreads, sizeof(R) == 4 ? 2 : 1) k_flow_comp(CompArgs<R> A)
+{
+    __shared__ uint32_t s_tile[kMaxColours + 1], s_off[kMaxColours + 1];
+    __shared__ R4<R> s_tab[64];
+    __shared__ int s_vote;
+    const int ncol = min((int)A.info->n_colours, kMaxColours);
+    const unsigned nb = gridDim.x;
+    const int lane = threadIdx.x & 31;
+    const uint32_t tw = (uint32_t)A.tile;
+    tile_offsets(A.col_off, ncol, tw, s_off, s_tile);
+    if (threadIdx.x < 64) {
+        s_tab[threadIdx.x].x = tab_cos<R>(threadIdx.x);
+        s_tab[threadIdx.x].y = tab_sin<R>(threadIdx.x);
+    }
+    __syncthreads();
+    const uint32_t ntile = s_tile[ncol];
+    const uint32_t W = nb * (blockDim.x >> 5), w0 = (threadIdx.x >> 5) * nb + blockIdx.x;
+    const bool work = w0 < ntile;
+    const double vref = v_ref_of(A.info, A.gdt_norm);
+    const int warm = A.warm ? 1 : 0, npass = A.max_sweeps + warm;
+    const uint32_t unit = (uint32_t)(lane / G);
+    bool ok = true;
+    CompRec<R> rr;
+    R4<R> pp;
+    uint32_t s = 0, T = w0;
+    int c = 0, k = 0;
+    bool on = false;
+    auto read = [&]() {   // the unit's contact of tile T
+        while (T >= s_tile[c + 1]) ++c;
+        s = s_off[c] + (T - s_tile[c]) * tw + unit;
+        on = unit < tw && s < s_off[c + 1];
+        if (on) {
+            rr = A.rec[s];
+            pp = A.p[s];
+        }
+    };
+    if (work) read();
+    for (int pass = 0; pass < npass; ++pass) {
+        const bool apply = pass < warm;
+        k = pass - warm;
+        if (!apply && blockIdx.x == 0 && threadIdx.x == 0 && k + 1 >= kHistKept) A.info->rk_bits[rk_slot(k + 1)] = 0ull;
+        R rmax = R(0);
+        const uint32_t base = (uint32_t)pass << 9;
+        for (bool more = work; more && ok;) {
+            uint32_t ia = 0, ib = 0;
+            R bias;
+            bool hasB = false;
+            CompBodies<R> B;
+            if (on) {
+                comp_ids<R>(rr, ia, ib, bias);
+                hasB = ib < (uint64_t)A.nb;
+            }
+            if (!hasB) ib = ia;
+            const uint32_t ia0 = __shfl_sync(kFull, ia, 0);
+            if (!on) ia = ib = ia0;
+            // what does not change, then the versioned velocities
+            const R4<R>* sa = A.bv + 4 * (int64_t)ia + 2;
+            const R4<R>* sb = A.bv + 4 * (int64_t)ib + 2;
+            B.ia1 = sa[0];
+            B.ia2 = sa[1];
+            B.ib1 = sb[0];
+            B.ib2 = sb[1];
+            const uint32_t dep = on ? dep_bits(pp.w) : 0u;
+            const bool va = (dep & kDepListA) != 0u, vb = hasB && (dep & kDepListB) != 0u;
+            const uint32_t ea = base | (dep & 0x1FFu), eb = base | ((dep >> 11) & 0x1FFu);
+            const uint32_t after = base | (uint32_t)(c + 1), next = base + 512u;
+            const uint4* qa = A.tv + Words<R>::N * (size_t)ia;
+            const uint4* qb = A.tv + Words<R>::N * (size_t)ib;
+            const long long t0 = clock64();
+            for (int polls = 0;;) {
+                uint32_t ta[Words<R>::N], tb[Words<R>::N];
+                load_body(qa, B.va, B.wa, ta);
+                load_body(qb, B.vb, B.wb, tb);
+                bool ready = true;
+#pragma unroll
+                for (int j = 0; j < Words<R>::N; ++j) ready = ready && (!va || ta[j] == ea) && (!vb || tb[j] == eb);
+                if (__all_sync(kFull, ready)) break;
+                if ((++polls & 255) == 0) {   // bounded like every other wait
+                    bool give_up = (((volatile uint32_t*)&A.info->err)[0] & kErrTimeout) != 0u;
+                    if (clock64() - t0 > (1LL << 31)) {
+                        if (lane == 0) atomicOr(&A.info->err, kErrTimeout);
+                        give_up = true;
+                    }
+                    if (__any_sync(kFull, give_up)) {
+                        ok = false;
+                        break;
+                    }
+                }
+            }
+            if (!ok) break;
+            B.va.w = B.ia2.z;
+            B.vb.w = hasB ? B.ib2.z : R(0);
+            if (!hasB) {
+                B.vb.x = B.vb.y = B.vb.z = R(0);
+                B.wb.x = B.wb.y = B.wb.z = R(0);
+            }
+            bool moves;
+            R r = R(0);
+            if (G > 1 || on) {
+                if (apply) r = relax_comp_bodies<R, true, G>(A.mu, A.omega, rr, hasB, pp, B, s_tab, on, moves);
+                else r = relax_comp_bodies<R, false, G>(A.mu, A.omega, rr, hasB, pp, B, s_tab, on, moves);
+            }
+            if (lane % G == 0) {
+                if (va) pack_body(A.tv + Words<R>::N * (size_t)ia, (dep & kDepLastA) ? next : after, B.va, B.wa);
+                if (vb) pack_body(A.tv + Words<R>::N * (size_t)ib, (dep & kDepLastB) ? next : after, B.vb, B.wb);
+                if (on && !apply) A.p[s] = pp;
+            }
+            if (on && !apply) rmax = r > rmax ? r : rmax;
+            __syncwarp();   // the lanes of a unit read back what one of them saved
+            more = T + W < ntile;
+            const uint32_t Tn = more ? T + W : w0;
+            if (Tn != T) {
+                T = Tn;
+                if (!more) c = 0;
+                read();
+            }
+        }
+        if (apply) continue;
+        const bool vote = ncol > 0 && A.tol > 0.0 && k + 2 < kHistKept;
+        const bool sync = ncol > 0 && !vote && (A.tol > 0.0 || k + 2 >= kHistKept);
+        if (!vote && !sync) {
+            if (!ok) break;
+            if (work) {
+                for (int o = 16; o > 0; o >>= 1) rmax = fmax(rmax, __shfl_xor_sync(kFull, rmax, o));
+                if (lane == 0) {
+                    double x = (double)rmax;
+                    if (!(x <= 1e300)) x = __longlong_as_double(0x7FF0000000000000LL);
+                    atomicMax(&A.info->rk_bits[rk_slot(k)], (unsigned long long)__double_as_longlong(x));
+                }
+            }
+            continue;
+        }
+        if (!__syncthreads_and(ok)) {
+            ok = false;
+            break;
+        }
+        const double rb = block_max_to<R>(rmax, &A.info->rk_bits[rk_slot(k)]);
+        if (vote) {
+            const int v = tol_vote(A.info, k, rb, vref, A.tol, nb, &s_vote);
+            if (v < 0) ok = false;
+            if (v <= 0) break;
+            continue;
+        }
+        if (!grid_barrier(A.info, nb)) {
+            ok = false;
+            break;
+        }
+        const double Rk = __longlong_as_double((long long)((volatile unsigned long long*)A.info->rk_bits)[rk_slot(k)]) / vref;
+        if (A.tol > 0.0 && Rk <= A.tol) break;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && ok)
+        A.info->sweeps_done = (uint32_t)(A.max_sweeps == 0 ? 0 : min(k + 1, A.max_sweeps));
+}
+
+// The solved velocities back into the body records, and the solve's outcome.
+template <class R>
+__global__ void k_flow_comp_out(CompArgs<R> A)
+{
+    const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int64_t i = gtid; i < A.nb; i += (int64_t)gridDim.x * blockDim.x) {
+        R4<R> v, w;
+        uint32_t tags[Words<R>::N];
+        load_body(A.tv + Words<R>::N * i, v, w, tags);
+        v.w = A.bv[4 * i + 3].z;
+        w.w = R(0);
+        A.bv[4 * i] = v;
+        A.bv[4 * i + 1] = w;
+    }
+    if (gtid == 0) {
+        const int k = (int)A.info->sweeps_done;
+        const double vref = v_ref_of(A.info, A.gdt_norm);
+        A.info->residual = k > 0 ? __longlong_as_double((long long)A.info->rk_bits[rk_slot(k - 1)]) / vref : 0.0;
         A.info->v_ref = vref;
     }
 }
@@ -837,6 +1094,29 @@ int comp_blocks(nbgs_scene* s)
     return occ * s->num_sms;
 }
 
+// Lanes per contact of the dataflow sweeps.  Few contacts at a time: the
+// sliding search of each is what a sweep waits for, so eight lanes share it;
+// with more the lanes' repeated arithmetic costs more than it hides.  50
+// sweeps of a pile, ms, one GB300 (FP32, 2 contacts per body, 14 to 22
+// colours; "windows" the colour phases of before):
+//   bodies       1k     10k    30k    100k   200k   300k   500k   1M
+//   windows      3.27   4.39   5.11   5.89          7.85          15.6
+//   1 lane       3.81   4.63   5.70   6.64   7.38   7.32   9.02   13.9
+//   4 lanes      1.52   1.84   2.25   2.65   3.75   4.78   8.14   16.4
+//   8 lanes      1.06   1.26   1.82   2.78   4.57   6.64   11.9   26.3
+// FP64: 29.5 / 13.0 / 9.3 at 1k and 47.7 / 30.5 / 38.7 at 100k (windows 23.6, 49.8).
+struct CompPlan {
+    const void* fn;
+    int tile;
+};
+template <class R>
+CompPlan comp_plan(int64_t nb)
+{
+    if (nb < 60000) return {(const void*)k_flow_comp<R, 8>, 4};
+    if (nb < 600000) return {(const void*)k_flow_comp<R, 4>, 8};
+    return {(const void*)k_flow_comp<R, 1>, 32};
+}
+
 template <class R>
 nbgs_status solve_comp_impl(nbgs_scene* s, int max_sweeps, double tol)
 {
@@ -848,9 +1128,14 @@ nbgs_status solve_comp_impl(nbgs_scene* s, int max_sweeps, double tol)
     const double* g = s->prm.gravity;
     const double3 gdt = make_double3(s->prm.dt * g[0], s->prm.dt * g[1], s->prm.dt * g[2]);
     if (s->timing) cudaEventRecord(s->ev[8], st);
+    // the dataflow sweeps unless a grid barrier per colour is asked for; their
+    // versioned records take the state-transfer staging buffer
+    const bool flow = s->n_contacts > 0 && !(s->prm.sweep_flags & NBGS_SWEEP_GLOBAL_SYNC);
+    uint4* tv = flow ? (uint4*)s->stage : nullptr;
     k_comp_velinit<R><<<grid_for(s->nb, T, 8, s->num_sms), T, 0, st>>>(s->nb, s->bquat, s->bI0, s->bIinv, s->binvm, gdt,
-                                                                       s->prm.dt, (R4<R>*)s->bvel);
+                                                                       s->prm.dt, (R4<R>*)s->bvel, tv);
     CompArgs<R> A;
+    A.tv = tv;
     A.C = s->n_contacts;
     A.nb = s->nb;
     A.rec = (const CompRec<R>*)s->crec;
@@ -866,15 +1151,25 @@ nbgs_status solve_comp_impl(nbgs_scene* s, int max_sweeps, double tol)
     A.warm = (s->prm.warm_start == NBGS_WARM_PREV && s->have_prev) ? 1 : 0;
     const int blocks = std::min(comp_blocks<R>(s), s->max_coop_blocks);
     if (blocks < 1) return fail(s, NBGS_EINVAL, "composite solve: the device cannot launch it cooperatively");
-    // local synchronisation unless a grid barrier per colour is asked for
-    A.local = (A.C > 0 && !(s->prm.sweep_flags & NBGS_SWEEP_GLOBAL_SYNC)) ? 1 : 0;
-    A.prog = s->prog;
-    A.dep = s->dep;
-    A.cstart = s->cstart;
-    if (A.local) {
-        k_comp_anchor<<<grid_for(s->nb, T, 8, s->num_sms), T, 0, st>>>(s->nb, s->bfirst, s->row_off, s->banchor);
-        nbgs_status rc = build_windows(s, blocks, s->nb, s->cb1, s->cb2, s->banchor, s->bfinite);
-        if (rc != NBGS_OK) return rc;
+    if (flow) {
+        cudaMemsetAsync(s->info->votes, 0, (size_t)(nk > 0 ? 2 * nk : 2) * sizeof(uint32_t), st);
+        const CompPlan P = comp_plan<R>(s->nb);
+        A.tile = P.tile;
+        int occ = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, P.fn, kCompThreads, 0);
+        cudaGetLastError();
+        const int grid = occ * s->num_sms;
+        if (grid < 1) return fail(s, NBGS_EINVAL, "composite solve: the device cannot launch it cooperatively");
+        void* fargs[] = {&A};
+        const cudaError_t fe = cudaLaunchCooperativeKernel(P.fn, dim3(grid), dim3(kCompThreads), fargs, 0, st);
+        if (s->timing) {
+            cudaEventRecord(s->ev[9], st);
+            s->phase_launches[2] += 3;
+            s->sweep_launches += 1;
+        }
+        if (fe != cudaSuccess) return cuda_check(s, fe, "composite solve: cooperative launch");
+        k_flow_comp_out<R><<<grid_for(s->nb, T, 8, s->num_sms), T, 0, st>>>(A);
+        return cuda_check(s, cudaGetLastError(), "composite solve");
     }
     void* args[] = {&A};
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_solve_comp<R>, dim3(blocks), dim3(kCompThreads), args, 0,
@@ -892,7 +1187,7 @@ nbgs_status solve_comp_impl(nbgs_scene* s, int max_sweeps, double tol)
 void free_composite_buffers(nbgs_scene* s)
 {
     void* ps[] = {s->bpos, s->bquat, s->bvel, s->bI0, s->bI0inv, s->bIinv, s->binvm, s->bfinite, s->mbody,
-                  s->moff, s->cb1, s->cb2, s->crec, s->bfirst, s->banchor};
+                  s->moff, s->cb1, s->cb2, s->crec};
     for (void* p : ps) dev_free(s, p);
 }
 
@@ -953,15 +1248,15 @@ nbgs_status run_comp_records(nbgs_scene* s, int warm)
                                                                              (float4*)s->bvel);
         k_comp_records<float><<<grid_for(C, T, 8, s->num_sms), T, 0, st>>>(
             C, s->n, s->perm, s->cj1, s->cj2, s->mbody, s->moff, s->bquat, s->bIinv, s->binvm, s->cgeo, s->clev,
-            s->prm.dt, s->prm.beta, s->prm.mu, warm, s->prev_row_off, s->prev_j2, s->prev_P,
-            (CompRec<float>*)s->crec, (float4*)s->sp);
+            s->prm.dt, s->prm.beta, s->prm.mu, warm, s->prev_row_off, s->prev_j2, s->prev_P, s->cstate, s->cpack,
+            s->cmask, (CompRec<float>*)s->crec, (float4*)s->sp);
     } else {
         k_comp_iinv<double><<<grid_for(s->nb, T, 8, s->num_sms), T, 0, st>>>(s->nb, s->bquat, s->bI0inv, s->bIinv,
                                                                               (double4_32a*)s->bvel);
         k_comp_records<double><<<grid_for(C, T, 8, s->num_sms), T, 0, st>>>(
             C, s->n, s->perm, s->cj1, s->cj2, s->mbody, s->moff, s->bquat, s->bIinv, s->binvm, s->cgeo, s->clev,
-            s->prm.dt, s->prm.beta, s->prm.mu, warm, s->prev_row_off, s->prev_j2, s->prev_P,
-            (CompRec<double>*)s->crec, (double4_32a*)s->sp);
+            s->prm.dt, s->prm.beta, s->prm.mu, warm, s->prev_row_off, s->prev_j2, s->prev_P, s->cstate, s->cpack,
+            s->cmask, (CompRec<double>*)s->crec, (double4_32a*)s->sp);
     }
     if (s->timing) s->phase_launches[1] += 2;
     return cuda_check(s, cudaGetLastError(), "composite: sweep records");

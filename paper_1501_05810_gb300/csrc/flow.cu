@@ -142,24 +142,7 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
     const unsigned nb = gridDim.x;
     const int lane = threadIdx.x & 31;
     const uint32_t tw = (uint32_t)A.tile;
-    for (int c = threadIdx.x; c <= ncol; c += blockDim.x) s_off[c] = A.col_off[c];
-    __syncthreads();
-    if (threadIdx.x < 32) {   // tiles before every colour
-        uint32_t carry = 0;
-        for (int c0 = 0; c0 < ncol; c0 += 32) {
-            const int c = c0 + lane;
-            uint32_t v = c < ncol ? (s_off[c + 1] - s_off[c] + tw - 1) / tw : 0u;
-            const uint32_t own = v;
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
-                if (lane >= o) v += y;
-            }
-            if (c < ncol) s_tile[c] = carry + v - own;
-            carry += __shfl_sync(0xffffffffu, v, 31);
-        }
-        if (lane == 0) s_tile[ncol] = carry;
-    }
-    __syncthreads();
+    tile_offsets(A.col_off, ncol, tw, s_off, s_tile);
     const uint32_t ntile = s_tile[ncol];
     // warp w of the grid: warps 0 of all blocks first, so that few tiles spread over the SMs
     const uint32_t W = nb * (blockDim.x >> 5), w0 = (threadIdx.x >> 5) * nb + blockIdx.x;

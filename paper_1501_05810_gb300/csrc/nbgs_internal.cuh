@@ -25,6 +25,7 @@ constexpr int kMaxPlanes = 16;
 constexpr int kMaxColours = 256;       // a colour is 8 bits of the colouring state
 constexpr int kCandCap = 32;           // sphere candidates per body with j > i
 constexpr uint32_t kUncoloured = 0xFFFFFFFFu;
+constexpr uint32_t kNoList = 0xFFFFFFFFu;   // a contact end without an incidence list (wall, infinite mass)
 constexpr int kMaxSweepsHist = 4096;   // residual slots: history, 3 rotating, 4 final
 constexpr int kHistKept = kMaxSweepsHist - 8;   // sweeps whose R_k is kept
 
@@ -510,8 +511,6 @@ struct nbgs_scene {
     double* binvm = nullptr;       // nb: 1/m (FP64)
     uint8_t* bfinite = nullptr;    // nb
     uint32_t* mbody = nullptr;     // n: body of each member
-    uint32_t* bfirst = nullptr;    // nb: first member of each body
-    uint32_t* banchor = nullptr;   // nb: a canonical contact position per body (dependency windows)
     double4_32a* moff = nullptr;   // n: body-frame offset from the centre of mass, radius
     uint32_t* cb1 = nullptr;       // comp_ccap: body of contact end j1
     uint32_t* cb2 = nullptr;       // comp_ccap: body of contact end j2 (nb: a wall)
@@ -580,8 +579,6 @@ bool subdomains_valid(int32_t mode, const int32_t g[3]);   // api.cu
 // composite particles (composite.cu)
 nbgs_status ensure_composite_buffers(nbgs_scene* s);
 nbgs_status run_comp_ends(nbgs_scene* s);               // bodies of the contact ends (colouring)
-nbgs_status build_windows(nbgs_scene* s, int B, int64_t ninc, const uint32_t* ib1, const uint32_t* ib2,
-                          const uint32_t* anchor, const uint8_t* finc);   // solve.cu
 nbgs_status run_comp_records(nbgs_scene* s, int warm);   // after colouring: inverse inertias, sweep records
 nbgs_status run_solve_comp(nbgs_scene* s, int max_sweeps, double tol);
 nbgs_status run_integrate_comp(nbgs_scene* s);

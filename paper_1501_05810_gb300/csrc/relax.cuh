@@ -261,6 +261,26 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, DevInf
     return true;
 }
 
+// One end of a contact's dependency word from the colours of its body's
+// contacts (mask, 256 bits): the colour below c and whether c is the highest.
+__device__ __forceinline__ uint32_t dep_end(const uint32_t* __restrict__ mask, uint32_t c)
+{
+    const uint4* q = reinterpret_cast<const uint4*>(mask);
+    const uint4 lo = q[0], hi = q[1];
+    const uint32_t m[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    const uint32_t wd = c >> 5, bit = c & 31u;
+    uint32_t pred = 0u;
+    bool last = true;
+#pragma unroll
+    for (uint32_t k = 0; k < 8; ++k) {
+        const uint32_t below = k < wd ? m[k] : (k == wd ? m[k] & ((1u << bit) - 1u) : 0u);
+        const uint32_t above = k > wd ? m[k] : (k == wd ? (m[k] >> bit) >> 1 : 0u);
+        if (below) pred = 32u * k + 32u - (uint32_t)__clz((int)below);   // colour + 1
+        if (above) last = false;
+    }
+    return pred | (last ? kDepLastA : 0u) | kDepListA;
+}
+
 // Rotating per-scene residual slot of sweep k (three, so that clearing the
 // slot of sweep k + 1 while sweep k runs touches nothing still read).
 __host__ __device__ __forceinline__ int scene_slot(int k) { return k % 3; }

@@ -839,33 +839,6 @@ __global__ void k_chunk_windows(DCount Cc, int64_t n, const uint32_t* __restrict
     }
 }
 
-// Chunk starts and dependency windows of a cooperative sweep over B blocks,
-// for contacts whose ends act on the bodies ib1, ib2 (>= ninc: a wall) of
-// finiteness finc, body x anchored at the canonical contact position
-// anchor[x] (any fixed position: the windows are offsets from it); the
-// progress words start at -1.  The body degree arrays of the colouring serve
-// as scratch.
-nbgs_status build_windows(nbgs_scene* s, int B, int64_t ninc, const uint32_t* ib1, const uint32_t* ib2,
-                          const uint32_t* anchor, const uint8_t* finc)
-{
-    const int T = 256;
-    const int64_t C = s->n_contacts;
-    cudaStream_t st = s->stream;
-    k_chunk_starts<<<grid_for((int64_t)kMaxColours * (B + 1), T, 8, s->num_sms), T, 0, st>>>(DCount{C, nullptr}, B, s->col_off,
-                                                                                          s->perm, s->info, s->cstart);
-    int* dmin = (int*)s->deg;
-    int* dmax = (int*)s->adj_off;
-    cudaMemsetAsync(dmin, 0x7F, (size_t)std::max<int64_t>(ninc, 1) * sizeof(int), st);
-    cudaMemsetAsync(dmax, 0x80, (size_t)std::max<int64_t>(ninc, 1) * sizeof(int), st);
-    k_body_blocks<<<grid_for(C, T, 8, s->num_sms), T, 0, st>>>(DCount{C, nullptr}, ninc, B, s->perm, ib1, ib2, anchor, finc, dmin,
-                                                                dmax);
-    k_chunk_windows<<<B, T, 0, st>>>(DCount{C, nullptr}, ninc, s->cstart, s->perm, ib1, ib2, anchor, finc, dmin, dmax, s->info,
-                                      s->dep);
-    cudaMemsetAsync(s->prog, 0xFF, (size_t)B * sizeof(int), st);
-    if (s->timing) s->phase_launches[2] += 3;
-    return cuda_check(s, cudaGetLastError(), "solve: dependency windows");
-}
-
 // --- one launch per colour ------------------------------------------------
 template <class R>
 __global__ void k_gravity(SolveArgs<R> A)

@@ -101,6 +101,32 @@ __device__ __forceinline__ SweepPre<double> ld_pre(const SweepPre<double>* p)
     return x;
 }
 
+// First tile of every colour (tw contacts per tile), and the colour offsets,
+// for the block; every thread takes part.
+__device__ __forceinline__ void tile_offsets(const uint32_t* col_off, int ncol, uint32_t tw, uint32_t* s_off,
+                                             uint32_t* s_tile)
+{
+    for (int c = threadIdx.x; c <= ncol; c += blockDim.x) s_off[c] = col_off[c];
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        uint32_t carry = 0;
+        for (int c0 = 0; c0 < ncol; c0 += 32) {
+            const int c = c0 + lane;
+            uint32_t v = c < ncol ? (s_off[c + 1] - s_off[c] + tw - 1) / tw : 0u;
+            const uint32_t own = v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, v, o);
+                if (lane >= o) v += y;
+            }
+            if (c < ncol) s_tile[c] = carry + v - own;
+            carry += __shfl_sync(kFull, v, 31);
+        }
+        if (lane == 0) s_tile[ncol] = carry;
+    }
+    __syncthreads();
+}
+
 template <class R, int L> struct Unit;
 
 // a b + c d + e f and a b - c d with the operations fused as the compiler

@@ -70,3 +70,34 @@ def test_flow_equals_grid_synchronised_sweeps(shape, precision, tol, omega, fixe
             for k in ("vel", "angvel"):
                 assert np.abs(ba[k] - bb[k]).max() <= bound * np.abs(bb[k]).max()
             assert np.abs(ca["impulse"] - cb["impulse"]).max() <= bound * np.abs(cb["impulse"]).max()
+
+
+@pytest.mark.parametrize("shape,precision,tol", [((2, 2, 2), "fp32", 0.0), ((6, 5, 4), "fp64", 1e-4), ((7, 7, 7), "fp32", 1e-3),
+                                                 ((40, 40, 38), "fp32", 0.0), ((85, 85, 84), "fp32", 0.0),
+                                                 ((25, 25, 24), "fp64", 0.0)])
+def test_composite_flow_equals_grid_synchronised_sweeps(shape, precision, tol):
+    """Lanes per contact by size (8, 4, 1); the slides found by several lanes
+    against the serial search."""
+    from paper_1501_05810_gb300 import nbgs
+    sc = scenes.composite_gas(*shape, seed=1, spacing=0.97, v_max=0.5, dt=5e-3, mu=0.4, omega=0.9,
+                              gravity=(0.0, 0.0, -9.81), precision=precision, warm_start="prev")
+    sc["vel"][:, 2] -= 3.0
+    out = []
+    for flags in (0, GLOBAL_SYNC):
+        s = dict(sc)
+        s["params"] = dict(sc["params"], sweep_flags=flags)
+        g = nbgs.Scene(s)
+        steps = [g.step(10, tol) for _ in range(2)]
+        out.append((steps, g.get_bodies(), g.get_contacts()))
+        g.close()
+    (sa, ba, ca), (sb, bb, cb) = out
+    for x, y in zip(sa, sb):
+        assert x["n_contacts"] == y["n_contacts"] and x["n_colours"] == y["n_colours"]
+    assert np.array_equal(ca["j1"], cb["j1"]) and np.array_equal(ca["j2"], cb["j2"])
+    # a few roundings per relaxation, some 8 x 10 relaxations per body and step, two steps, a gain of at most 10;
+    # where the tolerance may end one sweep earlier, what such a sweep still changes
+    eps = 6e-8 if precision == "fp32" else 1.1e-16
+    bound = eps * 4 * 80 * 2 * 10 + 10 * tol
+    for k in ("vel", "angvel"):
+        assert np.abs(ba[k] - bb[k]).max() <= bound * np.abs(bb[k]).max()
+    assert np.abs(ca["impulse"] - cb["impulse"]).max() <= bound * np.abs(cb["impulse"]).max()
