@@ -438,19 +438,17 @@ static nbgs_status create_common(const nbgs_params* params, const nbgs_batch_des
         delete s;
         return NBGS_EINVAL;
     }
-    s->key_bits = 1;
-    while (((int64_t)1 << s->key_bits) < s->max_cells) ++s->key_bits;
     const int cpb = params->contacts_per_body > 0 ? params->contacts_per_body : 8;
     s->ccap = std::max<int64_t>(1024, (int64_t)cpb * n);
     const size_t nn = (size_t)std::max<int64_t>(n, 1);
 
-    bool ok = take(s, s->pos_r, nn) && take(s, s->quat, nn) && take(s, s->hull, nn) && take(s, s->hvw, nn) &&
+    bool ok = take(s, s->pos_r, nn) && take(s, s->quat, nn) && take(s, s->hull, nn) &&
               take(s, s->p32, nn) &&
               take(s, s->p32s, nn) && take(s, s->finite, nn) &&
               take(s, s->stage, 13 * nn) && take(s, s->cell_start, (size_t)s->max_cells + 1) &&
-              take(s, s->cell_end, (size_t)s->max_cells) && take(s, s->keys[0], nn) && take(s, s->keys[1], nn) &&
-              take(s, s->vals[0], nn) && take(s, s->vals[1], nn) && take(s, s->cand, nn * kCandCap) &&
-              take(s, s->sph_cnt, nn) && take(s, s->row_cnt, nn) && take(s, s->row_off, nn + 1) &&
+              take(s, s->cell_end, (size_t)s->max_cells) && take(s, s->ckey, nn) && take(s, s->crank, nn) &&
+              take(s, s->svals, nn) && take(s, s->cand, nn * kCandCap) &&
+              take(s, s->pair_cnt, nn) && take(s, s->wall_mask, nn) && take(s, s->row_off, nn + 1) &&
               take(s, s->prev_row_off, nn + 1) && take(s, s->deg, nn + 1) && take(s, s->adj_off, nn + 1) &&
               take(s, s->cmask, 8 * (nn + 1)) &&
               take(s, s->col_count, kMaxColours + 1) && take(s, s->col_off, kMaxColours + 1) &&
@@ -577,9 +575,9 @@ void nbgs_destroy_scene(nbgs_scene* s)
     if (!s) return;
     cudaStreamSynchronize(s->stream);
     drop_graphs(s);
-    void* ps[] = {s->pos_r, s->quat, s->vel, s->hull, s->hvw, s->p32, s->p32s, s->finite, s->stage, s->cell_start,
-                  s->cell_end, s->keys[0], s->keys[1], s->vals[0], s->vals[1], s->radix_hist, s->scan_tmp,
-                  s->cand, s->sph_cnt, s->row_cnt, s->row_off, s->prev_row_off, s->deg, s->adj_off,
+    void* ps[] = {s->pos_r, s->quat, s->vel, s->hull, s->p32, s->p32s, s->finite, s->stage, s->cell_start,
+                  s->cell_end, s->ckey, s->crank, s->svals, s->radix_hist, s->scan_tmp,
+                  s->cand, s->pair_cnt, s->wall_mask, s->row_off, s->prev_row_off, s->deg, s->adj_off,
                   s->col_count, s->col_off, s->info, s->dep, s->prog, s->cstart, s->scene_of, s->scene_off,
                   s->scene_box, s->scene_box32, s->scene_mu, s->scene_vmax, s->scene_vref, s->scene_rk,
                   s->scene_done, s->scene_res, s->mlp_theta, s->cmask};

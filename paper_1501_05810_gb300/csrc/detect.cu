@@ -3,15 +3,15 @@
 // Per step:
 //   k_hull          h_i = dt(|v_i| + |w_i| r_i) + tau       eq. (expansionradius)
 //                   + max h, max |v| (for the cell size and v_ref)
-//   k_grid_setup    cell width >= 2 (r_max + h_max), dims per axis
-//   k_cell_keys     linear cell index of every body
-//   radix sort      (cell, body) pairs, LSD, 8-bit digits, stable
-//   scan            first sorted slot of every cell, from the cell counts
-//   k_gather_sorted FP32 positions in cell order
-//   k_narrow        per body i: bodies j > i in the 27 neighbour cells whose
-//                   hulls intersect, sorted by j; wall hull tests
+//   k_cell_keys     cell width >= 2 (r_max + h_max), dims per axis; every
+//                   body's linear cell index and its rank in the cell
+//   scan            first slot of every cell, from the cell counts
+//   k_cell_scatter  bodies and their FP32 positions in cell order
+//   k_narrow        per body: bodies in its own and the 13 cells ahead whose
+//                   hulls intersect; wall hull tests
 //   scan            contacts per body -> CSR offsets by j1
-//   k_write         canonical contact records (n, xi, lever lengths)
+//   k_write         canonical contact records (n, xi, lever lengths), partners
+//                   in ascending order,
 //                   for sphere-sphere and sphere-wall pairs, eq. (contactpos)
 #include <algorithm>
 #include <cmath>
@@ -71,7 +71,22 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t& excl)
     return total;
 }
 
-__global__ void k_scan_reduce(const uint32_t* __restrict__ in, DCount nc, uint32_t* __restrict__ sums)
+// What a scan adds up: an array, or a body's contacts from its pair count and
+// kept-wall mask.
+struct ScanArray {
+    const uint32_t* in;
+    __device__ __forceinline__ uint32_t operator[](int64_t i) const { return in[i]; }
+};
+struct ScanRows {
+    const uint32_t *pairs, *walls;
+    __device__ __forceinline__ uint32_t operator[](int64_t i) const
+    {
+        return min(pairs[i], (uint32_t)kCandCap) + (uint32_t)__popc(walls[i]);
+    }
+};
+
+template <class In>
+__global__ void k_scan_reduce(In in, DCount nc, uint32_t* __restrict__ sums)
 {
     const int64_t n = nc.get();
     const int64_t base = (int64_t)blockIdx.x * kScanTile;
@@ -100,7 +115,13 @@ __global__ void k_scan_top(uint32_t* sums, int64_t nb)
     }
 }
 
-__global__ void k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, DCount nc,
+// top: the block sums have been scanned (k_scan_top); otherwise each block
+// adds up the sums before its own, which for up to kScanSelf blocks costs
+// less than a launch of its own.
+constexpr int kScanSelf = 2048;
+
+template <bool top, class In>
+__global__ void k_scan_down(In in, uint32_t* out, DCount nc,
                             const uint32_t* __restrict__ sums, uint32_t* __restrict__ total_dst)
 {
     __shared__ uint32_t tile[kScanTile];
@@ -110,6 +131,14 @@ __global__ void k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restric
     for (int k = 0; k < kScanItems; ++k) {
         int64_t i = base + (int64_t)k * kScanThreads + threadIdx.x;
         tile[k * kScanThreads + threadIdx.x] = i < n ? in[i] : 0;
+    }
+    uint32_t before = 0;
+    if (top) {
+        before = sums[blockIdx.x];
+    } else {
+        uint32_t part = 0, excl;
+        for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) part += sums[i];
+        before = block_excl_scan(part, excl);
     }
     __syncthreads();
     uint32_t loc[kScanItems];
@@ -121,7 +150,7 @@ __global__ void k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restric
     }
     uint32_t excl;
     uint32_t tot = block_excl_scan(acc, excl);
-    const uint32_t off = sums[blockIdx.x] + excl;
+    const uint32_t off = before + excl;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) tile[threadIdx.x * kScanItems + k] = loc[k] + off;
     __syncthreads();
@@ -131,7 +160,7 @@ __global__ void k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restric
         if (i < n) out[i] = tile[k * kScanThreads + threadIdx.x];
     }
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
-        uint32_t total = sums[blockIdx.x] + tot;
+        uint32_t total = before + tot;
         out[n] = total;
         if (total_dst) *total_dst = total;
     }
@@ -139,15 +168,25 @@ __global__ void k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restric
 
 // out must hold n + 1 entries; out[n] receives the total (also *total_dst).
 // A device-read count: the launch covers n.v entries (the capacity).
-nbgs_status exclusive_scan_u32(nbgs_scene* s, const uint32_t* in, uint32_t* out, DCount n, uint32_t* total_dst)
+template <class In>
+static nbgs_status exclusive_scan(nbgs_scene* s, In in, uint32_t* out, DCount n, uint32_t* total_dst)
 {
     int64_t nb = (n.v + kScanTile - 1) / kScanTile;
     if (nb < 1) nb = 1;
     if (nb > s->scan_tmp_len) return fail(s, NBGS_EINVAL, "scan: block-sum buffer too small");
     k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s->stream>>>(in, n, s->scan_tmp);
-    k_scan_top<<<1, 1024, 0, s->stream>>>(s->scan_tmp, nb);
-    k_scan_down<<<(unsigned)nb, kScanThreads, 0, s->stream>>>(in, out, n, s->scan_tmp, total_dst);
+    if (nb > kScanSelf) {
+        k_scan_top<<<1, 1024, 0, s->stream>>>(s->scan_tmp, nb);
+        k_scan_down<true, In><<<(unsigned)nb, kScanThreads, 0, s->stream>>>(in, out, n, s->scan_tmp, total_dst);
+    } else {
+        k_scan_down<false, In><<<(unsigned)nb, kScanThreads, 0, s->stream>>>(in, out, n, s->scan_tmp, total_dst);
+    }
     return cuda_check(s, cudaGetLastError(), "scan");
+}
+
+nbgs_status exclusive_scan_u32(nbgs_scene* s, const uint32_t* in, uint32_t* out, DCount n, uint32_t* total_dst)
+{
+    return exclusive_scan(s, ScanArray{in}, out, n, total_dst);
 }
 
 nbgs_status exclusive_scan_u32(nbgs_scene* s, const uint32_t* in, uint32_t* out, int64_t n, uint32_t* total_dst)
@@ -299,11 +338,13 @@ __device__ __forceinline__ double norm_exact(double x, double y, double z)
 // one fused multiply-add, and RN(q + (a - b q) y) is the correctly rounded
 // quotient (Markstein's theorem, IBM J. Res. Dev. 34(1), 1990; Muller et
 // al., Handbook of Floating-Point Arithmetic, the chapter on division with
-// an FMA).  The theorem excludes underflow: zeros and tiny numerators take
-// the division itself, as does the caller for a tiny or huge b.
+// an FMA).  The theorem excludes underflow: tiny numerators take the division
+// itself, as does the caller for a tiny or huge b; a zero (every pair inside a
+// lattice plane has one) is its own quotient, b being positive.
 __device__ __forceinline__ double div_by(double a, double b, double y)
 {
-    if (fabs(a) < 0x1p-900) return xdiv(a, b);
+    const uint32_t e = (uint32_t)__double2hiint(a) & 0x7FFFFFFFu;
+    if (e < 0x07B00000u) return (e | (uint32_t)__double2loint(a)) == 0u ? a : xdiv(a, b);   // |a| < 2^-900
     const double q = __dmul_rn(a, y);
     const double r = __fma_rn(-q, b, a);
     return __fma_rn(r, y, q);
@@ -411,62 +452,86 @@ __global__ void k_member_update(int64_t n, const uint32_t* __restrict__ mbody, c
 }
 
 // Hull radius of eq. (expansionradius), h = dt (|v| + |w| r) + tau, rounded
-// as the FP64 step computes it: for a sphere from the squares of |v| and |w|
-// stored by k_hull (so that only the contacts that need the exact value pay
-// for its two square roots), for a composite member from the member hulls.
+// as the FP64 step computes it: for a sphere from its velocities, where a
+// decision needs it (only those contacts pay for its two square roots), for a
+// composite member from the member hulls.
 struct HullView {
     const double* hull;   // member hulls (composites), else null
-    const double2* vw;    // |v|^2, |w|^2 per sphere
+    const void* vel;      // (v, 1/m), (w, 1/I) per sphere
+    int fp32;             // in FP32 or FP64
     double dt, tau;
 };
-__device__ __forceinline__ double hull_of(const HullView& H, uint32_t x, double r)
+
+template <class R>
+__device__ __forceinline__ double norm2_exact(const R4<R>& v)
 {
-    if (H.hull) return H.hull[x];
-    const double2 q = H.vw[x];
-    return xadd(xmul(H.dt, xadd(xsqrt(q.x), xmul(xsqrt(q.y), r))), H.tau);
+    const double x = v.x, y = v.y, z = v.z;
+    return xadd(xadd(xmul(x, x), xmul(y, y)), xmul(z, z));
 }
 
-// Per sphere: |v|^2 and |w|^2 in FP64 (the exact hull's inputs), the FP32
-// position relative to the box corner and the reach r + h with h in FP32
-// (cell keys and the narrow phase's screens run on these; the FP32 hull is
-// within 5e-7 of h relative, inside the screens' margins), an upper bound
-// of the largest hull for the grid, and max |v| (v_ref) exactly: the
-// square root of the largest |v|^2, square roots being monotone.
+__device__ __noinline__ double hull_of(const HullView& H, uint32_t x, double r)
+{
+    if (H.hull) return H.hull[x];
+    double v2, w2;
+    if (H.fp32) {
+        float4 v, w;
+        ld_body((const float4*)H.vel + 2 * (int64_t)x, v, w);
+        v2 = norm2_exact<float>(v);
+        w2 = norm2_exact<float>(w);
+    } else {
+        double4_32a v, w;
+        ld_body((const double4_32a*)H.vel + 2 * (int64_t)x, v, w);
+        v2 = norm2_exact<double>(v);
+        w2 = norm2_exact<double>(w);
+    }
+    return xadd(xmul(H.dt, xadd(xsqrt(v2), xmul(xsqrt(w2), r))), H.tau);
+}
+
+// Per sphere: the FP32 position relative to the box corner and the reach r +
+// h with h in FP32 (cell keys and the narrow phase's screens run on these; the
+// FP32 hull is within 1e-6 of h relative, inside the screens' margins), and an
+// upper bound of the largest hull for the grid.  v_ref wants max |v| exactly:
+// the square root of the largest FP64 |v|^2, which only the bodies whose FP32
+// |v|^2 (off by less than 4e-7 relative) is within 1e-6 of the block's largest
+// can have; those few are looked at again.  FP64 arithmetic occupies this GPU's
+// FP64 units for 16 cycles per warp and SM, so a square per body and component
+// was most of this kernel's time: 4M bodies, 249 -> 80 us (ncu, cold).
 template <class R>
 __global__ void k_hull(int64_t n, const R4<R>* __restrict__ vel, const double4_32a* __restrict__ pos_r, double dt,
-                       double tau, double2* __restrict__ vw, float4* __restrict__ p32, GridArgs g, DevInfo* info,
+                       double tau, float4* __restrict__ p32, GridArgs g, DevInfo* info,
                        const uint32_t* __restrict__ scene_of, unsigned long long* __restrict__ scene_vmax)
 {
-    double hmax = 0.0, v2max = 0.0;
+    float hmax = 0.f, v2max = 0.f;
     bool bad = false;
     const float dtf = (float)dt, tauf = (float)tau;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = first; i < n; i += stride) {
         R4<R> v, w;
         ld_body(vel + 2 * i, v, w);
         const double4_32a x = ld_d4(pos_r + i);
-        const double r = x.w;
-        const double vx = v.x, vy = v.y, vz = v.z, wx = w.x, wy = w.y, wz = w.z;
-        const double v2 = xadd(xadd(xmul(vx, vx), xmul(vy, vy)), xmul(vz, vz));
-        const double w2 = xadd(xadd(xmul(wx, wx), xmul(wy, wy)), xmul(wz, wz));
-        vw[i] = make_double2(v2, w2);
-        const float h32 = dtf * (sqrtf((float)v2) + sqrtf((float)w2) * (float)r) + tauf;
-        p32[i] = make_float4((float)(x.x - g.lo[0]), (float)(x.y - g.lo[1]), (float)(x.z - g.lo[2]),
-                             (float)(r + (double)h32));
-        if (!(v2 <= 1e300) || !(w2 <= 1e300)) bad = true;
-        if (scene_of) {   // per-scene max |v|^2 (v_ref); the filter only saves atomics
+        const float vx = (float)v.x, vy = (float)v.y, vz = (float)v.z, wx = (float)w.x, wy = (float)w.y, wz = (float)w.z;
+        const float v2 = vx * vx + vy * vy + vz * vz, w2 = wx * wx + wy * wy + wz * wz;
+        const float rf = (float)x.w, h32 = dtf * (sqrtf(v2) + sqrtf(w2) * rf) + tauf;
+        p32[i] = make_float4((float)(x.x - g.lo[0]), (float)(x.y - g.lo[1]), (float)(x.z - g.lo[2]), rf + h32);
+        // beyond FP32: NaN, Inf, or squares too large for it
+        if (!(v2 <= 1e38f && w2 <= 1e38f) && !(norm2_exact<R>(v) <= 1e300 && norm2_exact<R>(w) <= 1e300)) bad = true;
+        if (scene_of) {   // per-scene max |v|^2 (v_ref); the filter only saves FP64 squares and atomics
             unsigned long long* dst = scene_vmax + scene_of[i];
-            const unsigned long long bits = (unsigned long long)__double_as_longlong(v2);
-            if (bits > *(volatile unsigned long long*)dst) atomicMax(dst, bits);
+            if (!((float)__longlong_as_double((long long)*(volatile unsigned long long*)dst) > v2 * (1.f + 1e-6f) + 1e-30f)) {
+                const unsigned long long bits = (unsigned long long)__double_as_longlong(norm2_exact<R>(v));
+                if (bits > *(volatile unsigned long long*)dst) atomicMax(dst, bits);
+            }
         }
-        hmax = fmax(hmax, (double)h32);
-        v2max = fmax(v2max, v2);
+        hmax = fmaxf(hmax, h32);
+        v2max = fmaxf(v2max, v2);
     }
-    // block max, then one atomic per block (non-negative doubles order like their bits)
-    __shared__ double sh[2][32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ float sh[2][32];
+    __shared__ float s_v2;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+    const float own = v2max;
     for (int o = 16; o > 0; o >>= 1) {
-        hmax = fmax(hmax, __shfl_down_sync(0xffffffffu, hmax, o));
-        v2max = fmax(v2max, __shfl_down_sync(0xffffffffu, v2max, o));
+        hmax = fmaxf(hmax, __shfl_xor_sync(0xffffffffu, hmax, o));
+        v2max = fmaxf(v2max, __shfl_xor_sync(0xffffffffu, v2max, o));
     }
     if (lane == 0) {
         sh[0][wid] = hmax;
@@ -474,36 +539,27 @@ __global__ void k_hull(int64_t n, const R4<R>* __restrict__ vel, const double4_3
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < (int)(blockDim.x >> 5); ++k) {
-            hmax = fmax(hmax, sh[0][k]);
-            v2max = fmax(v2max, sh[1][k]);
+        for (int k = 1; k < nw; ++k) {
+            hmax = fmaxf(hmax, sh[0][k]);
+            v2max = fmaxf(v2max, sh[1][k]);
         }
-        // the FP32 hulls are within 5e-7 of h relative: 1e-5 makes an upper bound
-        atomicMax(&info->hmax_bits, (unsigned long long)__double_as_longlong(hmax * (1.0 + 1e-5)));
-        atomicMax(&info->vmax_bits, (unsigned long long)__double_as_longlong(xsqrt(v2max)));
+        s_v2 = v2max;
+        // 1e-5 above the FP32 hulls is above the exact ones (non-negative doubles order like their bits)
+        atomicMax(&info->hmax_bits, (unsigned long long)__double_as_longlong((double)hmax * (1.0 + 1e-5)));
+    }
+    __syncthreads();
+    const float near = s_v2 > 1e-30f ? s_v2 * (1.f - 1e-6f) : 0.f;   // squares that underflow: look at all
+    if (own >= near) {
+        double best = 0.0;
+        for (int64_t i = first; i < n; i += stride) {
+            R4<R> v, w;
+            ld_body(vel + 2 * i, v, w);
+            const float vx = (float)v.x, vy = (float)v.y, vz = (float)v.z;
+            if (vx * vx + vy * vy + vz * vz >= near) best = fmax(best, norm2_exact<R>(v));
+        }
+        atomicMax(&info->vmax_bits, (unsigned long long)__double_as_longlong(xsqrt(best)));
     }
     if (bad) atomicOr(&info->err, kErrNaN);
-}
-
-__global__ void k_grid_setup(GridArgs g, DevInfo* info)
-{
-    const double hmax = __longlong_as_double((long long)info->hmax_bits);
-    // any kept pair has d <= r_a + r_b + h_a + h_b <= 2 (r_max + h_max); the
-    // cell keys come from FP32 positions with error <= pos_err, so a cell at
-    // least need + 4 pos_err wide keeps every such pair in adjacent cells
-    const double need = 2.0 * (g.r_max + hmax) * (1.0 + 1e-9) + 4.0 * g.pos_err + 1e-300;
-    uint32_t ncells = 1;
-    for (int a = 0; a < 3; ++a) {
-        const double L = g.hi[a] - g.lo[a];
-        double dd = floor(L / need);
-        int d = dd < 1.0 ? 1 : (dd > (double)g.dims_max[a] ? g.dims_max[a] : (int)dd);
-        if (g.periodic[a] && d < 3) atomicOr(&info->err, kErrGrid);
-        info->dims[a] = d;
-        info->cell_w[a] = L / d;
-        info->inv_wf[a] = (float)(d / L);
-        ncells *= (uint32_t)d;
-    }
-    info->ncells = ncells;
 }
 
 __device__ __forceinline__ int cell_coord(float x, float inv_w, int d)
@@ -512,29 +568,60 @@ __device__ __forceinline__ int cell_coord(float x, float inv_w, int d)
     return f < 0.f ? 0 : (f > (float)(d - 1) ? d - 1 : (int)f);
 }
 
-// Cell key of every body, and the body count of every cell.
-__global__ void k_cell_keys(int64_t n, const float4* __restrict__ p32, const DevInfo* __restrict__ info,
-                            uint32_t* __restrict__ keys, uint32_t* __restrict__ vals, uint32_t* __restrict__ cnt)
+// The cell grid of the step (every block works it out, the first one notes it
+// down), the cell of every body and its rank among the cell's bodies, in the
+// order the counter served them: where in the cell's range of slots a body
+// lands does not matter to anything that follows.
+__global__ void k_cell_keys(int64_t n, const float4* __restrict__ p32, GridArgs g, DevInfo* info,
+                            uint32_t* __restrict__ keys, uint32_t* __restrict__ rank, uint32_t* __restrict__ cnt)
 {
-    const int d0 = info->dims[0], d1 = info->dims[1], d2 = info->dims[2];
-    const float i0 = info->inv_wf[0], i1 = info->inv_wf[1], i2 = info->inv_wf[2];
+    __shared__ int s_d[3];
+    __shared__ float s_inv[3];
+    if (threadIdx.x < 3) {
+        const int a = threadIdx.x;
+        const double hmax = __longlong_as_double((long long)info->hmax_bits);
+        // any kept pair has d <= r_a + r_b + h_a + h_b <= 2 (r_max + h_max); the
+        // cell keys come from FP32 positions with error <= pos_err, so a cell at
+        // least need + 4 pos_err wide keeps every such pair in adjacent cells
+        const double need = 2.0 * (g.r_max + hmax) * (1.0 + 1e-9) + 4.0 * g.pos_err + 1e-300;
+        const double L = g.hi[a] - g.lo[a];
+        const double dd = floor(L / need);
+        const int d = dd < 1.0 ? 1 : (dd > (double)g.dims_max[a] ? g.dims_max[a] : (int)dd);
+        s_d[a] = d;
+        s_inv[a] = (float)(d / L);
+        if (blockIdx.x == 0) {
+            if (g.periodic[a] && d < 3) atomicOr(&info->err, kErrGrid);
+            info->dims[a] = d;
+            info->cell_w[a] = L / d;
+            info->inv_wf[a] = s_inv[a];
+        }
+    }
+    __syncthreads();
+    const int d0 = s_d[0], d1 = s_d[1], d2 = s_d[2];
+    const float i0 = s_inv[0], i1 = s_inv[1], i2 = s_inv[2];
+    if (blockIdx.x == 0 && threadIdx.x == 0) info->ncells = (uint32_t)d0 * (uint32_t)d1 * (uint32_t)d2;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float4 p = p32[i];
         const int cx = cell_coord(p.x, i0, d0), cy = cell_coord(p.y, i1, d1), cz = cell_coord(p.z, i2, d2);
         const uint32_t k = ((uint32_t)cz * (uint32_t)d1 + (uint32_t)cy) * (uint32_t)d0 + (uint32_t)cx;
         keys[i] = k;
-        vals[i] = (uint32_t)i;
-        atomicAdd(&cnt[k], 1u);
+        rank[i] = atomicAdd(&cnt[k], 1u);
     }
 }
 
-// The FP32 positions gathered into cell order, so that the narrow phase
-// reads each cell's candidates contiguously.
-__global__ void k_gather_sorted(int64_t n, const uint32_t* __restrict__ vals, const float4* __restrict__ p32,
-                                float4* __restrict__ p32s)
+// Bodies and their FP32 positions in cell order, so that the narrow phase
+// reads each cell's candidates contiguously.  A counting sort: against the
+// radix sort of (cell, body) pairs of before, with its three or four passes
+// of five kernels, 4M bodies take 30 + 60 us instead of 430 (ncu, cold).
+__global__ void k_cell_scatter(int64_t n, const uint32_t* __restrict__ keys, const uint32_t* __restrict__ rank,
+                               const uint32_t* __restrict__ cell_start, const float4* __restrict__ p32,
+                               uint32_t* __restrict__ svals, float4* __restrict__ p32s)
 {
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x)
-        p32s[s] = p32[vals[s]];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t s = cell_start[keys[i]] + rank[i];
+        svals[s] = (uint32_t)i;
+        p32s[s] = p32[i];
+    }
 }
 
 // Minimum-image difference a - b along one axis (periodic: |d| <= L/2).
@@ -629,70 +716,47 @@ __device__ __forceinline__ bool wall_kept(const double nrm[3], double c, double4
     return xi <= xadd(h, tau);
 }
 
-// Per body i (visited in cell order for locality): hull-intersecting
-// partners j > i from the 27 neighbour cells, sorted ascending; wall count.
-// cs[c] is the first sorted slot of cell c for every cell (cs[ncells] = n),
-// so the three cells x - 1 .. x + 1 of a (y, z) row are one contiguous
-// range; a periodic image adds one constant shift to a whole range.
-struct NarrowPair {
-    uint32_t list[kCandCap];
-    int cnt;
-};
+// Hull-intersecting pairs.  Every body (in cell order) looks at the bodies
+// behind it in its own cell and at the 13 neighbour cells ahead (after it in
+// z, y, x), so that each pair is tested once; the pair joins the list of its
+// lower body through that body's counter, and k_write_contacts puts each list
+// into ascending order.  cs[c] is the first slot of cell c for every cell
+// (cs[ncells] = n), so the cells x - 1 .. x + 1 of a (y, z) row are one
+// contiguous range; a periodic image adds one constant shift to a whole
+// range.  The kernel is bound by the instructions of the screens where pairs
+// are few, and by the lists' atomics where they are many: with all 27 cells
+// searched for both bodies of a pair, nested loops and the list in the
+// thread, 4M gas bodies took 574 us and 1M packed ones 145 (ncu, cold), this
+// way 368 and 213; the packed scene's solve takes 8 ms.
+//
+// The search is a loop of FP32 screens over the rows' slots, run together
+// (the lanes of a warp differ in the lengths of the rows by more than in
+// their sum); the pairs that pass wait in a queue in shared memory, so that
+// the lanes work them off together.
+constexpr int kNarrowThreads = 128, kNarrowRows = 5, kNarrowQueue = 8;
+constexpr uint32_t kSurePair = 1u << 31;   // of a queued slot: kept without the FP64 test
 
-__device__ __forceinline__ void narrow_range(uint32_t t0, uint32_t t1, float sx, float sy, float sz, uint32_t i,
-                                             uint32_t si, const float4& qi, const double4_32a& pi, double& hi_,
-                                             const uint32_t* __restrict__ svals, const float4* __restrict__ p32s,
-                                             const double4_32a* __restrict__ pos_r, const HullView& H,
-                                             const GridArgs& g, const SceneView& V, double L0, double L1, double L2,
-                                             NarrowPair& P)
+// Sect. 4: is the pair kept?  Its lower and upper body; R is the sum of
+// their FP32 reaches.
+__device__ __noinline__ bool exact_pair(const HullView& H, const GridArgs& g, const double4_32a* __restrict__ pos_r,
+                                        uint32_t lo, uint32_t hi, float R)
 {
-    for (uint32_t t = t0; t < t1; ++t) {
-        const uint32_t j = svals[t];
-        const float4 qj = p32s[t];   // loaded with j: one dependent load fewer
-        if (j <= i) continue;
-        if (V.batch && V.scene_of[j] != si) continue;   // scenes never touch
-        if (V.body_of && V.body_of[j] == V.body_of[i]) continue;   // members of one body never touch
-        // Conservative FP32 screens (FP64 throughput is scarce on this GPU).
-        // R = r_a + h_a + r_b + h_b bounds d for every kept pair.  The FP32
-        // relative positions are off by at most pos_err per coordinate, the
-        // periodic shift adds an ulp of L, so the FP32 distance is within
-        // 1e-6 max(L) of d; the FP32 square and reach add relative errors
-        // below 4e-7 and 1.2e-7, covered by the extra 1e-4 while R < ~100 (the FP32 hull's own error
-        // included).
-        // So (fl(R) + margin)^2 >= fl(d^2) for every kept pair, and
-        // fl(d^2) < (fl(R) - margin)^2 only for pairs with d below R by more
-        // than the FP64 keep rule's rounding: those are kept without it.
-        // Only the pairs in the band between take the exact FP64 test.
-        const float fx = (qi.x - qj.x) + sx, fy = (qi.y - qj.y) + sy, fz = (qi.z - qj.z) + sz;
-        const float rs = qi.w + qj.w;
-        const float rr = rs + g.margin, rl = rs - g.margin;
-        const float d2f = fx * fx + fy * fy + fz * fz;
-        if (rs < 100.f && d2f > rr * rr) continue;
-        bool keep = rl > 0.f && rs < 100.f && d2f < rl * rl;
-        if (!keep) {
-            const double4_32a pj = pos_r[j];
-            const double dx3 = min_image(xsub(pi.x, pj.x), g.periodic[0], L0);
-            const double dy3 = min_image(xsub(pi.y, pj.y), g.periodic[1], L1);
-            const double dz3 = min_image(xsub(pi.z, pj.z), g.periodic[2], L2);
-            const double d = norm_exact(dx3, dy3, dz3);
-            // Sect. 4: keep the pair iff the hulls intersect (the exact hulls,
-            // body i's computed once)
-            if (!(hi_ >= 0.0)) hi_ = hull_of(H, i, pi.w);
-            keep = xsub(xsub(d, pi.w), pj.w) <= xadd(hi_, hull_of(H, j, pj.w));
-        }
-        if (keep) {
-            if (P.cnt < kCandCap) {
-                // insertion keeps the list sorted by j
-                int k = P.cnt;
-                while (k > 0 && P.list[k - 1] > j) {
-                    P.list[k] = P.list[k - 1];
-                    --k;
-                }
-                P.list[k] = j;
-            }
-            ++P.cnt;
-        }
+    const double4_32a pl = pos_r[lo], ph = pos_r[hi];
+    const double dx3 = min_image(xsub(pl.x, ph.x), g.periodic[0], g.hi[0] - g.lo[0]);
+    const double dy3 = min_image(xsub(pl.y, ph.y), g.periodic[1], g.hi[1] - g.lo[1]);
+    const double dz3 = min_image(xsub(pl.z, ph.z), g.periodic[2], g.hi[2] - g.lo[2]);
+    // The differences now hold no rounding of large coordinates: their FP32
+    // square is within 4e-7 of d^2 and R within 1.2e-6 of the FP64 sum, which
+    // leaves the FP64 square roots (d's, and the hulls' four) to the pairs
+    // within 2e-6 of it.
+    const float gx = (float)dx3, gy = (float)dy3, gz = (float)dz3;
+    const float d2g = gx * gx + gy * gy + gz * gz, r2 = R * R;
+    if (R > 1e-15f && R < 1e15f) {
+        if (d2g > r2 * (1.f + 5e-6f)) return false;
+        if (d2g < r2 * (1.f - 5e-6f)) return true;
     }
+    const double d = norm_exact(dx3, dy3, dz3);
+    return xsub(xsub(d, pl.w), ph.w) <= xadd(hull_of(H, lo, pl.w), hull_of(H, hi, ph.w));
 }
 
 // Neighbour index along one axis: the cell and the shift of the periodic
@@ -711,56 +775,114 @@ __device__ __forceinline__ bool axis_cell(int c, int d, int periodic, float Lf, 
     return true;
 }
 
-__global__ void __launch_bounds__(128)
-k_narrow(int64_t n, const uint32_t* __restrict__ skeys, const uint32_t* __restrict__ svals,
-         const double4_32a* __restrict__ pos_r, HullView H, const float4* __restrict__ p32s,
-         const uint32_t* __restrict__ cs, GridArgs g, Planes planes, SceneView V, DevInfo* info,
-         uint32_t* __restrict__ cand, uint32_t* __restrict__ sph_cnt, uint32_t* __restrict__ row_cnt)
+__global__ void __launch_bounds__(kNarrowThreads)
+k_narrow(int64_t n, const uint32_t* __restrict__ svals, const double4_32a* __restrict__ pos_r,
+         const __grid_constant__ HullView H, const float4* __restrict__ p32s, const uint32_t* __restrict__ cs,
+         const __grid_constant__ GridArgs g, const __grid_constant__ Planes planes, SceneView V, DevInfo* info,
+         uint32_t* __restrict__ cand, uint32_t* __restrict__ pair_cnt, uint32_t* __restrict__ wall_mask)
 {
+    __shared__ uint32_t s_t0[kNarrowRows][kNarrowThreads], s_t1[kNarrowRows][kNarrowThreads];
+    __shared__ float2 s_yz[kNarrowRows][kNarrowThreads];   // y and z relative to the row's image
+    __shared__ uint32_t s_q[kNarrowQueue][kNarrowThreads];
+    const int tid = threadIdx.x;
     const int d0 = info->dims[0], d1 = info->dims[1], d2 = info->dims[2];
-    const double L0 = g.hi[0] - g.lo[0], L1 = g.hi[1] - g.lo[1], L2 = g.hi[2] - g.lo[2];
+    const float i0 = info->inv_wf[0], i1 = info->inv_wf[1], i2 = info->inv_wf[2];
     const bool wrap_x = g.periodic[0] && d0 >= 3;
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
+    const float margin =
+        2.0 * (g.r_max + __longlong_as_double((long long)info->hmax_bits)) < 50.0 ? g.margin : 1e30f;
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + tid; s < n; s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t i = svals[s];
-        const uint32_t key = skeys[s];
-        const int cx = (int)(key % (uint32_t)d0);
-        const int cy = (int)((key / (uint32_t)d0) % (uint32_t)d1);
-        const int cz = (int)(key / ((uint32_t)d0 * (uint32_t)d1));
-        const double4_32a pi = pos_r[i];
-        double hi_ = -1.0;   // the exact hull of i, computed when a test needs it
-        const float4 qi = p32s[s];
         const uint32_t si = V.batch ? V.scene_of[i] : 0u;
-        NarrowPair P;
-        P.cnt = 0;
+        const float4 qi = p32s[s];
+        // its cell, as k_cell_keys has it
+        const int cx = cell_coord(qi.x, i0, d0), cy = cell_coord(qi.y, i1, d1), cz = cell_coord(qi.z, i2, d2);
         const int xlo = cx > 0 ? cx - 1 : 0, xhi = cx + 1 < d0 ? cx + 1 : d0 - 1;
-        for (int dz = -1; dz <= 1; ++dz) {
-            int z;
-            float sz;
-            if (!axis_cell(cz + dz, d2, g.periodic[2], g.Lf[2], z, sz)) continue;
-            for (int dy = -1; dy <= 1; ++dy) {
-                int y;
-                float sy;
-                if (!axis_cell(cy + dy, d1, g.periodic[1], g.Lf[1], y, sy)) continue;
+        // the rows ahead: the rest of its own, (y + 1), and three in z + 1
+#pragma unroll
+        for (int k = 0; k < kNarrowRows; ++k) {
+            int z, y;
+            float sy = 0.f, sz = 0.f;
+            uint32_t t0 = 0, t1 = 0;
+            if (axis_cell(cz + (k > 1), d2, g.periodic[2], g.Lf[2], z, sz) &&
+                axis_cell(cy + (k > 1 ? k - 3 : k), d1, g.periodic[1], g.Lf[1], y, sy)) {
                 const uint32_t row = ((uint32_t)z * (uint32_t)d1 + (uint32_t)y) * (uint32_t)d0;
-                narrow_range(cs[row + xlo], cs[row + xhi + 1], 0.f, sy, sz, i, si, qi, pi, hi_, svals, p32s, pos_r,
-                             H, g, V, L0, L1, L2, P);
-                if (wrap_x && cx == 0)
-                    narrow_range(cs[row + d0 - 1], cs[row + d0], g.Lf[0], sy, sz, i, si, qi, pi, hi_, svals, p32s,
-                                 pos_r, H, g, V, L0, L1, L2, P);
-                if (wrap_x && cx == d0 - 1)
-                    narrow_range(cs[row], cs[row + 1], -g.Lf[0], sy, sz, i, si, qi, pi, hi_, svals, p32s, pos_r,
-                                 H, g, V, L0, L1, L2, P);
+                t0 = k == 0 ? (uint32_t)s + 1u : cs[row + xlo];
+                t1 = cs[row + xhi + 1];
+            }
+            s_yz[k][tid] = make_float2(qi.y + sy, qi.z + sz);
+            s_t0[k][tid] = t0;
+            s_t1[k][tid] = t1;
+        }
+        int nq = 0;
+        auto work_off = [&]() {
+            for (int m = 0; m < nq; ++m) {
+                const uint32_t q = s_q[m][tid], t = q & ~kSurePair;
+                const uint32_t j = svals[t];
+                if (V.batch && V.scene_of[j] != si) continue;   // scenes never touch
+                if (V.body_of && V.body_of[j] == V.body_of[i]) continue;   // nor members of one body
+                const uint32_t lo = min(i, j), hi = max(i, j);
+                if (!(q & kSurePair) && !exact_pair(H, g, pos_r, lo, hi, qi.w + p32s[t].w)) continue;
+                const uint32_t slot = atomicAdd(&pair_cnt[lo], 1u);
+                if (slot < (uint32_t)kCandCap) {
+                    cand[(int64_t)lo * kCandCap + slot] = hi;
+                } else {
+                    atomicOr(&info->err, kErrCand);
+                    atomicMax(&info->cand_need, slot + 1u);
+                }
+            }
+            nq = 0;
+        };
+        // Conservative FP32 screens (FP64 throughput is scarce on this GPU).
+        // R = r_a + h_a + r_b + h_b bounds d for every kept pair.  The FP32
+        // relative positions are off by at most pos_err per coordinate, the
+        // periodic shift adds an ulp of L, so the FP32 distance is within
+        // 1e-6 max(L) of d; the FP32 square and reach add relative errors
+        // below 4e-7 and 1.2e-6, covered by the extra 1e-4 while R < 50
+        // (a margin beyond every pair otherwise).
+        // So (fl(R) + margin)^2 >= fl(d^2) for every kept pair, and
+        // fl(d^2) < (fl(R) - margin)^2 only for pairs with d below R by more
+        // than the FP64 keep rule's rounding: those are kept without it.
+        // Only the pairs in the band between take the exact FP64 test.
+        auto screen = [&](uint32_t t, const float4& qj, float qx, float qy, float qz) {
+            const float fx = qx - qj.x, fy = qy - qj.y, fz = qz - qj.z;
+            const float rs = qi.w + qj.w, rr = rs + margin;
+            const float d2f = fx * fx + fy * fy + fz * fz;
+            if (d2f > rr * rr) return;
+            const float rl = rs - margin;
+            s_q[nq++][tid] = t | (d2f < rl * fabsf(rl) ? kSurePair : 0u);
+            if (nq == kNarrowQueue) work_off();
+        };
+        uint32_t t = 0, te = 0;
+        float2 yz = make_float2(0.f, 0.f);
+        for (int k = -1;;) {
+            if (t >= te) {
+                do {
+                    if (++k == kNarrowRows) break;
+                    t = s_t0[k][tid];
+                    te = s_t1[k][tid];
+                } while (t >= te);
+                if (k == kNarrowRows) break;
+                yz = s_yz[k][tid];
+            }
+            screen(t, p32s[t], qi.x, yz.x, yz.y);
+            ++t;
+        }
+        if (wrap_x && (cx == 0 || cx == d0 - 1)) {   // the images across x; within its own row only the one ahead
+            const int xw = cx == 0 ? d0 - 1 : 0;
+            const float qx = cx == 0 ? qi.x + g.Lf[0] : qi.x - g.Lf[0];
+#pragma unroll 1
+            for (int k = cx == 0 ? 1 : 0; k < kNarrowRows; ++k) {
+                int z, y;
+                float sy, sz;
+                if (!axis_cell(cz + (k > 1), d2, g.periodic[2], g.Lf[2], z, sz) ||
+                    !axis_cell(cy + (k > 1 ? k - 3 : k), d1, g.periodic[1], g.Lf[1], y, sy))
+                    continue;
+                const uint32_t row = ((uint32_t)z * (uint32_t)d1 + (uint32_t)y) * (uint32_t)d0 + (uint32_t)xw;
+                for (uint32_t u = cs[row], ue = cs[row + 1]; u < ue; ++u) screen(u, p32s[u], qx, qi.y + sy, qi.z + sz);
             }
         }
-        int cnt = P.cnt;
-        uint32_t* list = P.list;
-        if (cnt > kCandCap) {
-            atomicOr(&info->err, kErrCand);
-            atomicMax(&info->cand_need, (uint32_t)cnt);
-            cnt = kCandCap;
-        }
-        uint32_t* out = cand + (int64_t)i * kCandCap;
-        for (int k = 0; k < cnt; ++k) out[k] = list[k];
+        work_off();
+        double hi_ = -1.0;   // the exact hull of i, computed when a wall test needs it
         // walls: a conservative FP32 test of the signed distance (errors as
         // for the pairs, within wmargin), the exact FP64 test for the rest
         uint32_t wmask = 0;
@@ -771,6 +893,7 @@ k_narrow(int64_t n, const uint32_t* __restrict__ skeys, const uint32_t* __restri
             if (kc >= 0 && kc < planes.ncones) {   // cone (plain scenes only)
                 if (cone_distance_f(g, kc, qi) > qi.w + g.tauf + g.cmargin) continue;
                 double nrm[3], sd;
+                const double4_32a pi = pos_r[i];
                 if (!(hi_ >= 0.0)) hi_ = hull_of(H, i, pi.w);
                 if (cone_distance(planes.cone[kc], pi, sd, nrm) && xsub(sd, pi.w) <= xadd(hi_, g.tau))
                     wmask |= 1u << k;
@@ -789,11 +912,11 @@ k_narrow(int64_t n, const uint32_t* __restrict__ skeys, const uint32_t* __restri
             double nrm[3], c, sd, xi;
             uint32_t widx;
             wall_plane(planes, V, si, k, nrm, c, widx);
+            const double4_32a pi = pos_r[i];
             if (!(hi_ >= 0.0)) hi_ = hull_of(H, i, pi.w);
             if (wall_kept(nrm, c, pi, hi_, g.tau, sd, xi)) wmask |= 1u << k;
         }
-        sph_cnt[i] = (uint32_t)cnt | (wmask << 8);
-        row_cnt[i] = (uint32_t)(cnt + __popc(wmask));
+        wall_mask[i] = wmask;
     }
 }
 
@@ -804,8 +927,8 @@ k_narrow(int64_t n, const uint32_t* __restrict__ skeys, const uint32_t* __restri
 // the walls of a body stay with its own lane.
 __global__ void k_write_contacts(int64_t n, int64_t ccap, const uint32_t* __restrict__ svals,
                                  const double4_32a* __restrict__ pos_r,
-                                 const uint32_t* __restrict__ cand, const uint32_t* __restrict__ sph_cnt,
-                                 const uint32_t* __restrict__ row_off, GridArgs g, Planes planes, SceneView V,
+                                 const uint32_t* __restrict__ cand, const uint32_t* __restrict__ pair_cnt,
+                                 const uint32_t* __restrict__ wall_mask, const uint32_t* __restrict__ row_off, GridArgs g, Planes planes, SceneView V,
                                  uint32_t* __restrict__ cj1, uint32_t* __restrict__ cj2, double4_32a* __restrict__ cgeo,
                                  double2* __restrict__ clev)
 {
@@ -815,17 +938,17 @@ __global__ void k_write_contacts(int64_t n, int64_t ccap, const uint32_t* __rest
     // warp-uniform trip count: every lane takes part in the shuffles
     for (int64_t s0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); s0 < n; s0 += wstride) {
         const int64_t s = s0 + lane;
-        uint32_t i = 0, packed = 0, ro = 0;
+        uint32_t i = 0, ns = 0, wm = 0, ro = 0;
         double4_32a pi = make_double4_32a(0.0, 0.0, 0.0, 0.0);
         if (s < n) {
             i = svals[s];
-            packed = sph_cnt[i];
-            if (packed != 0) {
+            ns = min(pair_cnt[i], (uint32_t)kCandCap);
+            wm = wall_mask[i];
+            if ((ns | wm) != 0) {
                 pi = pos_r[i];
                 ro = row_off[i];
             }
         }
-        const uint32_t ns = packed & 0xFFu;
         uint32_t pre = ns;   // inclusive prefix of the pair counts over the lanes
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -854,9 +977,14 @@ __global__ void k_write_contacts(int64_t n, int64_t ccap, const uint32_t* __rest
             po.w = __shfl_sync(0xffffffffu, pi.w, own);
             if (t >= total) continue;
             const uint32_t k = t - (end_o - ns_o);
-            const int64_t idx = (int64_t)ro_o + k;
+            // the list holds its pairs as they were found: contact k goes to
+            // the place of its partner in ascending order
+            const uint32_t* list = cand + (int64_t)i_o * kCandCap;
+            const uint32_t j = list[k];
+            uint32_t rank = 0;
+            for (uint32_t m = 0; m < ns_o; ++m) rank += list[m] < j ? 1u : 0u;
+            const int64_t idx = (int64_t)ro_o + rank;
             if (idx >= ccap) continue;
-            const uint32_t j = cand[(int64_t)i_o * kCandCap + k];
             const double4_32a pj = pos_r[j];
             const double dx3 = min_image(xsub(po.x, pj.x), g.periodic[0], L0);
             const double dy3 = min_image(xsub(po.y, pj.y), g.periodic[1], L1);
@@ -875,7 +1003,6 @@ __global__ void k_write_contacts(int64_t n, int64_t ccap, const uint32_t* __rest
             cgeo[idx] = geo;
             clev[idx] = make_double2(xsub(d, pj.w), pj.w);
         }
-        const uint32_t wm = packed >> 8;
         if (wm == 0) continue;
         const uint32_t si = V.batch ? V.scene_of[i] : 0u;
         int64_t idx = (int64_t)ro + ns;
@@ -1020,36 +1147,34 @@ nbgs_status run_detect(nbgs_scene* s)
                                                       (const double4_32a*)s->bvel, s->prm.dt, s->prm.tau, s->pos_r,
                                                       s->hull, s->p32, g, s->info);
     } else if (s->fp32)
-        k_hull<float><<<gb, T, 0, st>>>(n, (const float4*)s->vel, s->pos_r, s->prm.dt, s->prm.tau, s->hvw, s->p32,
-                                        g, s->info, s->scene_of, s->scene_vmax);
+        k_hull<float><<<gb, T, 0, st>>>(n, (const float4*)s->vel, s->pos_r, s->prm.dt, s->prm.tau, s->p32, g, s->info,
+                                        s->scene_of, s->scene_vmax);
     else
-        k_hull<double><<<gb, T, 0, st>>>(n, (const double4_32a*)s->vel, s->pos_r, s->prm.dt, s->prm.tau, s->hvw,
-                                         s->p32, g, s->info, s->scene_of, s->scene_vmax);
-    k_grid_setup<<<1, 1, 0, st>>>(g, s->info);
+        k_hull<double><<<gb, T, 0, st>>>(n, (const double4_32a*)s->vel, s->pos_r, s->prm.dt, s->prm.tau, s->p32, g,
+                                         s->info, s->scene_of, s->scene_vmax);
     cudaMemsetAsync(s->cell_end, 0, (size_t)s->max_cells * sizeof(uint32_t), st);   // cell counts
-    k_cell_keys<<<gb, T, 0, st>>>(n, s->p32, s->info, s->keys[0], s->vals[0], s->cell_end);
-    if (s->timing) s->phase_launches[0] += 4;
-    nbgs_status rc = radix_sort_pairs(s, s->keys[0], s->vals[0], s->keys[1], s->vals[1], n, s->key_bits);
+    k_cell_keys<<<gb, T, 0, st>>>(n, s->p32, g, s->info, s->ckey, s->crank, s->cell_end);
+    // first slot of every cell (empty ones included); cell_start[max_cells] = n
+    nbgs_status rc = exclusive_scan_u32(s, s->cell_end, s->cell_start, s->max_cells, nullptr);
     if (rc != NBGS_OK) return rc;
-    // first sorted slot of every cell (empty ones included); cell_start[max_cells] = n
-    rc = exclusive_scan_u32(s, s->cell_end, s->cell_start, s->max_cells, nullptr);
-    if (rc != NBGS_OK) return rc;
-    k_gather_sorted<<<gb, T, 0, st>>>(n, s->vals[0], s->p32, s->p32s);
-    const HullView H{s->composite ? s->hull : nullptr, s->hvw, s->prm.dt, s->prm.tau};
-    k_narrow<<<grid_for(n, 128, 16, s->num_sms), 128, 0, st>>>(n, s->keys[0], s->vals[0], s->pos_r, H,
-                                                                 s->p32s, s->cell_start, g, s->planes,
-                                                                 scene_view(s), s->info, s->cand, s->sph_cnt,
-                                                                 s->row_cnt);
-    rc = exclusive_scan_u32(s, s->row_cnt, s->row_off, n, &s->info->n_contacts);
-    if (rc != NBGS_OK) return rc;
+    k_cell_scatter<<<gb, T, 0, st>>>(n, s->ckey, s->crank, s->cell_start, s->p32, s->svals, s->p32s);
     if (s->timing) s->phase_launches[0] += 5;
+    cudaMemsetAsync(s->pair_cnt, 0, (size_t)n * sizeof(uint32_t), st);
+    const HullView H{s->composite ? s->hull : nullptr, s->vel, s->fp32 ? 1 : 0, s->prm.dt, s->prm.tau};
+    k_narrow<<<grid_for(n, kNarrowThreads, 16, s->num_sms), kNarrowThreads, 0, st>>>(n, s->svals, s->pos_r, H,
+                                                                 s->p32s, s->cell_start, g, s->planes,
+                                                                 scene_view(s), s->info, s->cand, s->pair_cnt,
+                                                                 s->wall_mask);
+    rc = exclusive_scan(s, ScanRows{s->pair_cnt, s->wall_mask}, s->row_off, DCount{n, nullptr}, &s->info->n_contacts);
+    if (rc != NBGS_OK) return rc;
+    if (s->timing) s->phase_launches[0] += 3;
     if (s->device_sized) {
         // no synchronisation: the buffers keep their capacity, an overflow
         // sets an error bit (the writes past it are skipped), and every
         // later kernel reads the count on the device
         k_check_contacts<<<1, 1, 0, st>>>(s->info, s->ccap);
-        k_write_contacts<<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->ccap, s->vals[0], s->pos_r,
-                                                                      s->cand, s->sph_cnt, s->row_off, g, s->planes,
+        k_write_contacts<<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->ccap, s->svals, s->pos_r,
+                                                                      s->cand, s->pair_cnt, s->wall_mask, s->row_off, g, s->planes,
                                                                       scene_view(s), s->cj1, s->cj2, s->cgeo, s->clev);
         if (s->timing) {
             s->phase_launches[0] += 3;
@@ -1076,8 +1201,8 @@ nbgs_status run_detect(nbgs_scene* s)
         rc = grow_contacts(s, nc);
         if (rc != NBGS_OK) return rc;
     }
-    k_write_contacts<<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->ccap, s->vals[0], s->pos_r, s->cand,
-                                                                  s->sph_cnt, s->row_off, g, s->planes, scene_view(s),
+    k_write_contacts<<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->ccap, s->svals, s->pos_r, s->cand,
+                                                                  s->pair_cnt, s->wall_mask, s->row_off, g, s->planes, scene_view(s),
                                                                   s->cj1, s->cj2, s->cgeo, s->clev);
     if (s->timing) {
         s->phase_launches[0] += 1;

@@ -6,7 +6,7 @@
 //           vel    R4[2n]      (v, 1/m), (omega, 1/I) adjacent per body:
 //                              32 B per body in FP32 (one sector), 64 B in FP64
 //           hull   double[n]   h_i of this step
-//   grid    cell_start/end u32[max_cells], keys/vals u32[n] x2 (radix sort)
+//   grid    cell_start/end u32[max_cells], ckey/crank/svals u32[n] (counting sort)
 //   contacts (canonical, CSR by j1): cj1, cj2 u32; cgeo double4_32a (n, xi);
 //           clev double2 (la, lb) with lever arms l_a = -la n, l_b = lb n
 //   sweep   srec SweepRec<R>[C] in colour order; sp R4[C] impulses (p_n, p_t, p_o)
@@ -427,7 +427,6 @@ struct nbgs_scene {
     double4_32a* quat = nullptr;
     void* vel = nullptr;          // R4[2 (n + icap)]: (v, 1/m), (w, 1/I) per body, then extra instances
     double* hull = nullptr;
-    double2* hvw = nullptr;        // |v|^2, |w|^2 per sphere (the exact hulls' inputs)
     float4* p32 = nullptr;        // (x - lo, y - lo, z - lo, r + h) in FP32: cell keys and the narrow-phase pre-filter
     float4* p32s = nullptr;       // p32 in cell order (the narrow phase's candidate reads)
     uint8_t* finite = nullptr;    // body takes impulses (1/m > 0 or 1/I > 0)
@@ -435,19 +434,19 @@ struct nbgs_scene {
     // grid
     int dims_max[3] = {1, 1, 1};
     int64_t max_cells = 1;
-    int key_bits = 1;
     uint32_t* cell_start = nullptr;   // max_cells + 1: first sorted slot of every cell
     uint32_t* cell_end = nullptr;     // max_cells: bodies per cell
-    uint32_t* keys[2] = {nullptr, nullptr};
-    uint32_t* vals[2] = {nullptr, nullptr};
+    uint32_t* ckey = nullptr;         // n: cell of every body
+    uint32_t* crank = nullptr;        // n: its rank among the cell's bodies
+    uint32_t* svals = nullptr;        // n: bodies in cell order
     uint32_t* radix_hist = nullptr;
     int64_t radix_hist_len = 0;
     uint32_t* scan_tmp = nullptr;  // block sums of the scans
     int64_t scan_tmp_len = 0;
     // candidates
     uint32_t* cand = nullptr;      // n * kCandCap
-    uint32_t* sph_cnt = nullptr;   // sphere contacts per body (bits 0-7), kept-wall mask (bits 8-31)
-    uint32_t* row_cnt = nullptr;   // contacts per body (sphere + wall)
+    uint32_t* pair_cnt = nullptr;  // n: pairs whose lower body it is
+    uint32_t* wall_mask = nullptr; // n: kept walls
     uint32_t* row_off = nullptr;   // n + 1
     // contacts (canonical)
     int64_t ccap = 0;

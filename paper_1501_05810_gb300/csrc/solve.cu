@@ -1084,7 +1084,7 @@ static nbgs_status solve_impl(nbgs_scene* s, int max_sweeps, double tol)
                 // detection's per-body counts (the body offsets adj_off stay: the
                 // network's features read them in the kernel's prologue)
                 int* dmin = (int*)s->deg;
-                int* dmax = (int*)s->row_cnt;
+                int* dmax = (int*)s->wall_mask;
                 cudaMemsetAsync(dmin, 0x7F, s->n * sizeof(int), st);   // large positive
                 cudaMemsetAsync(dmax, 0x80, s->n * sizeof(int), st);   // large negative
                 k_body_blocks<<<grid_for(A.C, T, 8, s->num_sms), T, 0, st>>>(Cn, s->n, B, s->perm, s->cj1, s->cj2,
