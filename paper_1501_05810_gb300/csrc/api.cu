@@ -482,7 +482,7 @@ static nbgs_status create_common(const nbgs_params* params, const nbgs_batch_des
         bool okb = take(s, s->scene_of, nn) && take(s, s->scene_off, S + 1) && take(s, s->scene_box, 6 * S) &&
                    take(s, s->scene_box32, 6 * S) &&
                    take(s, s->scene_mu, S) && take(s, s->scene_vmax, S) && take(s, s->scene_vref, S) &&
-                   take(s, s->scene_rk, 3 * S) && take(s, s->scene_done, S) && take(s, s->scene_res, S);
+                   take(s, s->scene_rk, 3 * S + 3) && take(s, s->scene_par, S) && take(s, s->scene_done, S) && take(s, s->scene_res, S);
         uint32_t* h_of = okb ? (uint32_t*)malloc(nn * sizeof(uint32_t)) : nullptr;
         uint32_t* h_off = okb ? (uint32_t*)malloc((S + 1) * sizeof(uint32_t)) : nullptr;
         double* h_box = okb ? (double*)malloc(6 * S * sizeof(double)) : nullptr;
@@ -579,7 +579,7 @@ void nbgs_destroy_scene(nbgs_scene* s)
                   s->cell_end, s->ckey, s->crank, s->svals, s->radix_hist, s->scan_tmp,
                   s->cand, s->pair_cnt, s->wall_mask, s->row_off, s->prev_row_off, s->deg, s->adj_off,
                   s->col_count, s->col_off, s->info, s->dep, s->prog, s->cstart, s->scene_of, s->scene_off,
-                  s->scene_box, s->scene_box32, s->scene_mu, s->scene_vmax, s->scene_vref, s->scene_rk,
+                  s->scene_box, s->scene_box32, s->scene_mu, s->scene_vmax, s->scene_vref, s->scene_rk, s->scene_par,
                   s->scene_done, s->scene_res, s->mlp_theta, s->cmask};
     for (void* p : ps) dev_free(s, p);
     free_contact_arrays(s);

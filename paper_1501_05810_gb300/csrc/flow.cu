@@ -50,11 +50,6 @@ template <class R> struct FlowArgs {
     const typename Mass2<R>::T* mass;  // (1/m, 1/I), kept for the way back
     const SweepRec<R>* rec;
     const SweepPre<R>* pre;
-    __device__ __forceinline__ uint32_t body_a(uint32_t s) const
-    {
-        return sizeof(R) == 4 ? __float_as_uint(reinterpret_cast<const SweepRec<float>*>(rec)[s].a.x)
-                              : reinterpret_cast<const uint32_t*>(rec + s)[0];
-    }
     R4<R>* p;                         // impulses and dep words, colour order
     const uint32_t* col_off;
     DevInfo* info;
@@ -64,18 +59,89 @@ template <class R> struct FlowArgs {
     double tol;
     int warm;
     int tile;                         // contacts per tile: a power of two, at most 32
-    SceneView V;                      // batched scenes
+    // batched scenes
+    const uint32_t* scene_of;
     int64_t nscene;
-    unsigned long long* scene_rk;
+    const R4<R>* scene_par;           // (mu, r^2 at the tolerance, r^2 at which R_k exceeds it, -) per scene
+    const double* scene_vref;
+    unsigned long long* scene_rk;     // 3 x nscene rotating slots of max r^2 (bits), then 3 of "some R above tol"
     uint32_t* scene_done;
     double* scene_res;
 };
 
-// Gravity, versions 0 and the mass array.
+__device__ __forceinline__ unsigned long long bits_of(float x) { return __float_as_uint(x); }
+__device__ __forceinline__ unsigned long long bits_of(double x) { return (unsigned long long)__double_as_longlong(x); }
+__device__ __forceinline__ void from_bits(unsigned long long b, float& x) { x = __uint_as_float((uint32_t)b); }
+__device__ __forceinline__ void from_bits(unsigned long long b, double& x) { x = __longlong_as_double((long long)b); }
+
+__device__ __forceinline__ uint32_t body_a(const SweepRec<float>& r) { return __float_as_uint(r.a.x); }
+__device__ __forceinline__ uint32_t body_a(const SweepRec<double>& r) { return (uint32_t)__double2loint(r.ids_bias.x); }
+
+// R_k of a scene from the largest r^2 of its contacts
+template <class R> __device__ __forceinline__ double scene_residual(R r2, double vref) { return (double)sqrt(r2) / vref; }
+
+// The largest r^2 >= 0 whose residual (rounded to R first if asked: what the
+// record of R_k holds) is at or below tol.  Non-negative numbers order like
+// their bits and the residual does not fall as r^2 grows, so a bisection
+// finds it; it starts next to (tol v_ref)^2.
+template <class R> __device__ R r2_at_tol(double vref, double tol, bool rounded)
+{
+    auto meets = [&](unsigned long long b) {
+        R x;
+        from_bits(b, x);
+        const double r = scene_residual<R>(x, vref);
+        return (rounded ? (double)(R)r : r) <= tol;
+    };
+    const R t = (R)(tol * vref), guess = t * t;
+    unsigned long long lo = 0ull, hi = bits_of(sizeof(R) == 4 ? (R)__int_as_float(0x7F800000) : (R)__longlong_as_double(0x7FF0000000000000LL));
+    if (meets(hi)) lo = hi;   // an infinite tolerance
+    const unsigned long long g = bits_of(guess);
+    if (g > 32ull && g < hi && meets(g - 32ull)) lo = g - 32ull;
+    if (g + 32ull < hi && !meets(g + 32ull)) hi = g + 32ull;
+    while (hi - lo > 1ull) {   // meets(lo) and not meets(hi)
+        const unsigned long long m = lo + (hi - lo) / 2ull;
+        if (meets(m)) lo = m;
+        else hi = m;
+    }
+    R x;
+    from_bits(lo, x);
+    return x;
+}
+
+// max r^2 of the scenes of a tile's live contacts: the contacts of a tile are
+// mostly of one scene, whose maximum is then one atomic nobody waits for.
+__device__ __forceinline__ void scene_max(unsigned long long* rk, uint32_t scene, bool live, bool lead,
+                                          unsigned long long bits)
+{
+    const uint32_t m = __ballot_sync(kFull, live);   // some lane is
+    const int first = __ffs((int)m) - 1;
+    const uint32_t scene0 = __shfl_sync(kFull, scene, first);   // by every lane, live or not
+    if (__all_sync(kFull, !live || scene == scene0)) {
+        if (!live) bits = 0ull;
+        // non-negative numbers order like their bits, NaN above them
+        const uint32_t hi = __reduce_max_sync(kFull, (uint32_t)(bits >> 32));
+        const uint32_t lo = __reduce_max_sync(kFull, (uint32_t)(bits >> 32) == hi ? (uint32_t)bits : 0u);
+        if ((int)(threadIdx.x & 31) == first) atomicMax(rk + scene, (unsigned long long)hi << 32 | lo);
+    } else if (live && lead) {
+        atomicMax(rk + scene, bits);
+    }
+}
+
+// Gravity, versions 0 and the mass array; of batched scenes (nscene > 0) also
+// what their contacts ask for.
 template <class R>
 __global__ void k_flow_init(int64_t n, const R4<R>* __restrict__ vel, R gx, R gy, R gz, uint4* __restrict__ tv,
-                            typename Mass2<R>::T* __restrict__ mass)
+                            typename Mass2<R>::T* __restrict__ mass, int64_t nscene, const double* __restrict__ mu,
+                            const double* __restrict__ vref, double tol, R4<R>* __restrict__ par)
 {
+    for (int64_t sc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; sc < nscene; sc += (int64_t)gridDim.x * blockDim.x) {
+        R4<R> q;
+        q.x = (R)mu[sc];
+        q.y = r2_at_tol<R>(vref[sc], tol, false);
+        q.z = r2_at_tol<R>(vref[sc], tol, true);
+        q.w = R(0);
+        par[sc] = q;
+    }
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         R4<R> v, w;
         ld_body(vel + 2 * i, v, w);
@@ -110,9 +176,10 @@ __global__ void k_flow_out(FlowArgs<R> A, R4<R>* __restrict__ vel)
     if (Batch) {   // scenes still short of their tolerance ran every sweep
         for (int64_t sc = gtid; sc < A.nscene; sc += gstride) {
             if (A.scene_done[sc] == 0) {
+                R r2 = R(0);
+                if (k > 0) from_bits(A.scene_rk[scene_slot(k - 1) * A.nscene + sc], r2);
                 A.scene_done[sc] = (uint32_t)k;
-                A.scene_res[sc] =
-                    k > 0 ? __longlong_as_double((long long)A.scene_rk[scene_slot(k - 1) * A.nscene + sc]) : 0.0;
+                A.scene_res[sc] = scene_residual<R>(r2, A.scene_vref[sc]);
             }
         }
     }
@@ -148,7 +215,6 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
     const uint32_t W = nb * (blockDim.x >> 5), w0 = (threadIdx.x >> 5) * nb + blockIdx.x;
     const bool work = w0 < ntile;
     const double vref = v_ref_of(A.info, A.gdt_norm);
-    const double vnorm = Batch ? 1.0 : vref;   // batched residuals arrive already divided by v_ref_s
     const int warm = A.warm ? 1 : 0;
     const int npass = A.max_sweeps + warm;
     bool ok = true;
@@ -183,6 +249,10 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         npre = ld_pre(A.pre + sl);
         npp = A.p[sl];
     };
+    // of a batch: the contact's scene and what that asks of a contact
+    uint32_t na = 0, nscene = 0, scene = 0;
+    R4<R> par = {};
+    R prev = R(0);
     // the records of the warp's next tile: into registers, or, in the variant
     // whose many warps leave none to spare, into L1 (loads nobody waits for)
     constexpr bool Touch = sizeof(R) == 4 && L == 1;
@@ -193,11 +263,20 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         if constexpr (Touch) {
             uint32_t x;
             asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(A.rec + sl));
+            if (Batch) na = x;   // the record's first word
             asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(A.pre + sl));
             asm volatile("ld.global.b32 %0, [%1];" : "=r"(x) : "l"(A.p + sl));
         } else {
             read(sl);
+            if (Batch) na = body_a(nrec);
         }
+    };
+    auto scene_of = [&](bool live) { nscene = live ? A.scene_of[na] : 0u; };
+    // prev: the scene's largest r^2 of the sweep before, complete since the barrier (NaN: no sweep yet)
+    auto ask = [&](int sweep) {
+        par = A.scene_par[scene];
+        from_bits(sweep > 0 ? ((volatile unsigned long long*)A.scene_rk)[scene_slot(sweep - 1) * A.nscene + scene]
+                            : ~0ull, prev);
     };
     // the contact fetched (slot s) becomes the unit's current one
     auto take = [&]() {
@@ -212,7 +291,9 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
     if (work) {
         seek(at, w0, 0);
         fetch(at, s, on);
+        if (Batch) scene_of(on);
         take();
+        scene = nscene;
     }
     int k = 0;
     for (int pass = 0; pass < npass; ++pass) {
@@ -220,12 +301,16 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         k = pass - warm;
         if (!apply) {
             if (blockIdx.x == 0 && threadIdx.x == 0 && k + 1 >= kHistKept) A.info->rk_bits[rk_slot(k + 1)] = 0ull;
-            if (Batch)   // the slot of sweep k + 1 is neither read nor written during sweep k
+            if (Batch) {   // the slots of sweep k + 1 are neither read nor written during sweep k
+                if (blockIdx.x == 0 && threadIdx.x == 0) A.scene_rk[3 * A.nscene + scene_slot(k + 1)] = 0ull;
                 for (int64_t sc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; sc < A.nscene;
                      sc += (int64_t)gridDim.x * blockDim.x)
                     A.scene_rk[scene_slot(k + 1) * A.nscene + sc] = 0ull;
+            }
         }
         R rmax = R(0);
+        bool over = false;   // a scene's contact above its tolerance
+        if (Batch) ask(apply ? 0 : k);
         const uint32_t base = (uint32_t)pass << 9;
         for (bool more = work; more && ok;) {
             K.load(A.tv);
@@ -244,20 +329,9 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
                 fetch(at, sn, non);
             }
             const uint32_t dep = on ? dep_bits(K.pp.w) : 0u;
-            bool live = on;
-            R mu = A.mu;
-            double vref_s = 1.0;
-            uint32_t scene = 0;
-            if (Batch && on) {
-                scene = A.V.scene_of[A.body_a(s)];
-                if (!apply && k > 0) {   // this scene met its tolerance in an earlier sweep: it is done
-                    const double prev =
-                        __longlong_as_double((long long)A.scene_rk[scene_slot(k - 1) * A.nscene + scene]);
-                    if (prev <= A.tol) live = false;
-                }
-                mu = (R)A.V.mu[scene];
-                vref_s = A.V.vref[scene];
-            }
+            // a scene that met its tolerance in an earlier sweep is done
+            const bool live = on && !(Batch && prev <= par.y);
+            const R mu = Batch ? par.x : A.mu;
             const bool va = live && (dep & kDepListA) != 0u, vb = live && K.hasb && (dep & kDepListB) != 0u;
             const uint32_t ma = va ? ~0u : 0u, mb = vb ? ~0u : 0u;
             const uint32_t ea = base | (dep & 0x1FFu), eb = base | ((dep >> 11) & 0x1FFu);
@@ -283,22 +357,23 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
                 }
                 if (!ok) break;
             }
-            if (apply) {
+            if (Batch && !same) scene_of(non);   // the next tile's: its record has arrived
+            if (Batch && !__any_sync(kFull, live)) {
+                // nothing to do in this tile
+            } else if (apply) {
                 K.template relax<true>(live, mu, A.omega);
                 K.store(A.tv, va, vb, oa, ob);
             } else {
                 K.template relax<false>(live, mu, A.omega);
                 K.store(A.tv, va, vb, oa, ob);
                 if (live) K.save(A.p + s);
-                R r2 = K.residual();
-                if (Batch && live) {   // per-scene R_k; the read filter only saves atomics
-                    const double rn = (double)sqrt(r2) / vref_s;
-                    unsigned long long* dst = A.scene_rk + scene_slot(k) * A.nscene + scene;
-                    const unsigned long long bits = (unsigned long long)__double_as_longlong(rn);
-                    if (lane % L == 0 && bits > *(volatile unsigned long long*)dst) atomicMax(dst, bits);
-                    r2 = (R)rn;
+                const R r2 = K.residual();
+                if (Batch) {
+                    over = over || (live && !(r2 <= par.z));
+                    scene_max(A.scene_rk + scene_slot(k) * A.nscene, scene, live, lane % L == 0, bits_of(r2));
+                } else {
+                    rmax = live && above(r2, rmax) ? r2 : rmax;
                 }
-                rmax = live && above(r2, rmax) ? r2 : rmax;
             }
             __syncwarp();   // the lanes of a unit read back what one of them saved
             more = !wrap;
@@ -306,6 +381,10 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
                 s = sn;
                 on = non;
                 take();
+                if (Batch) {
+                    scene = nscene;
+                    ask(apply ? 0 : k);
+                }
             }
         }
         if (apply) continue;
@@ -330,9 +409,34 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
             ok = false;
             break;
         }
+        if (Batch) {
+            if (__syncthreads_or(over) && threadIdx.x == 0) atomicMax(A.scene_rk + 3 * A.nscene + scene_slot(k), 1ull);
+            if (!grid_barrier(A.info, nb)) {
+                ok = false;
+                break;
+            }
+            // the largest R_k and the scenes that met their tolerance in this
+            // sweep, by the last warps of the grid: they have the fewest tiles
+            for (int64_t sc = (int64_t)nb * blockDim.x - 1 - (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+                 sc < A.nscene; sc += (int64_t)nb * blockDim.x) {
+                R r2;
+                from_bits(((volatile unsigned long long*)A.scene_rk)[scene_slot(k) * A.nscene + sc], r2);
+                if (r2 == R(0) && A.scene_done[sc] != 0) continue;
+                const double rs = scene_residual<R>(r2, A.scene_vref[sc]);
+                double x = (double)(R)rs;
+                if (!(x <= 1e300)) x = __longlong_as_double(0x7FF0000000000000LL);
+                atomicMax(&A.info->rk_bits[rk_slot(k)], (unsigned long long)__double_as_longlong(x));
+                if (A.tol > 0.0 && A.scene_done[sc] == 0 && rs <= A.tol) {
+                    A.scene_done[sc] = (uint32_t)(k + 1);
+                    A.scene_res[sc] = rs;
+                }
+            }
+            if (A.tol > 0.0 && ((volatile unsigned long long*)A.scene_rk)[3 * A.nscene + scene_slot(k)] == 0ull) break;
+            continue;
+        }
         const double rb = block_max_to<R>(rmax, &A.info->rk_bits[rk_slot(k)]);
         if (vote) {
-            const int v = tol_vote(A.info, k, rb, vnorm, A.tol, nb, &s_vote);
+            const int v = tol_vote(A.info, k, rb, vref, A.tol, nb, &s_vote);
             if (v < 0) ok = false;
             if (v <= 0) break;
             continue;
@@ -341,18 +445,7 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
             ok = false;
             break;
         }
-        if (Batch && A.tol > 0.0) {   // scenes that met their tolerance in this sweep
-            for (int64_t sc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; sc < A.nscene;
-                 sc += (int64_t)gridDim.x * blockDim.x) {
-                const double rs = __longlong_as_double(
-                    (long long)((volatile unsigned long long*)A.scene_rk)[scene_slot(k) * A.nscene + sc]);
-                if (A.scene_done[sc] == 0 && rs <= A.tol) {
-                    A.scene_done[sc] = (uint32_t)(k + 1);
-                    A.scene_res[sc] = rs;
-                }
-            }
-        }
-        const double Rk = __longlong_as_double((long long)((volatile unsigned long long*)A.info->rk_bits)[rk_slot(k)]) / vnorm;
+        const double Rk = __longlong_as_double((long long)((volatile unsigned long long*)A.info->rk_bits)[rk_slot(k)]) / vref;
         if (A.tol > 0.0 && Rk <= A.tol) break;
     }
     // sweeps run: k + 1 after a break at sweep k, and max_sweeps at the end
@@ -375,10 +468,10 @@ int flow_occ(const void* fn, int threads)
     return o;
 }
 
-// Which kernel, and how many warps, for a scene of n bodies.
+// Which kernel, and how many warps, for a scene of n bodies and C contacts.
 //
-// A pile has 2 to 3 contacts per body (6 at most) in 13 to 18 colours.  Up to
-// some 10^5 bodies a sweep takes as long as its longest chain of contacts, so
+// A pile has 2.7 contacts per body (6 at most) in 13 to 18 colours.  Up to
+// some 10^5 contacts a sweep takes as long as its longest chain of contacts, so
 // the contact itself has to be quick (more lanes) and a warp beyond the tiles
 // of a colour only polls; above, it takes as long as the memory system needs
 // for the contacts in flight, so they have to be many.  50 sweeps of a pile,
@@ -391,25 +484,29 @@ int flow_occ(const void* fn, int threads)
 //   FP64, 4 lanes, 8 warps/SM    1.44    1.74    2.23    3.67    7.09
 //   FP64, 1 lane,  4 warps/SM    3.14    4.20    4.43    4.43    5.31
 //   FP64, 1 lane,  8 warps/SM    3.14    4.91    5.55    5.73    5.83
+// The FP32 kernels give the same bits, so their line is drawn by what decides,
+// the contacts (256 loose scenes, 1.1M bodies with 0.6M contacts, two steps:
+// 17.1 ms with two lanes, 19.2 with one); the FP64 ones by the bodies, which
+// do not change from step to step.
 struct FlowPlan {
     const void* fn;
     int tile, warps, blocks_per_sm;   // contacts per tile, warps per block
 };
 
 template <class R>
-FlowPlan flow_plan(int64_t n, bool batch);
+FlowPlan flow_plan(int64_t n, int64_t C, bool batch);
 
 template <>
-FlowPlan flow_plan<float>(int64_t n, bool batch)
+FlowPlan flow_plan<float>(int64_t, int64_t C, bool batch)
 {
-    if (n < 350000)
+    if (C < 950000)
         return {batch ? (const void*)k_solve_flow<float, 2, true> : (const void*)k_solve_flow<float, 2, false>, 16, 8,
-                n < 90000 ? 1 : 2};
+                C < 245000 ? 1 : 2};
     return {batch ? (const void*)k_solve_flow<float, 1, true> : (const void*)k_solve_flow<float, 1, false>, 32, 4, 6};
 }
 
 template <>
-FlowPlan flow_plan<double>(int64_t n, bool batch)
+FlowPlan flow_plan<double>(int64_t n, int64_t, bool batch)
 {
     if (n < 64000)
         return {batch ? (const void*)k_solve_flow<double, 4, true> : (const void*)k_solve_flow<double, 4, false>, 8, 8, 1};
@@ -444,12 +541,15 @@ nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm)
     A.max_sweeps = max_sweeps;
     A.tol = tol;
     A.warm = warm;
-    A.V = scene_view(s);
-    A.nscene = s->n_scenes;
+    A.scene_of = s->scene_of;
+    A.nscene = s->batch ? s->n_scenes : 0;
+    A.scene_par = (const R4<R>*)s->scene_par;
+    A.scene_vref = s->scene_vref;
     A.scene_rk = s->scene_rk;
     A.scene_done = s->scene_done;
     A.scene_res = s->scene_res;
-    const FlowPlan P = flow_plan<R>(s->n, s->batch);
+    // a device-sized step knows the count of the last step the host looked at
+    const FlowPlan P = flow_plan<R>(s->n, s->device_sized ? (int64_t)s->hinfo->n_contacts : s->n_contacts, s->batch);
     A.tile = P.tile;
     const void* fn = P.fn;
     const int threads = 32 * P.warps;
@@ -458,7 +558,8 @@ nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm)
     if (nblocks < 1) return fail(s, NBGS_ECUDA, "solve: sweep kernel does not fit");
     const int T = 256, gb = grid_for(std::max<int64_t>(n, 1), T, 8, s->num_sms);
     k_flow_init<R><<<gb, T, 0, st>>>(n, (const R4<R>*)s->vel, (R)(s->prm.dt * g[0]), (R)(s->prm.dt * g[1]),
-                                     (R)(s->prm.dt * g[2]), A.tv, mass);
+                                     (R)(s->prm.dt * g[2]), A.tv, mass, A.nscene, s->scene_mu, s->scene_vref, tol,
+                                     (R4<R>*)s->scene_par);
     void* args[] = {&A};
     if (s->timing) cudaEventRecord(s->ev[8], st);
     const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nblocks), dim3(threads), args, 0, st);

@@ -417,7 +417,9 @@ struct nbgs_scene {
     double* scene_mu = nullptr;         // S
     unsigned long long* scene_vmax = nullptr;  // S: max |v| at step start (bits)
     double* scene_vref = nullptr;       // S
-    unsigned long long* scene_rk = nullptr;    // 3 x S rotating slots: max r_j / v_ref per sweep (bits)
+    unsigned long long* scene_rk = nullptr;    // 3 x S rotating slots: max r_j / v_ref per sweep (bits; the
+                                               // dataflow sweeps: max r_j^2 and three words more)
+    double4_32a* scene_par = nullptr;          // S: mu and tolerances as the dataflow sweeps take them
     uint32_t* scene_done = nullptr;     // S: sweeps to tolerance
     double* scene_res = nullptr;        // S: R_k at that sweep
     int max_coop_blocks = 0;            // occupancy limit of the persistent kernel

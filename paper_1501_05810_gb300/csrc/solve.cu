@@ -1045,7 +1045,7 @@ static nbgs_status solve_impl(nbgs_scene* s, int max_sweeps, double tol)
     if (s->batch) {
         k_scene_vref<<<grid_for(s->n_scenes, 256, 8, s->num_sms), 256, 0, st>>>(s->n_scenes, s->scene_vmax, A.gdt_norm,
                                                                                s->scene_vref);
-        cudaMemsetAsync(s->scene_rk, 0, 3 * s->n_scenes * sizeof(unsigned long long), st);
+        cudaMemsetAsync(s->scene_rk, 0, (3 * s->n_scenes + 3) * sizeof(unsigned long long), st);
         cudaMemsetAsync(s->scene_done, 0, s->n_scenes * sizeof(uint32_t), st);
         cudaMemsetAsync(s->scene_res, 0, s->n_scenes * sizeof(double), st);
         if (s->timing) s->phase_launches[2] += 1;

@@ -72,6 +72,45 @@ def test_flow_equals_grid_synchronised_sweeps(shape, precision, tol, omega, fixe
             assert np.abs(ca["impulse"] - cb["impulse"]).max() <= bound * np.abs(cb["impulse"]).max()
 
 
+@pytest.mark.parametrize("sizes,precision,tol", [
+    ((1, 1, 2), "fp32", 1e-6), ((60, 151, 300, 97, 420, 33), "fp32", 1e-6), ((60, 151, 300), "fp32", 1e300),
+    ((37,) * 700, "fp32", 1e-4), ((2000, 20, 9000, 400, 20000), "fp32", 0.0), ((300, 20, 900), "fp64", 0.0)])
+def test_batch_flow_equals_grid_synchronised_sweeps(sizes, precision, tol):
+    """Scenes that share tiles or fill many, that meet their tolerance at
+    different sweeps, at once or never, with more scenes than a block has
+    threads."""
+    from paper_1501_05810_gb300 import nbgs
+    rng = np.random.default_rng(len(sizes))
+    scs = []
+    for k, n in enumerate(sizes):
+        sc = scenes.batch_scene(k, n, mu=float(rng.uniform(0.2, 0.8)), precision=precision, warm_start="prev")
+        sc["vel"], sc["angvel"] = rng.normal(0.0, 2.0, (2, n, 3))
+        sc["params"]["dt"] = 0.03
+        scs.append(sc)
+    out = []
+    for flags in (0, GLOBAL_SYNC):
+        batch = scenes.layout_batch(scs)
+        for sc in batch:
+            sc["params"] = dict(sc["params"], sweep_flags=flags)
+        g = nbgs.BatchScene(batch)
+        got = [g.step_scenes(30, tol) for _ in range(2)]
+        out.append((got, g.residual_history(), g.get_bodies(), g.get_contacts()))
+        g.close()
+    (ga, ha, ba, ca), (gb, hb, bb, cb) = out
+    for (ka, ra), (kb, rb) in zip(ga, gb):
+        assert np.array_equal(ka, kb)
+        if precision == "fp32":
+            assert np.array_equal(ra, rb)
+    if precision == "fp32":   # the same roundings in every kernel
+        assert np.array_equal(ha, hb) and np.array_equal(ca["impulse"], cb["impulse"])
+        for k in ("pos", "quat", "vel", "angvel"):
+            assert np.array_equal(ba[k], bb[k]), k
+    else:   # as above, with 30 sweeps a step
+        bound = 1.1e-16 * 4 * 360 * 2 * 10
+        for k in ("vel", "angvel"):
+            assert np.abs(ba[k] - bb[k]).max() <= bound * np.abs(bb[k]).max()
+
+
 @pytest.mark.parametrize("shape,precision,tol", [((2, 2, 2), "fp32", 0.0), ((6, 5, 4), "fp64", 1e-4), ((7, 7, 7), "fp32", 1e-3),
                                                  ((40, 40, 38), "fp32", 0.0), ((85, 85, 84), "fp32", 0.0),
                                                  ((25, 25, 24), "fp64", 0.0)])
