@@ -190,7 +190,7 @@ nbgs_status nbgs_update_bodies(nbgs_scene* scene, const double* pos, const doubl
                                const double* vel, const double* angvel);
 
 /* Sect. 4: hull radii h_i = dt(|v_i| + |w_i| r_i) + tau from the current
- * velocities, uniform cell grid sorted by radix sort, narrow phase
+ * velocities, uniform cell grid (counting sort), narrow phase
  * (sphere-sphere, sphere-wall, sphere-cone).  A pair is kept iff
  * (d - r_a) - r_b <= h_a + h_b (walls: h = tau).  Contacts are stored in
  * canonical order of (j1 << 32) | j2, j1 < j2.  With a warm start, the
@@ -265,7 +265,7 @@ nbgs_status nbgs_batch_step(nbgs_scene* scene, int32_t max_sweeps, double tol, i
  * batched extension: thousands of scenes in one persistent sweep launch
  * under a captured graph).  Every step does what nbgs_step(max_sweeps, tol)
  * does, with device-sized launches: the contact count stays on the device,
- * the colouring rounds run in one cooperative launch, and the buffers keep
+ * the colouring needs no host in any case, and the buffers keep
  * the capacities they had at capture (contacts: the capacity the last
  * nbgs_step left, at least contacts_per_body per body).  A step that needs
  * more sets an error

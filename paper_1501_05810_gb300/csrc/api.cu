@@ -63,10 +63,8 @@ static bool alloc_contact_arrays(nbgs_scene* s, int64_t cap)
     const size_t c = (size_t)cap;
     bool ok = take(s, s->cj1, c) && take(s, s->cj2, c) && take(s, s->cgeo, c) && take(s, s->clev, c) &&
               take(s, s->cimp, c) && take(s, s->cworld, c) && take(s, s->prev_j2, c) && take(s, s->prev_P, c) &&
-              take(s, s->adj, 2 * c) && take(s, s->cstate, c) && take(s, s->cprio, c) && take(s, s->wl[0], 2 * c) &&
-              take(s, s->wl[1], 2 * c) && take(s, s->colour_key, c) && take(s, s->colour_key2, c) &&
-              take(s, s->cpack, c) &&
-              take(s, s->perm, c) && take(s, s->perm_in, c);
+              take(s, s->adj, 2 * c) && take(s, s->cstate, c) && take(s, s->cprio, c) && take(s, s->clist[0], c) && take(s, s->clist[1], c) && take(s, s->cmeet, c) &&
+              take(s, s->cpack, c) && take(s, s->perm, c) && take(s, s->inv, c);
     if (!ok) return false;
     s->srec = dev_alloc(s, c * rec_bytes(s));
     s->sp = dev_alloc(s, c * vec4_bytes(s));
@@ -77,20 +75,19 @@ static bool alloc_contact_arrays(nbgs_scene* s, int64_t cap)
 static void free_contact_arrays(nbgs_scene* s)
 {
     void* ps[] = {s->cj1, s->cj2, s->cgeo, s->clev, s->cimp, s->cworld, s->prev_j2, s->prev_P, s->adj, s->cstate,
-                  s->cprio, s->wl[0], s->wl[1], s->colour_key, s->colour_key2, s->perm, s->perm_in, s->srec, s->sp,
-                  s->spre, s->cpack};
+                  s->cprio, s->clist[0], s->clist[1], s->cmeet, s->perm, s->inv, s->srec, s->sp, s->spre, s->cpack};
     for (void* p : ps) dev_free(s, p);
 }
 
 static bool alloc_sort_temps(nbgs_scene* s)
 {
-    const int64_t big = std::max<int64_t>(std::max<int64_t>(s->n, s->ccap), 1);
+    const int64_t big = std::max<int64_t>(s->ccap, 1);
     const int64_t nb = (big + 4095) / 4096;
-    s->radix_hist_len = 256 * nb;
+    s->sort_hist_len = 256 * nb;
     const int64_t scan_len =
-        std::max<int64_t>(std::max<int64_t>(s->radix_hist_len, s->n + 1), std::max<int64_t>(s->ccap, s->max_cells) + 1);
+        std::max<int64_t>(std::max<int64_t>(s->sort_hist_len, s->n + 1), std::max<int64_t>(s->ccap, s->max_cells) + 1);
     s->scan_tmp_len = (scan_len + 4095) / 4096 + 1;
-    return take(s, s->radix_hist, (size_t)s->radix_hist_len + 1) && take(s, s->scan_tmp, (size_t)s->scan_tmp_len);
+    return take(s, s->sort_hist, (size_t)s->sort_hist_len + 1) && take(s, s->scan_tmp, (size_t)s->scan_tmp_len);
 }
 
 // Grow every contact-sized buffer to hold `need` contacts; the previous
@@ -104,7 +101,7 @@ nbgs_status grow_contacts(nbgs_scene* s, int64_t need)
     s->prev_j2 = nullptr;
     s->prev_P = nullptr;
     free_contact_arrays(s);
-    dev_free(s, s->radix_hist);
+    dev_free(s, s->sort_hist);
     dev_free(s, s->scan_tmp);
     s->ccap = cap;
     if (!alloc_contact_arrays(s, cap) || !alloc_sort_temps(s)) {
@@ -451,7 +448,7 @@ static nbgs_status create_common(const nbgs_params* params, const nbgs_batch_des
               take(s, s->pair_cnt, nn) && take(s, s->wall_mask, nn) && take(s, s->row_off, nn + 1) &&
               take(s, s->prev_row_off, nn + 1) && take(s, s->deg, nn + 1) && take(s, s->adj_off, nn + 1) &&
               take(s, s->cmask, 8 * (nn + 1)) &&
-              take(s, s->col_count, kMaxColours + 1) && take(s, s->col_off, kMaxColours + 1) &&
+              take(s, s->col_off, kMaxColours + 1) &&
               take(s, s->info, 1);
     if (ok) {
         s->vel = dev_alloc(s, 2 * nn * vec4_bytes(s));
@@ -576,9 +573,9 @@ void nbgs_destroy_scene(nbgs_scene* s)
     cudaStreamSynchronize(s->stream);
     drop_graphs(s);
     void* ps[] = {s->pos_r, s->quat, s->vel, s->hull, s->p32, s->p32s, s->finite, s->stage, s->cell_start,
-                  s->cell_end, s->ckey, s->crank, s->svals, s->radix_hist, s->scan_tmp,
+                  s->cell_end, s->ckey, s->crank, s->svals, s->sort_hist, s->scan_tmp,
                   s->cand, s->pair_cnt, s->wall_mask, s->row_off, s->prev_row_off, s->deg, s->adj_off,
-                  s->col_count, s->col_off, s->info, s->dep, s->prog, s->cstart, s->scene_of, s->scene_off,
+                  s->col_off, s->info, s->dep, s->prog, s->cstart, s->scene_of, s->scene_off,
                   s->scene_box, s->scene_box32, s->scene_mu, s->scene_vmax, s->scene_vref, s->scene_rk, s->scene_par,
                   s->scene_done, s->scene_res, s->mlp_theta, s->cmask};
     for (void* p : ps) dev_free(s, p);

@@ -8,22 +8,23 @@
 //   k_colour_init   priority splitmix64(key ^ seed), body degrees
 //   scan + k_adj_fill  body -> contact incidence lists (finite bodies only)
 //   k_adj_sort_*    every incidence list in decreasing priority; each
-//                   contact's position in the lists of its bodies
-//   k_fr_round      rounds of first-fit greedy colouring in decreasing
-//                   priority, as Jones-Plassmann rounds give it: a contact
-//                   at the front of the remaining lists of all its bodies
-//                   takes the smallest colour absent from their coloured
-//                   prefixes (k_fr_persistent: every round in one
-//                   cooperative launch, for device-sized steps)
-//   k_colour_keys   colour histogram
-//   radix pass      stable counting sort by colour -> permutation
+//                   contact's successors in the lists of its bodies
+//   k_colour_chase  first-fit greedy colouring in decreasing priority: a
+//                   contact takes the smallest colour absent from the
+//                   coloured prefixes of its bodies' lists as soon as all
+//                   its predecessors have theirs
+//   k_colour_hist, scan, k_colour_scatter
+//                   stable counting sort by colour -> permutation
 //   k_build_sweep   sweep records in colour order, initial impulses
 #include <algorithm>
-#include <utility>
 
 #include "relax.cuh"
 
 namespace nbgs {
+
+// Successor word of a contact in a body's list: the next contact (or
+// kNoNext), and whether one comes before it.
+constexpr uint32_t kNoNext = 0x7FFFFFFFu, kHasPrev = 1u << 31;
 
 // Key of a contact in its own scene's numbering (bodies from 0, walls
 // after the scene's bodies: shared planes, then the six box faces), so that
@@ -49,18 +50,20 @@ __device__ __forceinline__ uint64_t local_key(uint32_t a, uint32_t b, const Scen
 __global__ void k_colour_init(DCount Cc, int64_t n, const uint32_t* __restrict__ cj1, const uint32_t* __restrict__ cj2,
                               const uint32_t* __restrict__ ib1, const uint32_t* __restrict__ ib2,
                               const uint8_t* __restrict__ finite, uint64_t seed, SceneView V, uint32_t* __restrict__ deg,
-                              uint64_t* __restrict__ prio, uint32_t* __restrict__ cstate, uint4* __restrict__ cpack)
+                              uint64_t* __restrict__ prio, uint32_t* __restrict__ cstate, uint4* __restrict__ cpack,
+                              unsigned long long* __restrict__ meet)
 {
     const int64_t C = Cc.get();
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
         prio[c] = splitmix64(local_key(cj1[c], cj2[c], V) ^ seed);
         cstate[c] = kUncoloured;
+        meet[c] = 0ull;
         const uint32_t a = ib1[c], b = ib2[c];
         const bool fa = finite[a] != 0, fb = b < n && finite[b];
         if (fa) atomicAdd(&deg[a], 1u);
         if (fb) atomicAdd(&deg[b], 1u);
-        // the bodies whose incidence lists hold c (none: no list), positions later
-        cpack[c] = make_uint4(fa ? a : kNoList, fb ? b : kNoList, 0u, 0u);
+        // the bodies whose incidence lists hold c (none: no list), successors later
+        cpack[c] = make_uint4(fa ? a : kNoList, fb ? b : kNoList, kNoNext, kNoNext);
     }
 }
 
@@ -88,103 +91,97 @@ __device__ __forceinline__ bool beats(uint64_t pd, uint32_t d, uint64_t pc, uint
 // colouring in decreasing priority gives each contact the smallest colour
 // none of its predecessors (incident contacts that beat it) has.  With the
 // incidence list of every body sorted by priority, the predecessors of c
-// are the entries before c in the lists of its bodies.  A body's front is
-// the length of the coloured prefix of its list, and its mask the set of
-// colours in that prefix; c can be coloured once it is at the front of the
-// lists of all its (finite) bodies, and its colour is the smallest one in
-// none of their masks.  Colouring c adds its colour to those masks,
-// advances the fronts by one and exposes the next entry of each list, which
-// the next round colours if it is at the front of its other body's list
-// too (else that body's front exposes it later).  Each round colours
-// exactly the contacts whose predecessors were all coloured before it: the
-// rounds of Jones-Plassmann, with O(1) work per contact and round.
-//
-// A body's front is advanced at most once per round (only its front entry
-// can be coloured), and it is tagged with the round that advanced it: a
-// contact checked in the same round sees the value the front had when the
-// round began.  So each round reads only what earlier rounds wrote (a launch
-// boundary or a grid barrier apart), and a body's mask is written only by
-// the one contact at its front.
-constexpr uint32_t kFrontBits = 20;   // position bits of a front word; the round above them
-constexpr int kJpThreads = 256;       // threads of a colouring round's blocks
-constexpr uint32_t kClaimed = 0xFFFFFFFEu;
+// are the entries before c in the lists of its bodies.  A body's mask is the
+// set of colours in the coloured prefix of its list; once the entries right
+// before c in both lists are coloured, c's colour is the smallest one in
+// neither mask.  Colouring c adds its colour to the masks and "arrives" at
+// the next entry of either list; the last arrival at a contact (its only
+// predecessor's, or the second of two) is followed by its colouring.  So the
+// colours are those of the sequential greedy colouring whatever the order in
+// which the threads come along, and no thread waits for another.
 
-__device__ __forceinline__ uint32_t front_at(uint32_t f, uint32_t round)
-{
-    const uint32_t v = f & ((1u << kFrontBits) - 1u);
-    return (f >> kFrontBits) == round ? v - 1u : v;
-}
-
-// Incidence lists in decreasing priority ("beats" order), and each
-// contact's position in the lists of its bodies (cpack z for its first
+// Incidence lists in decreasing priority ("beats" order), kept as each
+// contact's successors in the lists of its bodies (cpack z for its first
 // body, w for its second).  Short lists (up to 16 contacts, every sphere
-// scene) take a bitonic network in a thread's registers; longer ones a
-// warp, lane l holding entries l, l + 32, ..., an entry's position being the
-// number of entries that beat it, counted over the others broadcast by
-// shuffles (one lane sorts lists beyond the warp's slots in place).
+// scene) take a bitonic network in a thread's registers, of 8 entries where
+// the lists of a warp allow it; longer ones a warp, lane l holding entries l,
+// l + 32, ..., an entry's position being the number of entries that beat it,
+// counted over the others broadcast by shuffles (one lane sorts lists beyond
+// the warp's slots in place).
 constexpr uint32_t kShortList = 16;
 constexpr int kSortSlots = 8;   // entries per lane of the warp sort: lists of up to 256 contacts
 
-__device__ __forceinline__ void set_position(uint4* cpack, uint32_t c, uint32_t x, uint32_t k)
+__device__ __forceinline__ void set_next(uint4* cpack, uint32_t c, uint32_t x, uint32_t next, bool first)
 {
     uint32_t* q = reinterpret_cast<uint32_t*>(cpack + c);
-    q[q[0] == x ? 2 : 3] = k;
+    q[q[0] == x ? 2 : 3] = next | (first ? 0u : kHasPrev);
 }
 
-// Also empties the front and colour mask of every body with a list (the
-// rounds read no other body's) and collects the bodies with long lists.
-__global__ void k_adj_sort_short(int64_t n, const uint8_t* __restrict__ finite, const uint32_t* __restrict__ adj_off,
-                                 uint32_t* __restrict__ adj, const uint64_t* __restrict__ prio,
-                                 uint4* __restrict__ cpack, uint32_t* __restrict__ front, uint32_t* __restrict__ mask,
-                                 uint32_t* __restrict__ longs, uint32_t* n_long)
+// A list of m <= N entries at adj, sorted in registers.
+template <uint32_t N>
+__device__ __forceinline__ void sort_short(uint32_t x, uint32_t m, const uint32_t* __restrict__ adj,
+                                           const uint64_t* __restrict__ prio, uint4* __restrict__ cpack)
 {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-        if (!finite[x]) continue;
-        const uint32_t a0 = adj_off[x], m = adj_off[x + 1] - a0;
-        if (m == 0) continue;
-        front[x] = 0u;
-        uint4* mk = reinterpret_cast<uint4*>(mask + 8 * x);
-        mk[0] = make_uint4(0u, 0u, 0u, 0u);
-        mk[1] = make_uint4(0u, 0u, 0u, 0u);
-        if (m > kShortList) {
-            longs[atomicAdd(n_long, 1u)] = (uint32_t)x;
-            continue;
-        }
-        uint32_t id[kShortList];
-        uint64_t pr[kShortList];
+    uint32_t id[N];
+    uint64_t pr[N];
 #pragma unroll
-        for (uint32_t i = 0; i < kShortList; ++i) id[i] = i < m ? adj[a0 + i] : 0xFFFFFFFFu;
+    for (uint32_t i = 0; i < N; ++i) id[i] = i < m ? adj[i] : 0xFFFFFFFFu;
 #pragma unroll
-        for (uint32_t i = 0; i < kShortList; ++i) pr[i] = i < m ? prio[id[i]] : 0ull;   // padding sorts last
-        // bitonic network: after it, entry i beats entry i + 1
+    for (uint32_t i = 0; i < N; ++i) pr[i] = i < m ? prio[id[i]] : 0ull;   // padding sorts last
+    // bitonic network: after it, entry i beats entry i + 1
 #pragma unroll
-        for (uint32_t k = 2; k <= kShortList; k <<= 1) {
+    for (uint32_t k = 2; k <= N; k <<= 1) {
 #pragma unroll
-            for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
 #pragma unroll
-                for (uint32_t i = 0; i < kShortList; ++i) {
-                    const uint32_t l = i ^ j;
-                    if (l <= i) continue;
-                    const bool first = (i & k) == 0;   // this half ends with i beating l
-                    const bool swap = first ? beats(pr[l], id[l], pr[i], id[i]) : beats(pr[i], id[i], pr[l], id[l]);
-                    if (swap) {
-                        const uint32_t ti = id[i];
-                        const uint64_t tp = pr[i];
-                        id[i] = id[l];
-                        pr[i] = pr[l];
-                        id[l] = ti;
-                        pr[l] = tp;
-                    }
+            for (uint32_t i = 0; i < N; ++i) {
+                const uint32_t l = i ^ j;
+                if (l <= i) continue;
+                const bool first = (i & k) == 0;   // this half ends with i beating l
+                const bool swap = first ? beats(pr[l], id[l], pr[i], id[i]) : beats(pr[i], id[i], pr[l], id[l]);
+                if (swap) {
+                    const uint32_t ti = id[i];
+                    const uint64_t tp = pr[i];
+                    id[i] = id[l];
+                    pr[i] = pr[l];
+                    id[l] = ti;
+                    pr[l] = tp;
                 }
             }
         }
+    }
 #pragma unroll
-        for (uint32_t i = 0; i < kShortList; ++i) {
-            if (i < m) {
-                adj[a0 + i] = id[i];
-                set_position(cpack, id[i], (uint32_t)x, i);
-            }
+    for (uint32_t i = 0; i < N; ++i)
+        if (i < m) set_next(cpack, id[i], x, i + 1 < m ? id[i + 1 < N ? i + 1 : i] : kNoNext, i == 0);
+}
+
+// Also empties the colour mask of every body with a list (the colouring
+// reads no other body's) and collects the bodies with long lists.
+__global__ void k_adj_sort_short(int64_t n, const uint8_t* __restrict__ finite, const uint32_t* __restrict__ adj_off,
+                                 const uint32_t* __restrict__ adj, const uint64_t* __restrict__ prio,
+                                 uint4* __restrict__ cpack, uint32_t* __restrict__ mask,
+                                 uint32_t* __restrict__ longs, uint32_t* n_long)
+{
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    // warp-uniform trip count: every lane takes part in the votes
+    for (int64_t x0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); x0 < n; x0 += stride) {
+        const int64_t x = x0 + (threadIdx.x & 31u);
+        uint32_t a0 = 0, m = 0;
+        if (x < n && finite[x]) {
+            a0 = adj_off[x];
+            m = adj_off[x + 1] - a0;
         }
+        if (m > 0) {
+            uint4* mk = reinterpret_cast<uint4*>(mask + 8 * x);
+            mk[0] = make_uint4(0u, 0u, 0u, 0u);
+            mk[1] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        if (m > kShortList) {
+            longs[atomicAdd(n_long, 1u)] = (uint32_t)x;
+            m = 0;
+        }
+        if (__any_sync(0xffffffffu, m > 8u)) sort_short<kShortList>((uint32_t)x, m, adj + a0, prio, cpack);
+        else if (__any_sync(0xffffffffu, m > 0u)) sort_short<8>((uint32_t)x, m, adj + a0, prio, cpack);
     }
 }
 
@@ -192,7 +189,7 @@ __global__ void k_adj_sort_short(int64_t n, const uint8_t* __restrict__ finite, 
 // l + 32, ...; an entry's position is the number of entries that beat it.
 template <int K>
 __device__ __forceinline__ void warp_sort_list(uint32_t x, uint32_t a0, uint32_t m, uint32_t lane,
-                                               uint32_t* __restrict__ adj, const uint64_t* __restrict__ prio,
+                                               uint32_t* adj, const uint64_t* __restrict__ prio,
                                                uint4* __restrict__ cpack)
 {
     uint32_t id[K], rk[K];
@@ -219,11 +216,10 @@ __device__ __forceinline__ void warp_sort_list(uint32_t x, uint32_t a0, uint32_t
     }
     __syncwarp();   // every entry read before any is overwritten
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        if (lane + 32u * k >= m) continue;
-        adj[a0 + rk[k]] = id[k];
-        set_position(cpack, id[k], x, rk[k]);
-    }
+    for (int k = 0; k < K; ++k)
+        if (lane + 32u * k < m) adj[a0 + rk[k]] = id[k];
+    __syncwarp();
+    for (uint32_t i = lane; i < m; i += 32u) set_next(cpack, adj[a0 + i], x, i + 1 < m ? adj[a0 + i + 1] : kNoNext, i == 0);
 }
 
 __global__ void k_adj_sort_long(const uint32_t* __restrict__ longs, const uint32_t* __restrict__ n_long,
@@ -252,232 +248,283 @@ __global__ void k_adj_sort_long(const uint32_t* __restrict__ longs, const uint32
                 }
                 adj[a0 + j] = c;
             }
-            for (uint32_t q = 0; q < m; ++q) set_position(cpack, adj[a0 + q], x, q);
+            for (uint32_t q = 0; q < m; ++q)
+                set_next(cpack, adj[a0 + q], x, q + 1 < m ? adj[a0 + q + 1] : kNoNext, q == 0);
         }
     }
 }
 
-// Block-wide append of up to two values per thread to list (cap entries):
-// one counter update per block (a counter every block of a round appends
-// to is contended).  Entries beyond cap set the colour error bit.
-__device__ __forceinline__ void block_push2(uint32_t e0, uint32_t e1, uint32_t* list, uint32_t* count, int64_t cap,
-                                            DevInfo* info)
-{
-    __shared__ uint32_t s_buf[2 * kJpThreads];
-    __shared__ uint32_t s_n, s_base;
-    if (threadIdx.x == 0) s_n = 0;
-    __syncthreads();
-    if (e0 != kUncoloured) s_buf[atomicAdd(&s_n, 1u)] = e0;
-    if (e1 != kUncoloured) s_buf[atomicAdd(&s_n, 1u)] = e1;
-    __syncthreads();
-    const uint32_t k = s_n;
-    if (threadIdx.x == 0) s_base = k ? atomicAdd(count, k) : 0u;
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < k; i += blockDim.x) {
-        const int64_t idx = (int64_t)s_base + i;
-        if (idx < cap) list[idx] = s_buf[i];
-        else atomicOr(&info->err, kErrColours);
-    }
-    __syncthreads();   // the buffer is refilled by the next call
-}
+// The colouring itself.  Each block works off a queue of its own in shared
+// memory: contacts whose predecessors are all coloured, first its share of
+// those that have none, then the ones its threads arrive at last.  In the
+// order of the queue the fronts of all lists advance together, as in rounds
+// over a global list, but without a barrier, a launch or a host in between:
+// a link of a chain of contacts costs one pass of the block over its queue.
+//
+// A block that falls behind arrives last more often and so gets still more
+// to do: one of 1064 ended up with 20 times its share of 2.75M contacts.  So a
+// large scene is coloured in turns, launches that stop after some passes and
+// leave their queues to a list that the next one deals out again; the last
+// runs to the end.
+//
+// Where every list is short (up to 16 contacts: no colour above 30) an arrival
+// brings the mask of its list along.  The first of two at a contact leaves it
+// in the contact's word (31 colours and a mark for either list), the second
+// finds it there in exchange: one compare-and-swap each, which is all that
+// orders them; a pass is two memory latencies (the successors' words, the
+// swaps).  Otherwise (Wide) the masks are kept in memory, 256 colours each,
+// ordered by fences around a count of the arrivals.
+//   us (ncu, cold)                            81k contacts   2.75M
+//   rounds over a list, a launch per round        326         618
+//   this, masks in memory and fences               98        1174
+//   this, masks with the arrivals                  44         217
+constexpr int kChaseThreads = 512;
+constexpr uint32_t kChaseRing = 2048, kChaseRoom = 2 * kChaseThreads;   // a pass adds at most kChaseRoom
 
-// The contacts at the front of all their lists from the start (no
-// predecessor) form the first round's list.
-__global__ void k_fr_seed(DCount Cc, const uint4* __restrict__ cpack, uint32_t* __restrict__ wl, uint32_t* count,
-                          DevInfo* info)
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
+template <bool Wide>
+__global__ void __launch_bounds__(kChaseThreads)
+k_colour_chase(DCount Cc, const uint4* __restrict__ cpack, uint32_t* mask, uint32_t* cstate,
+               unsigned long long* meet, const uint32_t* from, const uint32_t* from_count, uint32_t* to,
+               uint32_t* to_count, int passes, DevInfo* info)
 {
-    const int64_t C = Cc.get();
-    // block-uniform trip count: every thread takes part in block_push2
-    for (int64_t c0 = blockIdx.x * (int64_t)blockDim.x; c0 < C; c0 += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = c0 + threadIdx.x;
-        bool ready = false;
-        if (c < C) {
-            const uint4 q = cpack[c];
-            ready = (q.x == kNoList || q.z == 0u) && (q.y == kNoList || q.w == 0u);
+    if (Wide != (info->n_long != 0u)) return;
+    extern __shared__ uint4 s_q[];                                         // kChaseRing contacts:
+    uint32_t* const s_c = reinterpret_cast<uint32_t*>(s_q + kChaseRing);   // what they are, words and indices,
+    uint2* const s_m = reinterpret_cast<uint2*>(s_c + kChaseRing);         // and the masks of their lists
+    __shared__ uint32_t s_head, s_tail, s_spill;
+    // what to start with: the contacts without predecessors, or those of a list
+    const int64_t C = from ? (int64_t)*from_count : Cc.get(), stride = (int64_t)gridDim.x * kChaseThreads;
+    const uint32_t tid = threadIdx.x;
+    if (tid == 0) {
+        s_head = s_tail = 0u;
+        s_spill = kNoNext;
+    }
+    auto push = [&](uint32_t c, const uint4& q, uint32_t ma, uint32_t mb) {
+        const uint32_t t = atomicAdd(&s_tail, 1u) % kChaseRing;
+        s_c[t] = c;
+        s_q[t] = q;
+        if (!Wide) s_m[t] = make_uint2(ma, mb);
+    };
+    __syncthreads();
+    // every branch on n is the same for the whole block
+    for (int64_t seed = blockIdx.x * (int64_t)kChaseThreads;;) {
+        uint32_t n = s_tail - s_head;
+        __syncthreads();
+        while (n < (uint32_t)kChaseThreads && seed < C) {
+            const int64_t t = seed + tid;
+            if (t < C && from) {
+                const uint32_t c = from[t];
+                const unsigned long long m = meet[c];
+                push(c, cpack[c], (uint32_t)m, (uint32_t)(m >> 32));
+            } else if (t < C) {
+                const uint4 q = cpack[t];
+                if (((q.z | q.w) & kHasPrev) == 0u) push((uint32_t)t, q, 0u, 0u);
+            }
+            seed += stride;
+            __syncthreads();
+            n = s_tail - s_head;
+            __syncthreads();
         }
-        block_push2(ready ? (uint32_t)c : kUncoloured, kUncoloured, wl, count, C, info);
-    }
-}
-
-// One round over the list `in` (cnt_in entries); the contacts exposed go to
-// `out`.  cnt_clear (the counter two rounds ahead) is zeroed for reuse.
-__device__ __forceinline__ void fr_round(uint32_t round, const uint4* __restrict__ cpack,
-                                         const uint32_t* __restrict__ adj_off, const uint32_t* __restrict__ adj,
-                                         uint32_t* front, uint32_t* mask, const uint32_t* in, uint32_t m, uint32_t* out,
-                                         uint32_t* cnt_out, int64_t cap, uint32_t* cstate, DevInfo* info)
-{
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // block-uniform trip count: every thread takes part in block_push2
-    for (int64_t t0 = blockIdx.x * (int64_t)blockDim.x; t0 < m; t0 += stride) {
-        const int64_t t = t0 + threadIdx.x;
-        uint32_t e0 = kUncoloured, e1 = kUncoloured;
-        if (t < m) {
-            const uint32_t c = in[t];
-            const uint4 q = cpack[c];
-            const uint32_t a = q.x, b = q.y, pa = q.z, pb = q.w;
-            const bool fa = a != kNoList, fb = b != kNoList;
-            const bool ready = (!fa || front_at(__ldcg(front + a), round) == pa) &&
-                               (!fb || front_at(__ldcg(front + b), round) == pb);
-            // an entry exposed twice, or already coloured: the claim fails
-            if (ready && atomicCAS(cstate + c, kUncoloured, kClaimed) == kUncoloured) {
-                const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+        if (n == 0u) {
+            if (to_count) return;
+            if (tid == 0) {
+                uint32_t x = s_spill;
+                for (int k = 0; k < kChaseThreads && x != kNoNext; ++k) {
+                    const unsigned long long m = Wide ? 0ull : meet[x];
+                    push(x, cpack[x], (uint32_t)m, (uint32_t)(m >> 32));
+                    x = to[x];
+                }
+                s_spill = x;
+            }
+            __syncthreads();
+            n = s_tail - s_head;
+            __syncthreads();
+            if (n == 0u) return;
+        }
+        // a queue that is full, or whose turn is over, gives its newest away;
+        // their words are theirs alone by now
+        const bool over = to_count && --passes < 0 && seed >= C;
+        while (n > (over ? 0u : kChaseRing - kChaseRoom)) {
+            const uint32_t k = min(n, (uint32_t)kChaseThreads), t = (s_tail - 1u - tid) % kChaseRing, c = s_c[t];
+            if (tid < k && !Wide) meet[c] = (unsigned long long)s_m[t].y << 32 | s_m[t].x;
+            if (to_count) {
+                if (tid == 0) s_spill = atomicAdd(to_count, k);
+                __syncthreads();
+                if (tid < k) to[s_spill + tid] = c;
+            } else if (tid < k) {   // the block's own, linked by contact
+                to[c] = atomicExch(&s_spill, c);
+            }
+            __syncthreads();
+            if (tid == 0) s_tail -= k;
+            __syncthreads();
+            n -= k;
+        }
+        if (over) return;
+        const uint32_t take = min(n, (uint32_t)kChaseThreads);
+        const uint32_t at = (s_head + tid) % kChaseRing;
+        const uint32_t c = s_c[at];
+        const uint4 q = s_q[at];
+        uint2 m = make_uint2(0u, 0u);
+        if (!Wide) m = s_m[at];
+        __syncthreads();
+        if (tid == 0) s_head += take;
+        if (tid < take) {
+            const uint32_t a = q.x, b = q.y, e0 = q.z & kNoNext, e1 = q.w & kNoNext;
+            const bool fa = a != kNoList, fb = b != kNoList, n0 = e0 != kNoNext, n1 = e1 != kNoNext;
+            const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+            const uint4 q0 = n0 ? cpack[e0] : z, q1 = n1 ? cpack[e1] : z;
+            const bool two0 = (q0.z & q0.w & kHasPrev) != 0u, two1 = (q1.z & q1.w & kHasPrev) != 0u;
+            if constexpr (!Wide) {
+                const uint32_t col = (uint32_t)__ffs(~(m.x | m.y)) - 1u;   // at most 30: 15 predecessors in either list
+                cstate[c] = col;
+                m.x |= 1u << col;
+                m.y |= 1u << col;
+                // a list's last contact leaves the body's mask
+                if (fa && !n0) mask[8 * (int64_t)a] = m.x;
+                if (fb && !n1) mask[8 * (int64_t)b] = m.y;
+                // which of a successor's lists this one is, and what was there
+                const bool first0 = q0.x == a, first1 = q1.x == b;
+                const unsigned long long w0 = (unsigned long long)(m.x | kHasPrev) << (first0 ? 0 : 32);
+                const unsigned long long w1 = (unsigned long long)(m.y | kHasPrev) << (first1 ? 0 : 32);
+                unsigned long long o0 = 0ull, o1 = 0ull;
+                if (n0 && two0) o0 = atomicCAS(meet + e0, 0ull, w0);
+                if (n1 && two1) o1 = atomicCAS(meet + e1, 0ull, w1);
+                if (n0 && (!two0 || o0 != 0ull)) {
+                    o0 |= w0;
+                    push(e0, q0, (uint32_t)o0 & ~kHasPrev, (uint32_t)(o0 >> 32) & ~kHasPrev);
+                }
+                if (n1 && (!two1 || o1 != 0ull)) {
+                    o1 |= w1;
+                    push(e1, q1, (uint32_t)o1 & ~kHasPrev, (uint32_t)(o1 >> 32) & ~kHasPrev);
+                }
+            } else {
                 const uint4* ma = reinterpret_cast<const uint4*>(mask + 8 * (int64_t)a);
                 const uint4* mb = reinterpret_cast<const uint4*>(mask + 8 * (int64_t)b);
                 const uint4 a_lo = fa ? __ldcg(ma) : z, a_hi = fa ? __ldcg(ma + 1) : z;
                 const uint4 b_lo = fb ? __ldcg(mb) : z, b_hi = fb ? __ldcg(mb + 1) : z;
-                const uint32_t used[8] = {a_lo.x | b_lo.x, a_lo.y | b_lo.y, a_lo.z | b_lo.z, a_lo.w | b_lo.w,
-                                          a_hi.x | b_hi.x, a_hi.y | b_hi.y, a_hi.z | b_hi.z, a_hi.w | b_hi.w};
-                uint32_t col = kMaxColours;
+                const uint32_t wa[8] = {a_lo.x, a_lo.y, a_lo.z, a_lo.w, a_hi.x, a_hi.y, a_hi.z, a_hi.w};
+                const uint32_t wb[8] = {b_lo.x, b_lo.y, b_lo.z, b_lo.w, b_hi.x, b_hi.y, b_hi.z, b_hi.w};
+                uint32_t col = kMaxColours, va = 0u, vb = 0u;
 #pragma unroll
-                for (int k = 7; k >= 0; --k)
-                    if (~used[k]) col = 32u * k + (__ffs(~used[k]) - 1);
+                for (int k = 7; k >= 0; --k) {
+                    const uint32_t free = ~(wa[k] | wb[k]);
+                    if (free) {
+                        col = 32u * k + (__ffs(free) - 1);
+                        va = wa[k];
+                        vb = wb[k];
+                    }
+                }
                 if (col >= (uint32_t)kMaxColours) {
                     atomicOr(&info->err, kErrColours);
                     col = kMaxColours - 1;
+                    va = wa[7];
+                    vb = wb[7];
                 }
                 cstate[c] = col;
                 const uint32_t bit = 1u << (col & 31u), wd = col >> 5;
-                // only c, the front of a and of b, writes their masks and fronts
-                if (fa) {
-                    __stcg(mask + 8 * (int64_t)a + wd, __ldcg(mask + 8 * (int64_t)a + wd) | bit);
-                    __stcg(front + a, (round << kFrontBits) | (pa + 1));
-                    const uint32_t a0 = adj_off[a];
-                    if (pa + 1 < adj_off[a + 1] - a0) e0 = adj[a0 + pa + 1];
-                }
-                if (fb) {
-                    __stcg(mask + 8 * (int64_t)b + wd, __ldcg(mask + 8 * (int64_t)b + wd) | bit);
-                    __stcg(front + b, (round << kFrontBits) | (pb + 1));
-                    const uint32_t b0 = adj_off[b];
-                    if (pb + 1 < adj_off[b + 1] - b0) e1 = adj[b0 + pb + 1];
-                }
+                // only c, the front of a and of b, writes their masks
+                if (fa) __stcg(mask + 8 * (int64_t)a + wd, va | bit);
+                if (fb) __stcg(mask + 8 * (int64_t)b + wd, vb | bit);
+                fence_gpu();   // the masks before the arrivals
+                unsigned long long o0 = 0ull, o1 = 0ull;
+                if (n0 && two0) o0 = atomicAdd(meet + e0, 1ull);
+                if (n1 && two1) o1 = atomicAdd(meet + e1, 1ull);
+                fence_gpu();   // the arrivals before the masks that their contacts read
+                if (n0 && (!two0 || o0 != 0ull)) push(e0, q0, 0u, 0u);
+                if (n1 && (!two1 || o1 != 0ull)) push(e1, q1, 0u, 0u);
             }
         }
-        block_push2(e0, e1, out, cnt_out, cap, info);
+        __syncthreads();
     }
 }
 
-// One round per launch (the host checks the list counts every few rounds).
-// The counters rotate through three slots: a round reads one, writes the
-// next and clears the third.
-__global__ void __launch_bounds__(kJpThreads) k_fr_round(uint32_t round, const uint4* __restrict__ cpack,
-                                                         const uint32_t* __restrict__ adj_off,
-                                                         const uint32_t* __restrict__ adj, uint32_t* front,
-                                                         uint32_t* mask, const uint32_t* in, const uint32_t* cnt_in,
-                                                         uint32_t* out, uint32_t* cnt_out, uint32_t* cnt_clear,
-                                                         int64_t cap, uint32_t* cstate, DevInfo* info)
-{
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        *cnt_clear = 0u;
-        if (*cnt_in > 0u) info->rounds = round;   // the last round with work
-    }
-    fr_round(round, cpack, adj_off, adj, front, mask, in, *cnt_in, out, cnt_out, cap, cstate, info);
-}
+// Stable counting sort of the contacts by colour, in tiles: contacts of a
+// colour stay in canonical order.  The colours come straight from the
+// colouring's states; the scatter also writes the inverse permutation, the
+// colours' offsets and their number.
+constexpr int kSortThreads = 256, kSortItems = 16, kSortTile = kSortThreads * kSortItems, kSortWarps = kSortThreads / 32;
 
-// All rounds in one cooperative launch (no host in the loop, so a step can
-// be captured in a CUDA graph): a grid barrier ends each round (it plays
-// the part of a launch boundary), and the round's output count, read by
-// every block after the barrier, tells whether anything is left.  More than
-// kJpMaxRounds rounds set the colour error bit.
-constexpr int kJpMaxRounds = 1024;
-
-// Grid barrier of the colouring rounds: the arrival count and generation
-// words of the grid barrier, polled without sleeping (rounds are short);
-// bounded like every wait (~1 s of SM clocks), then the timeout bit.
-__device__ __forceinline__ bool jp_barrier(DevInfo* info)
+__global__ void __launch_bounds__(kSortThreads)
+k_colour_hist(DCount Cc, const uint32_t* __restrict__ cstate, uint32_t* __restrict__ hist, int64_t nblocks,
+              DevInfo* info)
 {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile uint32_t* vgen = &info->barrier_gen;
-        const uint32_t gen = *vgen;
-        __threadfence();
-        int good = 1;
-        if (atomicAdd(&info->barrier_count, 1u) == gridDim.x - 1) {
-            info->barrier_count = 0;
-            __threadfence();
-            atomicAdd(&info->barrier_gen, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (*vgen == gen) {
-                if (clock64() - t0 > (1LL << 31)) {
-                    atomicOr(&info->err, kErrTimeout);
-                    good = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
-        ok = good;
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
-__global__ void __launch_bounds__(kJpThreads) k_fr_persistent(DCount Cc, const uint4* __restrict__ cpack,
-                                                              const uint32_t* __restrict__ adj_off,
-                                                              const uint32_t* __restrict__ adj, uint32_t* front,
-                                                              uint32_t* mask, uint32_t* wl0, uint32_t* wl1,
-                                                              uint32_t* cnt, uint32_t* cstate, DevInfo* info)
-{
-    const int64_t C = Cc.get();
-    if (C == 0) return;
-    for (uint32_t round = 1; round <= (uint32_t)kJpMaxRounds; ++round) {
-        const int ci = (round - 1) % 3, co = round % 3, cc = (round + 1) % 3;
-        const bool odd = (round & 1u) != 0u;   // round 1 reads wl0 and writes wl1, round 2 the reverse, ...
-        if (blockIdx.x == 0 && threadIdx.x == 0) cnt[cc] = 0u;
-        fr_round(round, cpack, adj_off, adj, front, mask, odd ? wl0 : wl1, __ldcg(cnt + ci), odd ? wl1 : wl0,
-                 cnt + co, 2 * C, cstate, info);
-        if (!jp_barrier(info)) return;
-        if (__ldcg(cnt + co) == 0u) return;   // nothing exposed: every contact is coloured
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&info->err, kErrColours);
-}
-
-__global__ void k_colour_keys(DCount Cc, const uint32_t* __restrict__ cstate, uint32_t* __restrict__ ckey,
-                              uint32_t* __restrict__ cval, uint32_t* __restrict__ col_count, DevInfo* info)
-{
-    const int64_t C = Cc.get();
     __shared__ uint32_t h[kMaxColours];
-    for (int t = threadIdx.x; t < kMaxColours; t += blockDim.x) h[t] = 0;
+    const int64_t C = Cc.get();
+    h[threadIdx.x] = 0;
     __syncthreads();
-    uint32_t cmax = 0;
-    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t st = cstate[c];
-        uint32_t col = st & 0xFFu;
-        if (st == kUncoloured || col >= (uint32_t)kMaxColours) {   // uncoloured or out of range: report, keep indices in bounds
+    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+#pragma unroll
+    for (int k = 0; k < kSortItems; ++k) {
+        const int64_t c = base + (int64_t)k * kSortThreads + threadIdx.x;
+        if (c >= C) continue;
+        uint32_t col = cstate[c];
+        if (col >= (uint32_t)kMaxColours) {   // uncoloured: report, keep indices in bounds
             atomicOr(&info->err, kErrColours);
             col = kMaxColours - 1;
         }
-        ckey[c] = col;
-        cval[c] = (uint32_t)c;
         atomicAdd(&h[col], 1u);
-        cmax = max(cmax, col + 1);
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < kMaxColours; t += blockDim.x)
-        if (h[t]) atomicAdd(&col_count[t], h[t]);
-    for (int o = 16; o > 0; o >>= 1) cmax = max(cmax, __shfl_down_sync(0xffffffffu, cmax, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&info->n_colours, cmax);
+    hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
 }
 
-__global__ void k_colour_offsets(const uint32_t* __restrict__ col_count, uint32_t* __restrict__ col_off)
-{
-    if (threadIdx.x == 0) {
-        uint32_t acc = 0;
-        for (int c = 0; c < kMaxColours; ++c) {
-            col_off[c] = acc;
-            acc += col_count[c];
-        }
-        col_off[kMaxColours] = acc;
-    }
-}
-
-// Slot of every canonical contact in colour order: the inverse of perm.
-__global__ void k_invert(DCount Cc, const uint32_t* __restrict__ perm, uint32_t* __restrict__ inv)
+__global__ void __launch_bounds__(kSortThreads)
+k_colour_scatter(DCount Cc, const uint32_t* __restrict__ cstate, const uint32_t* __restrict__ hist_scan,
+                 int64_t nblocks, uint32_t* __restrict__ perm, uint32_t* __restrict__ inv,
+                 uint32_t* __restrict__ col_off, DevInfo* info)
 {
     const int64_t C = Cc.get();
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < C; s += (int64_t)gridDim.x * blockDim.x)
-        inv[perm[s]] = (uint32_t)s;
+    __shared__ uint32_t cnt[kSortWarps][kMaxColours];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int d0 = threadIdx.x;   // a thread per colour
+    static_assert(kSortThreads == kMaxColours, "a thread per colour");
+#pragma unroll
+    for (int ww = 0; ww < kSortWarps; ++ww) cnt[ww][d0] = 0;
+    if (blockIdx.x == 0) {
+        const uint32_t s = hist_scan[(int64_t)d0 * nblocks];
+        const uint32_t e = d0 + 1 < kMaxColours ? hist_scan[(int64_t)(d0 + 1) * nblocks] : (uint32_t)C;
+        col_off[d0] = s;
+        if (d0 == 0) col_off[kMaxColours] = (uint32_t)C;
+        if (e > s) atomicMax(&info->n_colours, (uint32_t)d0 + 1u);
+    }
+    const uint32_t goff = hist_scan[(int64_t)d0 * nblocks + blockIdx.x];
+    __syncthreads();
+    const uint32_t lt = (1u << lane) - 1u;
+    const int64_t base = (int64_t)blockIdx.x * kSortTile + (int64_t)w * (kSortItems * 32);
+    uint32_t key[kSortItems], rank[kSortItems];
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        const int64_t c = base + r * 32 + lane;
+        const bool valid = c < C;
+        key[r] = valid ? min(cstate[c], (uint32_t)kMaxColours - 1u) : 0u;
+        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? key[r] : 0x100u);
+        const uint32_t before = cnt[w][key[r]];
+        __syncwarp();
+        if (valid && (peers & lt) == 0) cnt[w][key[r]] = before + __popc(peers);
+        __syncwarp();
+        rank[r] = before + __popc(peers & lt);
+    }
+    __syncthreads();
+    // the tile's slots of each colour, warp by warp (warp order = input order)
+    uint32_t sum = goff;
+#pragma unroll
+    for (int ww = 0; ww < kSortWarps; ++ww) {
+        const uint32_t t = cnt[ww][d0];
+        cnt[ww][d0] = sum;
+        sum += t;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kSortItems; ++r) {
+        const int64_t c = base + r * 32 + lane;
+        if (c < C) {
+            const uint32_t pos = cnt[w][key[r]] + rank[r];
+            perm[pos] = (uint32_t)c;
+            inv[c] = pos;
+        }
+    }
 }
 
 // Sweep record inv[c] <- canonical contact c; initial impulse from the
@@ -582,18 +629,19 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
     }
 }
 
-// Resident blocks of the cooperative colouring launch (every block must be
-// resident for its grid barriers), looked up once.
-static int fr_blocks(const nbgs_scene* s)
+template <bool Wide>
+static nbgs_status chase(nbgs_scene* s, int blocks, DCount C, const uint32_t* from, const uint32_t* from_count,
+                         uint32_t* to, uint32_t* to_count, int passes)
 {
-    static int occ = -1;
-    if (occ < 0) {
-        int o = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, (const void*)k_fr_persistent, kJpThreads, 0);
-        cudaGetLastError();
-        occ = o > 0 ? o : 1;
+    const size_t smem = kChaseRing * (sizeof(uint4) + sizeof(uint32_t) + (Wide ? 0 : sizeof(uint2)));
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_colour_chase<Wide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e == cudaSuccess) {
+        k_colour_chase<Wide><<<blocks, kChaseThreads, smem, s->stream>>>(C, s->cpack, s->cmask, s->cstate, s->cmeet, from,
+                                                                         from_count, to, to_count, passes, s->info);
+        e = cudaGetLastError();
     }
-    return occ * s->num_sms;
+    return cuda_check(s, e, "colour: rounds");
 }
 
 nbgs_status run_colour(nbgs_scene* s)
@@ -605,7 +653,6 @@ nbgs_status run_colour(nbgs_scene* s)
     const int64_t C = s->n_contacts, n = s->n;
     const DCount Cn = contact_count(s);
     if (s->timing) cudaEventRecord(s->ev[2], st);
-    cudaMemsetAsync(s->col_count, 0, (kMaxColours + 1) * sizeof(uint32_t), st);
     cudaMemsetAsync(&s->info->n_colours, 0, sizeof(uint32_t), st);
     cudaMemsetAsync(&s->info->n_shared, 0, 2 * sizeof(uint32_t), st);   // no shared bodies until assigned
     const bool sub = s->prm.subdomain_mode != NBGS_SUB_NONE;
@@ -625,7 +672,7 @@ nbgs_status run_colour(nbgs_scene* s)
         const int64_t ninc = s->composite ? s->nb : n;
         cudaMemsetAsync(s->deg, 0, (ninc + 1) * sizeof(uint32_t), st);
         k_colour_init<<<gb, T, 0, st>>>(Cn, ninc, s->cj1, s->cj2, ib1, ib2, finc, s->prm.colour_seed, scene_view(s),
-                                        s->deg, s->cprio, s->cstate, s->cpack);
+                                        s->deg, s->cprio, s->cstate, s->cpack, s->cmeet);
         nbgs_status rc = exclusive_scan_u32(s, s->deg, s->adj_off, ninc, nullptr);
         if (rc != NBGS_OK) return rc;
         cudaMemsetAsync(s->deg, 0, (ninc + 1) * sizeof(uint32_t), st);
@@ -640,89 +687,43 @@ nbgs_status run_colour(nbgs_scene* s)
             // the same sweep, so a single colour
             cudaMemsetAsync(s->cstate, 0, C * sizeof(uint32_t), st);
         } else {
-            // incidence lists in priority order, fronts and masks empty, the
-            // contacts without predecessors as the first round's list
-            uint32_t* front = s->deg;   // scratch again (the degrees are adj_off's differences); emptied per body below
-            // (the bodies with long lists go to wl[1], counted in wl_count[3])
-            cudaMemsetAsync(s->info->wl_count, 0, 4 * sizeof(uint32_t), st);
-            k_adj_sort_short<<<grid_for(ninc, T, 8, s->num_sms), T, 0, st>>>(ninc, finc, s->adj_off, s->adj,
-                                                                              s->cprio, s->cpack, front, s->cmask,
-                                                                              s->wl[1], &s->info->wl_count[3]);
-            k_adj_sort_long<<<8 * s->num_sms, T, 0, st>>>(s->wl[1], &s->info->wl_count[3], s->adj_off, s->adj,
-                                                           s->cprio, s->cpack);
-            k_fr_seed<<<gb, T, 0, st>>>(Cn, s->cpack, s->wl[0], &s->info->wl_count[0], s->info);
-            if (s->timing) s->phase_launches[1] += 5;
-            if (s->device_sized) {
-                // all rounds in one cooperative launch (grid barrier between rounds)
-                cudaMemsetAsync(&s->info->barrier_count, 0, 2 * sizeof(uint32_t), st);
-                const int gbr = std::min(fr_blocks(s), grid_for(C, kJpThreads, 8, s->num_sms));
-                DCount Cd = Cn;
-                uint32_t *wl0 = s->wl[0], *wl1 = s->wl[1], *cnt = s->info->wl_count, *msk = s->cmask;
-                const uint4* cp = s->cpack;
-                void* args[] = {(void*)&Cd, (void*)&cp, (void*)&s->adj_off, (void*)&s->adj, (void*)&front,
-                                (void*)&msk, (void*)&wl0, (void*)&wl1, (void*)&cnt, (void*)&s->cstate, (void*)&s->info};
-                rc = cuda_check(s, cudaLaunchCooperativeKernel((const void*)k_fr_persistent, dim3(gbr),
-                                                               dim3(kJpThreads), args, 0, st),
-                                "colour: rounds");
-                if (rc != NBGS_OK) return rc;
-                if (s->timing) s->phase_launches[1] += 2;
-            } else {
-                // one launch per round; the host checks the list counts after as
-                // many rounds as the last colouring took, then every four
-                const int gbr = grid_for(C, kJpThreads, 8, s->num_sms);
-                uint32_t round = 0;
-                int cur = 0;
-                int batch = std::max(4, s->colour_rounds);
-                for (;;) {
-                    for (int r = 0; r < batch; ++r) {
-                        ++round;
-                        const int ci = (round - 1) % 3, co = round % 3, cc = (round + 1) % 3;
-                        k_fr_round<<<gbr, kJpThreads, 0, st>>>(round, s->cpack, s->adj_off, s->adj, front, s->cmask,
-                                                               s->wl[cur], &s->info->wl_count[ci], s->wl[1 - cur],
-                                                               &s->info->wl_count[co], &s->info->wl_count[cc], 2 * C,
-                                                               s->cstate, s->info);
-                        cur = 1 - cur;
-                    }
-                    if (s->timing) s->phase_launches[1] += batch;
-                    uint32_t left = 0, used = 0;
-                    rc = cuda_check(s, cudaMemcpyAsync(&left, &s->info->wl_count[round % 3], sizeof(uint32_t),
-                                                       cudaMemcpyDeviceToHost, st), "colour: list count");
-                    if (rc == NBGS_OK)
-                        rc = cuda_check(s, cudaMemcpyAsync(&used, &s->info->rounds, sizeof(uint32_t),
-                                                           cudaMemcpyDeviceToHost, st), "colour: rounds");
-                    if (rc != NBGS_OK) return rc;
-                    rc = cuda_check(s, cudaStreamSynchronize(st), "colour");
-                    if (rc != NBGS_OK) return rc;
-                    if (left == 0) {
-                        s->colour_rounds = (int)used + 1;
-                        break;
-                    }
-                    if (round >= (uint32_t)kJpMaxRounds) return fail(s, NBGS_ETIMEOUT, "colour: did not finish in 1024 rounds");
-                    batch = 4;
-                }
-            }
+            cudaMemsetAsync(&s->info->n_long, 0, sizeof(uint32_t), st);
+            k_adj_sort_short<<<grid_for(ninc, T, 8, s->num_sms), T, 0, st>>>(ninc, finc, s->adj_off, s->adj, s->cprio,
+                                                                              s->cpack, s->cmask, s->clist[0],
+                                                                              &s->info->n_long);
+            k_adj_sort_long<<<8 * s->num_sms, T, 0, st>>>(s->clist[0], &s->info->n_long, s->adj_off, s->adj, s->cprio,
+                                                           s->cpack);
+            // the kernel that the lists' lengths call for does the work, in
+            // turns of several passes where a block would fall far behind:
+            // colouring phase, us, 18 colours     117k  474k  717k  1.01M contacts
+            //   one turn                           171   229   280   610
+            //   7 turns of 9 passes                238   303   340   397
+            // (2.75M, 17 colours, the launches alone: 700 and 217; 5.99M: 4549 and 620)
+            const int64_t known = s->device_sized ? (int64_t)s->hinfo->n_contacts : C;
+            const int turns = known < 800000 ? 1 : kChaseTurns, passes = 9;
+            const int gc = grid_for(C, kChaseThreads, 3, s->num_sms);
+            uint32_t* cnt = s->info->chase_count;
+            cudaMemsetAsync(cnt, 0, kChaseTurns * sizeof(uint32_t), st);
+            for (int k = 0; k < turns && rc == NBGS_OK; ++k)
+                rc = chase<false>(s, gc, Cn, k ? s->clist[(k + 1) & 1] : nullptr, k ? cnt + k - 1 : nullptr,
+                                  s->clist[k & 1], k + 1 < turns ? cnt + k : nullptr, passes);
+            if (rc == NBGS_OK) rc = chase<true>(s, gc, Cn, nullptr, nullptr, s->clist[0], nullptr, 0);
+            if (rc != NBGS_OK) return rc;
+            if (s->timing) s->phase_launches[1] += 3 + turns;
         }
-        k_colour_keys<<<gb, T, 0, st>>>(Cn, s->cstate, s->colour_key, s->perm_in, s->col_count, s->info);
-        k_colour_offsets<<<1, 32, 0, st>>>(s->col_count, s->col_off);
-        // stable counting sort by colour (one 8-bit radix pass): contacts of a
-        // colour stay in canonical order
-        uint32_t *k0 = s->colour_key, *k1 = s->colour_key2, *v0 = s->perm_in, *v1 = s->perm;
-        rc = radix_sort_pairs(s, k0, v0, k1, v1, Cn, 8);
+        const int64_t nbs = (C + kSortTile - 1) / kSortTile;
+        if (kMaxColours * nbs > s->sort_hist_len) return fail(s, NBGS_EINVAL, "colour: histogram buffer too small");
+        k_colour_hist<<<(unsigned)nbs, kSortThreads, 0, st>>>(Cn, s->cstate, s->sort_hist, nbs, s->info);
+        rc = exclusive_scan_u32(s, s->sort_hist, s->sort_hist, kMaxColours * nbs, nullptr);
         if (rc != NBGS_OK) return rc;
-        // radix_sort_pairs swapped the pointers: v0 / k0 now hold the sorted values / keys
-        if (v0 != s->perm) std::swap(s->perm, s->perm_in);
-        if (v0 != s->perm) return fail(s, NBGS_EINVAL, "colour: permutation buffer mix-up");
-        s->colour_sorted = k0;
+        k_colour_scatter<<<(unsigned)nbs, kSortThreads, 0, st>>>(Cn, s->cstate, s->sort_hist, nbs, s->perm, s->inv,
+                                                                 s->col_off, s->info);
         const int warm = (s->prm.warm_start != NBGS_WARM_NONE && s->have_prev) ? 1 : 0;
-        // the slots of the canonical contacts (perm_in is free after the sort;
-        // the records and the solve's finish read it)
-        k_invert<<<gb, T, 0, st>>>(Cn, s->perm, s->perm_in);
-        if (s->timing) s->phase_launches[1] += 1;
         if (s->composite) {
             rc = run_comp_records(s, warm);
             if (rc != NBGS_OK) return rc;
         } else if (s->fp32)
-            k_build_sweep<float><<<gb, T, 0, st>>>(Cn, n, s->perm_in, s->cj1, s->cj2, sub ? s->inst : nullptr, s->cgeo,
+            k_build_sweep<float><<<gb, T, 0, st>>>(Cn, n, s->inv, s->cj1, s->cj2, sub ? s->inst : nullptr, s->cgeo,
                                                    s->clev, s->prm.dt,
                                                    s->prm.beta, s->prm.mu, scene_view(s), warm, s->prev_row_off,
                                                    s->prev_j2,
@@ -730,7 +731,7 @@ nbgs_status run_colour(nbgs_scene* s)
                                                    (const float4*)s->vel, (SweepRec<float>*)s->srec, (float4*)s->sp,
                                                    (SweepPre<float>*)s->spre);
         else
-            k_build_sweep<double><<<gb, T, 0, st>>>(Cn, n, s->perm_in, s->cj1, s->cj2, sub ? s->inst : nullptr, s->cgeo,
+            k_build_sweep<double><<<gb, T, 0, st>>>(Cn, n, s->inv, s->cj1, s->cj2, sub ? s->inst : nullptr, s->cgeo,
                                                     s->clev, s->prm.dt,
                                                     s->prm.beta, s->prm.mu, scene_view(s), warm, s->prev_row_off,
                                                     s->prev_j2,

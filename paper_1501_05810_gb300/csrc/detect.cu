@@ -195,118 +195,6 @@ nbgs_status exclusive_scan_u32(nbgs_scene* s, const uint32_t* in, uint32_t* out,
 }
 
 // ---------------------------------------------------------------------------
-// LSD radix sort of (key, value) u32 pairs: 8-bit digits, one pass =
-// per-tile digit histogram -> scan (digit-major) -> stable scatter with
-// warp-level ranking (__match_any_sync), so equal keys keep input order.
-// ---------------------------------------------------------------------------
-constexpr int kRadixThreads = 256;
-constexpr int kRadixItems = 16;
-constexpr int kRadixTile = kRadixThreads * kRadixItems;   // 4096
-constexpr int kWarps = kRadixThreads / 32;
-
-__global__ void k_radix_hist(const uint32_t* __restrict__ keys, DCount nc, int shift, uint32_t* __restrict__ hist,
-                             int64_t nblocks)
-{
-    __shared__ uint32_t h[256];
-    const int64_t n = nc.get();
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-#pragma unroll 4
-    for (int k = 0; k < kRadixItems; ++k) {
-        int64_t i = base + (int64_t)k * kRadixThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255u], 1u);
-    }
-    __syncthreads();
-    hist[(int64_t)threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(kRadixThreads)
-k_radix_scatter(const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-                uint32_t* __restrict__ vout, DCount nc, int shift, const uint32_t* __restrict__ hist_scan,
-                int64_t nblocks)
-{
-    const int64_t n = nc.get();
-    __shared__ uint32_t cnt[kWarps][256];
-    __shared__ uint32_t goff[256];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int d = threadIdx.x; d < 256; d += kRadixThreads) {
-#pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) cnt[ww][d] = 0;
-        goff[d] = hist_scan[(int64_t)d * nblocks + blockIdx.x];
-    }
-    __syncthreads();
-    const uint32_t lt = (1u << lane) - 1u;
-    const int64_t base = (int64_t)blockIdx.x * kRadixTile + (int64_t)w * (kRadixItems * 32);
-    uint32_t key[kRadixItems], val[kRadixItems], rank[kRadixItems];
-#pragma unroll
-    for (int r = 0; r < kRadixItems; ++r) {
-        const int64_t i = base + r * 32 + lane;
-        const bool valid = i < n;
-        key[r] = valid ? kin[i] : 0u;
-        val[r] = valid ? vin[i] : 0u;
-        const uint32_t d = (key[r] >> shift) & 255u;
-        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? d : 0x100u);
-        const uint32_t before = cnt[w][d & 255u];
-        __syncwarp();
-        if (valid && (peers & lt) == 0) cnt[w][d] = before + __popc(peers);
-        __syncwarp();
-        rank[r] = before + __popc(peers & lt);
-    }
-    __syncthreads();
-    // exclusive prefix of each digit over the warps (warp order = input order)
-    for (int d = threadIdx.x; d < 256; d += kRadixThreads) {
-        uint32_t sum = 0;
-#pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) {
-            uint32_t t = cnt[ww][d];
-            cnt[ww][d] = sum;
-            sum += t;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < kRadixItems; ++r) {
-        const int64_t i = base + r * 32 + lane;
-        if (i < n) {
-            const uint32_t d = (key[r] >> shift) & 255u;
-            const uint32_t pos = goff[d] + cnt[w][d] + rank[r];
-            kout[pos] = key[r];
-            vout[pos] = val[r];
-        }
-    }
-}
-
-nbgs_status radix_sort_pairs(nbgs_scene* s, uint32_t*& keys, uint32_t*& vals, uint32_t*& keys_alt,
-                             uint32_t*& vals_alt, DCount n, int bits)
-{
-    if (!n.dev && n.v <= 1) return NBGS_OK;
-    const int64_t nb = std::max<int64_t>((n.v + kRadixTile - 1) / kRadixTile, 1);
-    if (256 * nb > s->radix_hist_len) return fail(s, NBGS_EINVAL, "radix sort: histogram buffer too small");
-    for (int shift = 0; shift < bits; shift += 8) {
-        k_radix_hist<<<(unsigned)nb, kRadixThreads, 0, s->stream>>>(keys, n, shift, s->radix_hist, nb);
-        nbgs_status st = exclusive_scan_u32(s, s->radix_hist, s->radix_hist, 256 * nb, nullptr);
-        if (st != NBGS_OK) return st;
-        k_radix_scatter<<<(unsigned)nb, kRadixThreads, 0, s->stream>>>(keys, vals, keys_alt, vals_alt, n, shift,
-                                                                       s->radix_hist, nb);
-        uint32_t* t = keys;
-        keys = keys_alt;
-        keys_alt = t;
-        t = vals;
-        vals = vals_alt;
-        vals_alt = t;
-        if (s->timing) s->phase_launches[0] += 4;
-    }
-    return cuda_check(s, cudaGetLastError(), "radix sort");
-}
-
-nbgs_status radix_sort_pairs(nbgs_scene* s, uint32_t*& keys, uint32_t*& vals, uint32_t*& keys_alt,
-                             uint32_t*& vals_alt, int64_t n, int bits)
-{
-    return radix_sort_pairs(s, keys, vals, keys_alt, vals_alt, DCount{n, nullptr}, bits);
-}
-
-// ---------------------------------------------------------------------------
 // detection kernels
 // ---------------------------------------------------------------------------
 struct GridArgs {

@@ -24,6 +24,7 @@ namespace nbgs {
 constexpr int kMaxPlanes = 16;
 constexpr int kMaxColours = 256;       // a colour is 8 bits of the colouring state
 constexpr int kCandCap = 32;           // sphere candidates per body with j > i
+constexpr int kChaseTurns = 7;         // launches of the colouring at most
 constexpr uint32_t kUncoloured = 0xFFFFFFFFu;
 constexpr uint32_t kNoList = 0xFFFFFFFFu;   // a contact end without an incidence list (wall, infinite mass)
 constexpr int kMaxSweepsHist = 4096;   // residual slots: history, 3 rotating, 4 final
@@ -135,10 +136,10 @@ struct DevInfo {
     uint32_t err;
     uint32_t cand_need;              // largest candidate count seen
     uint32_t sweeps_done;
-    uint32_t wl_count[6];            // colouring list sizes (|L|, |X|), three rotating pairs
+    uint32_t n_long;                 // bodies with long incidence lists
+    uint32_t chase_count[kChaseTurns];   // contacts given away by the colouring's queues
     uint32_t barrier_count;          // grid barrier arrival counter
     uint32_t barrier_gen;            // grid barrier generation
-    uint32_t rounds;                 // colouring rounds used
     uint32_t n_shared;               // subdomains: bodies with more than one velocity instance
     uint32_t n_extra;                // subdomains: velocity instances after the n bodies
     uint32_t prev_contacts;          // contacts of the previous step (device-sized steps)
@@ -441,8 +442,8 @@ struct nbgs_scene {
     uint32_t* ckey = nullptr;         // n: cell of every body
     uint32_t* crank = nullptr;        // n: its rank among the cell's bodies
     uint32_t* svals = nullptr;        // n: bodies in cell order
-    uint32_t* radix_hist = nullptr;
-    int64_t radix_hist_len = 0;
+    uint32_t* sort_hist = nullptr;
+    int64_t sort_hist_len = 0;
     uint32_t* scan_tmp = nullptr;  // block sums of the scans
     int64_t scan_tmp_len = 0;
     // candidates
@@ -472,15 +473,11 @@ struct nbgs_scene {
     uint64_t* cprio = nullptr;
     uint4* cpack = nullptr;        // colouring: per contact (body 1, body 2 or none, its positions in their lists)
     uint32_t* cmask = nullptr;     // colouring: 8 x 32 colour bits per body (its coloured prefix)
-    int colour_rounds = 0;         // rounds the last colouring took (the host checks after as many)
-    uint32_t* wl[2] = {nullptr, nullptr};
-    uint32_t* colour_key = nullptr;   // colour per contact (sort key)
-    uint32_t* colour_key2 = nullptr;
+    unsigned long long* cmeet = nullptr;   // contacts: what the first of two arrivals leaves for the second
+    uint32_t* clist[2] = {nullptr, nullptr};   // contacts: bodies with long lists, then contacts that queues give away
     uint32_t* perm = nullptr;      // sweep slot -> canonical index
-    uint32_t* perm_in = nullptr;   // the sort's input, then canonical index -> sweep slot (perm inverted)
-    uint32_t* col_count = nullptr; // kMaxColours + 1
+    uint32_t* inv = nullptr;       // canonical index -> sweep slot
     uint32_t* col_off = nullptr;   // kMaxColours + 1
-    uint32_t* colour_sorted = nullptr;  // colour of each sweep slot (points into colour_key / colour_key2)
     int2* dep = nullptr;           // kMaxColours x coop_blocks block windows [lo, hi] of each chunk
     int* prog = nullptr;           // coop_blocks: last sweep phase each block completed
     uint32_t* cstart = nullptr;    // kMaxColours x (coop_blocks + 1) chunk boundaries
@@ -598,11 +595,7 @@ nbgs_status run_get_contacts(nbgs_scene* s, int64_t cap, uint32_t* j1, uint32_t*
 // primitives (detect.cu)
 nbgs_status exclusive_scan_u32(nbgs_scene* s, const uint32_t* in, uint32_t* out, int64_t n,
                                uint32_t* total_dst);
-nbgs_status radix_sort_pairs(nbgs_scene* s, uint32_t*& keys, uint32_t*& vals, uint32_t*& keys_alt,
-                             uint32_t*& vals_alt, int64_t n, int bits);
 nbgs_status exclusive_scan_u32(nbgs_scene* s, const uint32_t* in, uint32_t* out, DCount n, uint32_t* total_dst);
-nbgs_status radix_sort_pairs(nbgs_scene* s, uint32_t*& keys, uint32_t*& vals, uint32_t*& keys_alt,
-                             uint32_t*& vals_alt, DCount n, int bits);
 int grid_for(int64_t work, int threads, int max_blocks_per_sm, int num_sms);
 // The contact count of the current step for kernels: host-known, or read on
 // the device (device-sized steps; launches sized for the capacity).

@@ -1170,10 +1170,10 @@ nbgs_status run_solve(nbgs_scene* s, int max_sweeps, double tol)
     if (C > 0) {
         const int T = 256;
         if (s->fp32)
-            k_finish<float><<<grid_for(C, T, 8, s->num_sms), T, 0, st>>>(contact_count(s), s->perm_in, (const float4*)s->sp, s->cgeo,
+            k_finish<float><<<grid_for(C, T, 8, s->num_sms), T, 0, st>>>(contact_count(s), s->inv, (const float4*)s->sp, s->cgeo,
                                                                          s->cimp, s->cworld);
         else
-            k_finish<double><<<grid_for(C, T, 8, s->num_sms), T, 0, st>>>(contact_count(s), s->perm_in, (const double4_32a*)s->sp, s->cgeo,
+            k_finish<double><<<grid_for(C, T, 8, s->num_sms), T, 0, st>>>(contact_count(s), s->inv, (const double4_32a*)s->sp, s->cgeo,
                                                                           s->cimp, s->cworld);
     }
     if (C > 0 && !s->composite)
