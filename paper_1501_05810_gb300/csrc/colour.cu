@@ -699,8 +699,7 @@ nbgs_status run_colour(nbgs_scene* s)
             //   one turn                           171   229   280   610
             //   7 turns of 9 passes                238   303   340   397
             // (2.75M, 17 colours, the launches alone: 700 and 217; 5.99M: 4549 and 620)
-            const int64_t known = s->device_sized ? (int64_t)s->hinfo->n_contacts : C;
-            const int turns = known < 800000 ? 1 : kChaseTurns, passes = 9;
+            const int turns = known_contacts(s) < 800000 ? 1 : kChaseTurns, passes = 9;
             const int gc = grid_for(C, kChaseThreads, 3, s->num_sms);
             uint32_t* cnt = s->info->chase_count;
             cudaMemsetAsync(cnt, 0, kChaseTurns * sizeof(uint32_t), st);

@@ -10,9 +10,9 @@
 //   k_narrow        per body: bodies in its own and the 13 cells ahead whose
 //                   hulls intersect; wall hull tests
 //   scan            contacts per body -> CSR offsets by j1
-//   k_write         canonical contact records (n, xi, lever lengths), partners
-//                   in ascending order,
-//                   for sphere-sphere and sphere-wall pairs, eq. (contactpos)
+//   k_write_ends    canonical contacts, partners in ascending order
+//   k_contact_geometry  their normals, gaps and lever lengths, for
+//                   sphere-sphere and sphere-wall pairs, eq. (contactpos)
 #include <algorithm>
 #include <cmath>
 #include <utility>
@@ -228,14 +228,18 @@ __device__ __forceinline__ double norm_exact(double x, double y, double z)
 // al., Handbook of Floating-Point Arithmetic, the chapter on division with
 // an FMA).  The theorem excludes underflow: tiny numerators take the division
 // itself, as does the caller for a tiny or huge b; a zero (every pair inside a
-// lattice plane has one) is its own quotient, b being positive.
+// lattice plane has one) is its own quotient, b being positive, and does not
+// take its warp through the division (three of them made 93 FP64 instructions
+// of a dense lattice's 45 a pair).
 __device__ __forceinline__ double div_by(double a, double b, double y)
 {
     const uint32_t e = (uint32_t)__double2hiint(a) & 0x7FFFFFFFu;
-    if (e < 0x07B00000u) return (e | (uint32_t)__double2loint(a)) == 0u ? a : xdiv(a, b);   // |a| < 2^-900
+    const bool zero = (e | (uint32_t)__double2loint(a)) == 0u;
+    if (e < 0x07B00000u && !zero) return xdiv(a, b);   // |a| < 2^-900
     const double q = __dmul_rn(a, y);
     const double r = __fma_rn(-q, b, a);
-    return __fma_rn(r, y, q);
+    const double v = __fma_rn(r, y, q);
+    return zero ? a : v;   // keeps its sign
 }
 
 // Sphere pair geometry of eq. (contactpos) from the centre difference
@@ -246,7 +250,8 @@ __device__ __forceinline__ double div_by(double a, double b, double y)
 __device__ __forceinline__ double pair_normal(double dx, double dy, double dz, double n[3])
 {
     const double d = norm_exact(dx, dy, dz);
-    if (d > 0x1p-1000 && d < 0x1p1000) {
+    // 2^-1000 <= d < 2^1000, by its upper word (d is not negative)
+    if ((uint32_t)__double2hiint(d) - 0x01700000u < 0x7D000000u) {
         const double y = __drcp_rn(d);
         n[0] = div_by(dx, d, y);
         n[1] = div_by(dy, d, y);
@@ -515,7 +520,9 @@ __global__ void k_cell_scatter(int64_t n, const uint32_t* __restrict__ keys, con
 // Minimum-image difference a - b along one axis (periodic: |d| <= L/2).
 __device__ __forceinline__ double min_image(double d, int periodic, double L)
 {
-    if (periodic) {
+    // |d| <= L / 2 is read off the upper words for all but the pairs across a
+    // face: FP64 comparisons would cost as much as the arithmetic
+    if (periodic && ((uint32_t)__double2hiint(d) & 0x7FFFFFFFu) >= (uint32_t)__double2hiint(L) - 0x00100000u) {
         const double half = xmul(0.5, L);
         if (d > half) d = xsub(d, L);
         else if (d < -half) d = xadd(d, L);
@@ -808,34 +815,27 @@ k_narrow(int64_t n, const uint32_t* __restrict__ svals, const double4_32a* __res
     }
 }
 
-// Canonical contact records: row i of the CSR holds (i, j) for the sorted
-// partners j, then the walls in the order they were added.  A warp takes 32
-// bodies (in cell order) and spreads their sphere pairs over its lanes, one
-// pair per lane and pass, so that the FP64 chains of a row run side by side;
-// the walls of a body stay with its own lane.
-__global__ void k_write_contacts(int64_t n, int64_t ccap, const uint32_t* __restrict__ svals,
-                                 const double4_32a* __restrict__ pos_r,
-                                 const uint32_t* __restrict__ cand, const uint32_t* __restrict__ pair_cnt,
-                                 const uint32_t* __restrict__ wall_mask, const uint32_t* __restrict__ row_off, GridArgs g, Planes planes, SceneView V,
-                                 uint32_t* __restrict__ cj1, uint32_t* __restrict__ cj2, double4_32a* __restrict__ cgeo,
-                                 double2* __restrict__ clev)
+// The contacts' bodies: row i of the CSR holds (i, j) for the sorted partners
+// j, then the walls in the order they were added.  A warp takes 32 bodies (in
+// cell order) and spreads their sphere pairs over its lanes, one pair per
+// lane and pass; the walls of a body stay with its own lane.
+__global__ void k_write_ends(int64_t n, int64_t ccap, const uint32_t* __restrict__ svals,
+                             const uint32_t* __restrict__ cand, const uint32_t* __restrict__ pair_cnt,
+                             const uint32_t* __restrict__ wall_mask, const uint32_t* __restrict__ row_off,
+                             int nplanes, int ncones, SceneView V, uint32_t* __restrict__ cj1,
+                             uint32_t* __restrict__ cj2)
 {
-    const double L0 = g.hi[0] - g.lo[0], L1 = g.hi[1] - g.lo[1], L2 = g.hi[2] - g.lo[2];
     const int lane = threadIdx.x & 31;
     const int64_t wstride = (int64_t)gridDim.x * blockDim.x;
     // warp-uniform trip count: every lane takes part in the shuffles
     for (int64_t s0 = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); s0 < n; s0 += wstride) {
         const int64_t s = s0 + lane;
         uint32_t i = 0, ns = 0, wm = 0, ro = 0;
-        double4_32a pi = make_double4_32a(0.0, 0.0, 0.0, 0.0);
         if (s < n) {
             i = svals[s];
             ns = min(pair_cnt[i], (uint32_t)kCandCap);
             wm = wall_mask[i];
-            if ((ns | wm) != 0) {
-                pi = pos_r[i];
-                ro = row_off[i];
-            }
+            if ((ns | wm) != 0) ro = row_off[i];
         }
         uint32_t pre = ns;   // inclusive prefix of the pair counts over the lanes
 #pragma unroll
@@ -858,11 +858,6 @@ __global__ void k_write_contacts(int64_t n, int64_t ccap, const uint32_t* __rest
             const uint32_t ro_o = __shfl_sync(0xffffffffu, ro, own);
             const uint32_t end_o = __shfl_sync(0xffffffffu, pre, own);
             const uint32_t ns_o = __shfl_sync(0xffffffffu, ns, own);
-            double4_32a po;
-            po.x = __shfl_sync(0xffffffffu, pi.x, own);
-            po.y = __shfl_sync(0xffffffffu, pi.y, own);
-            po.z = __shfl_sync(0xffffffffu, pi.z, own);
-            po.w = __shfl_sync(0xffffffffu, pi.w, own);
             if (t >= total) continue;
             const uint32_t k = t - (end_o - ns_o);
             // the list holds its pairs as they were found: contact k goes to
@@ -873,50 +868,73 @@ __global__ void k_write_contacts(int64_t n, int64_t ccap, const uint32_t* __rest
             for (uint32_t m = 0; m < ns_o; ++m) rank += list[m] < j ? 1u : 0u;
             const int64_t idx = (int64_t)ro_o + rank;
             if (idx >= ccap) continue;
-            const double4_32a pj = pos_r[j];
-            const double dx3 = min_image(xsub(po.x, pj.x), g.periodic[0], L0);
-            const double dy3 = min_image(xsub(po.y, pj.y), g.periodic[1], L1);
-            const double dz3 = min_image(xsub(po.z, pj.z), g.periodic[2], L2);
-            // eq. (contactpos) for spheres: n = (x_i - x_j)/d, the outward
-            // normal of S_j at its point closest to x_i; xi = d - r_i - r_j
-            double nrm[3];
-            const double d = pair_normal(dx3, dy3, dz3, nrm);
-            double4_32a geo;
-            geo.x = nrm[0];
-            geo.y = nrm[1];
-            geo.z = nrm[2];
-            geo.w = xsub(xsub(d, po.w), pj.w);
             cj1[idx] = i_o;
             cj2[idx] = j;
-            cgeo[idx] = geo;
-            clev[idx] = make_double2(xsub(d, pj.w), pj.w);
         }
         if (wm == 0) continue;
         const uint32_t si = V.batch ? V.scene_of[i] : 0u;
         int64_t idx = (int64_t)ro + ns;
         for (uint32_t m = wm; m; m &= m - 1) {   // the walls k_narrow kept, in wall order
             const int k = __ffs(m) - 1;
-            double nrm[3], c, sd, xi;
-            uint32_t widx;
-            const int kc = k - planes.count;
-            if (kc >= 0 && kc < planes.ncones) {
-                // the point of the cone's solid nearest to x_i is x_i - sd n:
-                // a wall contact with xi = sd - r_i and l_i = -sd n
-                cone_distance(planes.cone[kc], pi, sd, nrm);
-                xi = xsub(sd, pi.w);
-                widx = (uint32_t)(V.n + k);
-            } else {
-                wall_plane(planes, V, si, k, nrm, c, widx);
-                wall_kept(nrm, c, pi, 0.0, g.tau, sd, xi);   // kept already: only sd and xi are used
-            }
+            // planes and cones count from n, then six faces a scene
+            const uint32_t w = (uint32_t)(V.n + k) + (k >= nplanes + ncones ? 6u * si : 0u);
             if (idx < ccap) {
                 cj1[idx] = i;
-                cj2[idx] = widx;
-                cgeo[idx] = make_double4_32a(nrm[0], nrm[1], nrm[2], xi);
-                clev[idx] = make_double2(sd, 0.0);
+                cj2[idx] = w;
             }
             ++idx;
         }
+    }
+}
+
+// Normal, gap and levers of every contact, eq. (contactpos): a thread per
+// contact.  A pair takes 35 FP64 instructions, each of which occupies its
+// scheduler's FP64 unit for 64 cycles; that bounds the kernel (5.99M contacts
+// 372 us, ncu, cold), so comparisons and the zeros of a lattice are read off
+// the numbers' words.  Beside the colouring, on a stream of its own, it would
+// spare a step of 2.75M contacts 100 us and one of 5.99M nothing.
+__global__ void k_contact_geometry(DCount Cc, const double4_32a* __restrict__ pos_r,
+                                   const uint32_t* __restrict__ cj1, const uint32_t* __restrict__ cj2, GridArgs g,
+                                   const __grid_constant__ Planes planes, SceneView V, double4_32a* __restrict__ cgeo,
+                                   double2* __restrict__ clev)
+{
+    const int64_t C = Cc.get();
+    const double L0 = g.hi[0] - g.lo[0], L1 = g.hi[1] - g.lo[1], L2 = g.hi[2] - g.lo[2];
+    for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = cj1[c], j = cj2[c];
+        const double4_32a pi = pos_r[i];
+        double nrm[3], xi, la, lb;
+        if (j < (uint64_t)V.n) {
+            const double4_32a pj = pos_r[j];
+            const double dx3 = min_image(xsub(pi.x, pj.x), g.periodic[0], L0);
+            const double dy3 = min_image(xsub(pi.y, pj.y), g.periodic[1], L1);
+            const double dz3 = min_image(xsub(pi.z, pj.z), g.periodic[2], L2);
+            // for spheres: n = (x_i - x_j)/d, the outward normal of S_j at its
+            // point closest to x_i; xi = d - r_i - r_j
+            const double d = pair_normal(dx3, dy3, dz3, nrm);
+            xi = xsub(xsub(d, pi.w), pj.w);
+            la = xsub(d, pj.w);
+            lb = pj.w;
+        } else {
+            const uint32_t w = (uint32_t)(j - V.n);
+            double sd, cc;
+            if (w >= (uint32_t)planes.count && w < (uint32_t)(planes.count + planes.ncones)) {
+                // the point of the cone's solid nearest to x_i is x_i - sd n:
+                // a wall contact with xi = sd - r_i and l_i = -sd n
+                cone_distance(planes.cone[w - planes.count], pi, sd, nrm);
+                xi = xsub(sd, pi.w);
+            } else {
+                uint32_t widx;
+                const uint32_t f = w - (uint32_t)planes.count;   // of a batch's boxes
+                const bool face = w >= (uint32_t)planes.count;
+                wall_plane(planes, V, face ? f / 6u : 0u, face ? planes.count + (int)(f % 6u) : (int)w, nrm, cc, widx);
+                wall_kept(nrm, cc, pi, 0.0, g.tau, sd, xi);   // kept already: only sd and xi are used
+            }
+            la = sd;
+            lb = 0.0;
+        }
+        cgeo[c] = make_double4_32a(nrm[0], nrm[1], nrm[2], xi);
+        clev[c] = make_double2(la, lb);
     }
 }
 
@@ -995,6 +1013,17 @@ __global__ void k_check_contacts(DevInfo* info, int64_t ccap)
     if ((int64_t)info->n_contacts > ccap) atomicOr(&info->err, kErrContacts);
 }
 
+static nbgs_status write_contacts(nbgs_scene* s, const GridArgs& g, DCount C)
+{
+    const int T = 256;
+    k_write_ends<<<grid_for(s->n, T, 8, s->num_sms), T, 0, s->stream>>>(
+        s->n, s->ccap, s->svals, s->cand, s->pair_cnt, s->wall_mask, s->row_off, s->planes.count, s->planes.ncones,
+        scene_view(s), s->cj1, s->cj2);
+    k_contact_geometry<<<grid_for(std::max<int64_t>(C.v, 1), T, 8, s->num_sms), T, 0, s->stream>>>(
+        C, s->pos_r, s->cj1, s->cj2, g, s->planes, scene_view(s), s->cgeo, s->clev);
+    return cuda_check(s, cudaGetLastError(), "detect");
+}
+
 nbgs_status run_detect(nbgs_scene* s)
 {
     const int64_t n = s->n;
@@ -1061,11 +1090,10 @@ nbgs_status run_detect(nbgs_scene* s)
         // sets an error bit (the writes past it are skipped), and every
         // later kernel reads the count on the device
         k_check_contacts<<<1, 1, 0, st>>>(s->info, s->ccap);
-        k_write_contacts<<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->ccap, s->svals, s->pos_r,
-                                                                      s->cand, s->pair_cnt, s->wall_mask, s->row_off, g, s->planes,
-                                                                      scene_view(s), s->cj1, s->cj2, s->cgeo, s->clev);
+        rc = write_contacts(s, g, contact_count(s));
+        if (rc != NBGS_OK) return rc;
         if (s->timing) {
-            s->phase_launches[0] += 3;
+            s->phase_launches[0] += 4;
             cudaEventRecord(s->ev[1], st);
         }
         s->n_contacts = s->ccap;   // an upper bound; the count itself stays on the device
@@ -1089,14 +1117,13 @@ nbgs_status run_detect(nbgs_scene* s)
         rc = grow_contacts(s, nc);
         if (rc != NBGS_OK) return rc;
     }
-    k_write_contacts<<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->ccap, s->svals, s->pos_r, s->cand,
-                                                                  s->pair_cnt, s->wall_mask, s->row_off, g, s->planes, scene_view(s),
-                                                                  s->cj1, s->cj2, s->cgeo, s->clev);
+    s->n_contacts = nc;
+    rc = write_contacts(s, g, DCount{nc, nullptr});
+    if (rc != NBGS_OK) return rc;
     if (s->timing) {
-        s->phase_launches[0] += 1;
+        s->phase_launches[0] += 2;
         cudaEventRecord(s->ev[1], st);
     }
-    s->n_contacts = nc;
     s->detected = true;
     return cuda_check(s, cudaGetLastError(), "detect");
 }

@@ -548,8 +548,7 @@ nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm)
     A.scene_rk = s->scene_rk;
     A.scene_done = s->scene_done;
     A.scene_res = s->scene_res;
-    // a device-sized step knows the count of the last step the host looked at
-    const FlowPlan P = flow_plan<R>(s->n, s->device_sized ? (int64_t)s->hinfo->n_contacts : s->n_contacts, s->batch);
+    const FlowPlan P = flow_plan<R>(s->n, known_contacts(s), s->batch);
     A.tile = P.tile;
     const void* fn = P.fn;
     const int threads = 32 * P.warps;

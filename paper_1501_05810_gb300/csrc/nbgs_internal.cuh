@@ -596,6 +596,12 @@ nbgs_status run_get_contacts(nbgs_scene* s, int64_t cap, uint32_t* j1, uint32_t*
 nbgs_status exclusive_scan_u32(nbgs_scene* s, const uint32_t* in, uint32_t* out, int64_t n,
                                uint32_t* total_dst);
 nbgs_status exclusive_scan_u32(nbgs_scene* s, const uint32_t* in, uint32_t* out, DCount n, uint32_t* total_dst);
+// The contacts as the host knows them: a device-sized step's count stays on the
+// device, the last one that came to the host stands for it.
+inline int64_t known_contacts(const nbgs_scene* s)
+{
+    return s->device_sized ? (int64_t)s->hinfo->n_contacts : s->n_contacts;
+}
 int grid_for(int64_t work, int threads, int max_blocks_per_sm, int num_sms);
 // The contact count of the current step for kernels: host-known, or read on
 // the device (device-sized steps; launches sized for the capacity).
