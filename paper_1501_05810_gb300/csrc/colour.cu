@@ -527,13 +527,77 @@ k_colour_scatter(DCount Cc, const uint32_t* __restrict__ cstate, const uint32_t*
     }
 }
 
+// With subdomains: what the ends of a contact need to know of their instances.
+struct SubView {
+    const uint32_t* inst;      // two instances per contact (null: no subdomains)
+    const uint32_t* ext_off;   // a body's extra instances
+    const uint32_t* ends;      // two dependency ends per contact, of bodies with several instances
+    int jacobi;                // an instance per contact, one colour
+};
+
+// Dependency ends (as dep_end) of the contacts of every body with several
+// instances: a contact comes after those of the same instance and a lower
+// colour.  A thread per body, which looks its list up once; for each contact
+// to look through its bodies' lists instead cost 120 us with 1.57M contacts.
+__global__ void k_sub_ends(const uint32_t* __restrict__ shared, const uint32_t* __restrict__ adj_off,
+                           const uint32_t* __restrict__ adj, const uint32_t* __restrict__ inst,
+                           const uint32_t* __restrict__ cj1, const uint32_t* __restrict__ cstate,
+                           const DevInfo* __restrict__ info, uint32_t* __restrict__ ends)
+{
+    const int64_t ns = info->n_shared;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < ns; t += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t x = shared[t], e0 = adj_off[x], m = adj_off[x + 1] - e0;
+        constexpr uint32_t kKept = 16;   // entries kept at hand; longer lists read theirs again
+        uint32_t slot[kKept], col[kKept];
+        auto look = [&](uint32_t e, uint32_t& s, uint32_t& k) {
+            const uint32_t d = adj[e0 + e];
+            s = inst[2 * (int64_t)d + (cj1[d] == x ? 0 : 1)];
+            k = cstate[d] & 0xFFu;
+        };
+        for (uint32_t e = 0; e < min(m, kKept); ++e) look(e, slot[e], col[e]);
+        for (uint32_t e = 0; e < m; ++e) {
+            uint32_t s, k, pred = 0u;
+            bool last = true;
+            if (e < kKept) {
+                s = slot[e];
+                k = col[e];
+            } else {
+                look(e, s, k);
+            }
+            for (uint32_t f = 0; f < m; ++f) {
+                uint32_t sf, kf;
+                if (f < kKept) {
+                    sf = slot[f];
+                    kf = col[f];
+                } else {
+                    look(f, sf, kf);
+                }
+                if (sf != s) continue;
+                if (kf < k) pred = max(pred, kf + 1u);
+                if (kf > k) last = false;
+            }
+            const uint32_t d = adj[e0 + e];
+            ends[2 * (int64_t)d + (cj1[d] == x ? 0 : 1)] = pred | (last ? kDepLastA : 0u) | kDepListA;
+        }
+    }
+}
+
+// End `side` of contact c (colour col) at body x.
+__device__ __forceinline__ uint32_t sub_end(const SubView& S, uint32_t x, int side, int64_t c, uint32_t col,
+                                            const uint32_t* __restrict__ mask, bool& several)
+{
+    several = S.ext_off[x + 1] != S.ext_off[x];
+    if (S.jacobi) return kDepLastA | kDepListA;
+    return several ? S.ends[2 * c + side] : dep_end(mask + 8 * (int64_t)x, col);
+}
+
 // Sweep record inv[c] <- canonical contact c; initial impulse from the
 // previous step (world frame, re-projected onto the new frame and the cone)
 // or zero.  A thread per canonical contact: the contact arrays and the
 // previous step's rows are read in order, the records written scattered.
 template <class R>
 __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__ inv, const uint32_t* __restrict__ cj1,
-                              const uint32_t* __restrict__ cj2, const uint32_t* __restrict__ inst,
+                              const uint32_t* __restrict__ cj2, SubView S,
                               const double4_32a* __restrict__ cgeo,
                               const double2* __restrict__ clev, double dt, double beta, double mu_all, SceneView V,
                               int warm,
@@ -549,7 +613,7 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
         const uint32_t a = cj1[c], b = cj2[c];
         // the velocity records the sweep reads: the bodies, or with subdomains
         // their instances for the contact's subdomain
-        const uint32_t ra = inst ? inst[2 * (int64_t)c] : a, rb = inst ? inst[2 * (int64_t)c + 1] : b;
+        const uint32_t ra = S.inst ? S.inst[2 * (int64_t)c] : a, rb = S.inst ? S.inst[2 * (int64_t)c + 1] : b;
         const double4_32a g = cgeo[c];
         const double2 l = clev[c];
         // eq. (nonpenetration): gap term xi/dt, scaled by beta when xi < 0
@@ -567,7 +631,7 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
             r.nz_ = make_double2(g.z, -1.0 / (copysign(1.0, g.z) + g.z));
         }
         rec[s] = r;
-        if (mask) {
+        {
             const bool dyn_b = b < (uint64_t)n;
             const R ima = vel[2 * (int64_t)a].w, iIa = vel[2 * (int64_t)a + 1].w;
             const R imb = dyn_b ? vel[2 * (int64_t)b].w : R(0), iIb = dyn_b ? vel[2 * (int64_t)b + 1].w : R(0);
@@ -587,12 +651,19 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
         // the friction cone; in the sweep precision (FP64 arithmetic is scarce
         // on this GPU, and an FP32 sweep starts from an FP32 impulse anyway)
         R pn = R(0), pt = R(0), po = R(0);
-        uint32_t dep = 0u;   // mask: the colours of every body's contacts (no subdomains)
-        if (mask) {
+        uint32_t dep = 0u;
+        {
             const uint32_t col = cstate[c] & 0xFFu;
             const uint4 q = cpack[c];
-            if (q.x != kNoList) dep |= dep_end(mask + 8 * (int64_t)q.x, col);
-            if (q.y != kNoList) dep |= dep_end(mask + 8 * (int64_t)q.y, col) << 11;
+            if (S.inst) {
+                bool sa = false, sb = false;
+                if (q.x != kNoList) dep |= sub_end(S, q.x, 0, c, col, mask, sa);
+                if (q.y != kNoList) dep |= sub_end(S, q.y, 1, c, col, mask, sb) << 11;
+                dep |= (sa ? kDepSharedA : 0u) | (sb ? kDepSharedB : 0u);
+            } else {
+                if (q.x != kNoList) dep |= dep_end(mask + 8 * (int64_t)q.x, col);
+                if (q.y != kNoList) dep |= dep_end(mask + 8 * (int64_t)q.y, col) << 11;
+            }
         }
         if (warm) {
             const uint32_t e = prev_row_off[a + 1];
@@ -718,23 +789,28 @@ nbgs_status run_colour(nbgs_scene* s)
         k_colour_scatter<<<(unsigned)nbs, kSortThreads, 0, st>>>(Cn, s->cstate, s->sort_hist, nbs, s->perm, s->inv,
                                                                  s->col_off, s->info);
         const int warm = (s->prm.warm_start != NBGS_WARM_NONE && s->have_prev) ? 1 : 0;
+        uint32_t* ends = (uint32_t*)s->cprio;   // the priorities have served
+        const SubView S{sub ? s->inst : nullptr, s->ext_off, ends, jacobi ? 1 : 0};
+        if (sub && !jacobi)
+            k_sub_ends<<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(s->shared, s->adj_off, s->adj, s->inst, s->cj1,
+                                                                    s->cstate, s->info, ends);
         if (s->composite) {
             rc = run_comp_records(s, warm);
             if (rc != NBGS_OK) return rc;
         } else if (s->fp32)
-            k_build_sweep<float><<<gb, T, 0, st>>>(Cn, n, s->inv, s->cj1, s->cj2, sub ? s->inst : nullptr, s->cgeo,
+            k_build_sweep<float><<<gb, T, 0, st>>>(Cn, n, s->inv, s->cj1, s->cj2, S, s->cgeo,
                                                    s->clev, s->prm.dt,
                                                    s->prm.beta, s->prm.mu, scene_view(s), warm, s->prev_row_off,
                                                    s->prev_j2,
-                                                   s->prev_P, s->ccap, s->cstate, s->cpack, sub ? nullptr : s->cmask,
+                                                   s->prev_P, s->ccap, s->cstate, s->cpack, s->cmask,
                                                    (const float4*)s->vel, (SweepRec<float>*)s->srec, (float4*)s->sp,
                                                    (SweepPre<float>*)s->spre);
         else
-            k_build_sweep<double><<<gb, T, 0, st>>>(Cn, n, s->inv, s->cj1, s->cj2, sub ? s->inst : nullptr, s->cgeo,
+            k_build_sweep<double><<<gb, T, 0, st>>>(Cn, n, s->inv, s->cj1, s->cj2, S, s->cgeo,
                                                     s->clev, s->prm.dt,
                                                     s->prm.beta, s->prm.mu, scene_view(s), warm, s->prev_row_off,
                                                     s->prev_j2,
-                                                    s->prev_P, s->ccap, s->cstate, s->cpack, sub ? nullptr : s->cmask,
+                                                    s->prev_P, s->ccap, s->cstate, s->cpack, s->cmask,
                                                     (const double4_32a*)s->vel, (SweepRec<double>*)s->srec,
                                                     (double4_32a*)s->sp, (SweepPre<double>*)s->spre);
         if (s->timing) s->phase_launches[1] += 3;

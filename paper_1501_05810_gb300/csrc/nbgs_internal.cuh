@@ -222,8 +222,11 @@ template <> struct __align__(32) SweepPre<double> {
 // Dependency word of a contact (bits of .w of its sweep impulse): per end,
 // the colour + 1 of the contact before it in its body's colour order (9 bits,
 // 0: it is the first), whether it is the body's last, and whether the body
-// takes impulses at all; bit 31: the contact existed in the previous step.
+// takes impulses at all; bits 22 and 23: with subdomains, whether the body has
+// several instances (colours count within the end's own); bit 31: the contact
+// existed in the previous step.
 constexpr uint32_t kDepLastA = 1u << 9, kDepListA = 1u << 10, kDepLastB = 1u << 20, kDepListB = 1u << 21;
+constexpr uint32_t kDepSharedA = 1u << 22, kDepSharedB = 1u << 23;
 constexpr uint32_t kDepFound = 1u << 31;
 
 __device__ __forceinline__ uint32_t dep_bits(float w) { return __float_as_uint(w); }

@@ -1055,7 +1055,7 @@ static nbgs_status solve_impl(nbgs_scene* s, int max_sweeps, double tol)
         if (rc != NBGS_OK) return rc;
     }
     // no scheduling flag: the dataflow sweeps
-    if (s->prm.solver == NBGS_SOLVER_PERSISTENT && s->prm.sweep_flags == 0 && !A.sub)
+    if (s->prm.solver == NBGS_SOLVER_PERSISTENT && s->prm.sweep_flags == 0)
         return run_flow<R>(s, max_sweeps, tol, A.warm);
     if (s->prm.solver == NBGS_SOLVER_PERSISTENT) {
         // scheduling units: blocks, or warps with NBGS_SWEEP_WARP_SYNC

@@ -72,6 +72,33 @@ def test_flow_equals_grid_synchronised_sweeps(shape, precision, tol, omega, fixe
             assert np.abs(ca["impulse"] - cb["impulse"]).max() <= bound * np.abs(cb["impulse"]).max()
 
 
+@pytest.mark.parametrize("shape,sub,precision,tol,fixed", [
+    ((5, 6, 2), (2, 2, 2), "fp32", 0.0, False), ((5, 6, 4), "jacobi", "fp32", 0.0, True),
+    ((9, 10, 9), (3, 1, 2), "fp32", 1e-3, True), ((20, 20, 20), (20, 20, 20), "fp32", 0.0, False),
+    ((44, 46, 44), (4, 4, 1), "fp32", 0.0, True), ((55, 56, 54), (8, 8, 1), "fp32", 0.0, False),
+    ((55, 56, 54), "jacobi", "fp32", 0.0, False), ((7, 8, 6), (2, 2, 2), "fp64", 1e-6, True),
+    ((9, 10, 9), "jacobi", "fp64", 0.0, False), ((40, 42, 40), (5, 5, 5), "fp64", 0.0, True)])
+def test_subdomain_flow_equals_grid_synchronised_sweeps(shape, sub, precision, tol, fixed):
+    """Bodies with one instance, a few, one per contact; sums that fill no
+    tile or more than the grid has warps."""
+    sc = _scene(shape, precision, omega=0.5, subdomains=sub)
+    sweeps = 12
+    flow, ref = _run(sc, 0, tol, sweeps, fixed), _run(sc, GLOBAL_SYNC, tol, sweeps, fixed)
+    for (sa, ha, ba, ca), (sb, hb, bb, cb) in zip(flow, ref):
+        assert sa["n_contacts"] == sb["n_contacts"] and sa["n_colours"] == sb["n_colours"]
+        assert sa["sweeps_done"] == sb["sweeps_done"]
+        if precision == "fp32":   # the same roundings in every kernel
+            for k in ("pos", "quat", "vel", "angvel"):
+                assert np.array_equal(ba[k], bb[k]), k
+            assert np.array_equal(ca["impulse"], cb["impulse"])
+            assert np.array_equal(ha, hb) and sa["residual"] == sb["residual"]
+        else:   # as above
+            bound = 1.1e-16 * 4 * 144 * 2 * 10
+            for k in ("vel", "angvel"):
+                assert np.abs(ba[k] - bb[k]).max() <= bound * np.abs(bb[k]).max()
+            assert np.abs(ca["impulse"] - cb["impulse"]).max() <= bound * np.abs(cb["impulse"]).max()
+
+
 @pytest.mark.parametrize("sizes,precision,tol", [
     ((1, 1, 2), "fp32", 1e-6), ((60, 151, 300, 97, 420, 33), "fp32", 1e-6), ((60, 151, 300), "fp32", 1e300),
     ((37,) * 700, "fp32", 1e-4), ((2000, 20, 9000, 400, 20000), "fp32", 0.0), ((300, 20, 900), "fp64", 0.0)])
