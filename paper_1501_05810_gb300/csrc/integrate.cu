@@ -88,34 +88,63 @@ nbgs_status run_integrate(nbgs_scene* s)
 }
 
 // ---------------------------------------------------------------------------
-// state transfer: staging holds pos (3n) | quat (4n) | vel (3n) | angvel (3n)
+// state transfer: arrays on this GPU are read and written where they are;
+// others go through the staging buffer, pos (3n) | quat (4n) | vel (3n) |
+// angvel (3n).  4M bodies: the four copies beside each kernel took 125 us.
 // ---------------------------------------------------------------------------
+// Is [p, p + bytes) doubles in one allocation of this GPU?  (A copy of an array
+// that ends before that fails; so it is left to the copy to say so.)
+static bool on_device(const void* p, size_t bytes)
+{
+    if (((uintptr_t)p & 7u) != 0) return false;
+    cudaPointerAttributes at;
+    int dev = -1;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (at.type != cudaMemoryTypeDevice || at.device != dev) return false;
+    using Range = int (*)(unsigned long long*, size_t*, unsigned long long);
+    static const Range range = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+        if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return (Range)f;
+    }();
+    unsigned long long base = 0;
+    size_t size = 0;
+    if (!range || range(&base, &size, (unsigned long long)(uintptr_t)p) != 0) return false;
+    return (unsigned long long)(uintptr_t)p + bytes <= base + size;
+}
+
+// Null arrays are left alone.
 template <class R>
-__global__ void k_unpack_state(int64_t n, const double* __restrict__ stg, int has_pos, int has_quat, int has_vel,
-                               int has_ang, double4_32a* __restrict__ pos_r, double4_32a* __restrict__ quat,
+__global__ void k_unpack_state(int64_t n, const double* __restrict__ P, const double* __restrict__ Q,
+                               const double* __restrict__ V, const double* __restrict__ W,
+                               double4_32a* __restrict__ pos_r, double4_32a* __restrict__ quat,
                                R4<R>* __restrict__ vel)
 {
-    const double* P = stg;
-    const double* Q = stg + 3 * n;
-    const double* V = stg + 7 * n;
-    const double* W = stg + 10 * n;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        if (has_pos) {
+        if (P) {
             double4_32a x = pos_r[i];
             x.x = P[3 * i];
             x.y = P[3 * i + 1];
             x.z = P[3 * i + 2];
             pos_r[i] = x;
         }
-        if (has_quat) quat[i] = make_double4_32a(Q[4 * i], Q[4 * i + 1], Q[4 * i + 2], Q[4 * i + 3]);
-        if (has_vel) {
+        if (Q) quat[i] = make_double4_32a(Q[4 * i], Q[4 * i + 1], Q[4 * i + 2], Q[4 * i + 3]);
+        if (V) {
             R4<R> v = vel[2 * i];
             v.x = (R)V[3 * i];
             v.y = (R)V[3 * i + 1];
             v.z = (R)V[3 * i + 2];
             vel[2 * i] = v;
         }
-        if (has_ang) {
+        if (W) {
             R4<R> w = vel[2 * i + 1];
             w.x = (R)W[3 * i];
             w.y = (R)W[3 * i + 1];
@@ -126,30 +155,36 @@ __global__ void k_unpack_state(int64_t n, const double* __restrict__ stg, int ha
 }
 
 template <class R>
-__global__ void k_pack_state(int64_t n, double* __restrict__ stg, const double4_32a* __restrict__ pos_r,
-                             const double4_32a* __restrict__ quat, const R4<R>* __restrict__ vel)
+__global__ void k_pack_state(int64_t n, double* P, double* Q, double* V, double* W,
+                             const double4_32a* __restrict__ pos_r, const double4_32a* __restrict__ quat,
+                             const R4<R>* __restrict__ vel)
 {
-    double* P = stg;
-    double* Q = stg + 3 * n;
-    double* V = stg + 7 * n;
-    double* W = stg + 10 * n;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double4_32a x = pos_r[i];
-        P[3 * i] = x.x;
-        P[3 * i + 1] = x.y;
-        P[3 * i + 2] = x.z;
-        const double4_32a q = quat[i];
-        Q[4 * i] = q.x;
-        Q[4 * i + 1] = q.y;
-        Q[4 * i + 2] = q.z;
-        Q[4 * i + 3] = q.w;
-        const R4<R> v = vel[2 * i], w = vel[2 * i + 1];
-        V[3 * i] = v.x;
-        V[3 * i + 1] = v.y;
-        V[3 * i + 2] = v.z;
-        W[3 * i] = w.x;
-        W[3 * i + 1] = w.y;
-        W[3 * i + 2] = w.z;
+        if (P) {
+            const double4_32a x = pos_r[i];
+            P[3 * i] = x.x;
+            P[3 * i + 1] = x.y;
+            P[3 * i + 2] = x.z;
+        }
+        if (Q) {
+            const double4_32a q = quat[i];
+            Q[4 * i] = q.x;
+            Q[4 * i + 1] = q.y;
+            Q[4 * i + 2] = q.z;
+            Q[4 * i + 3] = q.w;
+        }
+        if (V) {
+            const R4<R> v = vel[2 * i];
+            V[3 * i] = v.x;
+            V[3 * i + 1] = v.y;
+            V[3 * i + 2] = v.z;
+        }
+        if (W) {
+            const R4<R> w = vel[2 * i + 1];
+            W[3 * i] = w.x;
+            W[3 * i + 1] = w.y;
+            W[3 * i + 2] = w.z;
+        }
     }
 }
 
@@ -189,21 +224,18 @@ static nbgs_status set_bodies_impl(nbgs_scene* s, const double* pos, const doubl
 {
     const int64_t n = s->n;
     cudaStream_t st = s->stream;
-    nbgs_status rc = NBGS_OK;
-    if (pos) rc = cuda_check(s, cudaMemcpyAsync(s->stage, pos, 3 * n * sizeof(double), cudaMemcpyDefault, st), "set pos");
-    if (rc == NBGS_OK && quat)
-        rc = cuda_check(s, cudaMemcpyAsync(s->stage + 3 * n, quat, 4 * n * sizeof(double), cudaMemcpyDefault, st),
-                        "set quat");
-    if (rc == NBGS_OK && vel)
-        rc = cuda_check(s, cudaMemcpyAsync(s->stage + 7 * n, vel, 3 * n * sizeof(double), cudaMemcpyDefault, st),
-                        "set vel");
-    if (rc == NBGS_OK && angvel)
-        rc = cuda_check(s, cudaMemcpyAsync(s->stage + 10 * n, angvel, 3 * n * sizeof(double), cudaMemcpyDefault, st),
-                        "set angvel");
-    if (rc != NBGS_OK) return rc;
+    const double* src[4] = {pos, quat, vel, angvel};
+    const int64_t at[4] = {0, 3 * n, 7 * n, 10 * n}, len[4] = {3 * n, 4 * n, 3 * n, 3 * n};
+    const char* what[4] = {"set pos", "set quat", "set vel", "set angvel"};
+    for (int k = 0; k < 4; ++k) {
+        if (!src[k] || on_device(src[k], len[k] * sizeof(double))) continue;
+        nbgs_status rc = cuda_check(s, cudaMemcpyAsync(s->stage + at[k], src[k], len[k] * sizeof(double),
+                                                       cudaMemcpyDefault, st), what[k]);
+        if (rc != NBGS_OK) return rc;
+        src[k] = s->stage + at[k];
+    }
     const int T = 256;
-    k_unpack_state<R><<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->stage, pos != nullptr, quat != nullptr,
-                                                                   vel != nullptr, angvel != nullptr, s->pos_r,
+    k_unpack_state<R><<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, src[0], src[1], src[2], src[3], s->pos_r,
                                                                    s->quat, (R4<R>*)s->vel);
     s->detected = s->coloured = false;
     return cuda_check(s, cudaGetLastError(), "set_bodies");
@@ -223,25 +255,29 @@ nbgs_status run_get_bodies(nbgs_scene* s, double* pos, double* quat, double* vel
     const int64_t n = s->n;
     if (n == 0) return NBGS_OK;
     cudaStream_t st = s->stream;
+    double* const out[4] = {pos, quat, vel, angvel};
+    const int64_t at[4] = {0, 3 * n, 7 * n, 10 * n}, len[4] = {3 * n, 4 * n, 3 * n, 3 * n};
+    const char* what[4] = {"get pos", "get quat", "get vel", "get angvel"};
+    double* dst[4];
+    for (int k = 0; k < 4; ++k) {
+        // arrays that overlap are written one after the other, by the copies
+        bool alone = true;
+        for (int q = 0; q < 4; ++q)
+            alone = alone && (q == k || !out[q] || !out[k] || (uintptr_t)(out[q] + len[q]) <= (uintptr_t)out[k] ||
+                              (uintptr_t)(out[k] + len[k]) <= (uintptr_t)out[q]);
+        dst[k] = !out[k] ? nullptr : alone && on_device(out[k], len[k] * sizeof(double)) ? out[k] : s->stage + at[k];
+    }
     const int T = 256;
     if (s->fp32)
-        k_pack_state<float><<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->stage, s->pos_r, s->quat,
-                                                                         (const float4*)s->vel);
+        k_pack_state<float><<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, dst[0], dst[1], dst[2], dst[3], s->pos_r,
+                                                                         s->quat, (const float4*)s->vel);
     else
-        k_pack_state<double><<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, s->stage, s->pos_r, s->quat,
-                                                                          (const double4_32a*)s->vel);
+        k_pack_state<double><<<grid_for(n, T, 8, s->num_sms), T, 0, st>>>(n, dst[0], dst[1], dst[2], dst[3], s->pos_r,
+                                                                          s->quat, (const double4_32a*)s->vel);
     nbgs_status rc = cuda_check(s, cudaGetLastError(), "get_bodies");
-    if (rc == NBGS_OK && pos)
-        rc = cuda_check(s, cudaMemcpyAsync(pos, s->stage, 3 * n * sizeof(double), cudaMemcpyDefault, st), "get pos");
-    if (rc == NBGS_OK && quat)
-        rc = cuda_check(s, cudaMemcpyAsync(quat, s->stage + 3 * n, 4 * n * sizeof(double), cudaMemcpyDefault, st),
-                        "get quat");
-    if (rc == NBGS_OK && vel)
-        rc = cuda_check(s, cudaMemcpyAsync(vel, s->stage + 7 * n, 3 * n * sizeof(double), cudaMemcpyDefault, st),
-                        "get vel");
-    if (rc == NBGS_OK && angvel)
-        rc = cuda_check(s, cudaMemcpyAsync(angvel, s->stage + 10 * n, 3 * n * sizeof(double), cudaMemcpyDefault, st),
-                        "get angvel");
+    for (int k = 0; k < 4 && rc == NBGS_OK; ++k)
+        if (out[k] && dst[k] != out[k])
+            rc = cuda_check(s, cudaMemcpyAsync(out[k], dst[k], len[k] * sizeof(double), cudaMemcpyDefault, st), what[k]);
     if (rc == NBGS_OK) rc = cuda_check(s, cudaStreamSynchronize(st), "get_bodies");
     return rc;
 }
