@@ -408,9 +408,16 @@ __global__ void k_hull(int64_t n, const R4<R>* __restrict__ vel, const double4_3
         p32[i] = make_float4((float)(x.x - g.lo[0]), (float)(x.y - g.lo[1]), (float)(x.z - g.lo[2]), rf + h32);
         // beyond FP32: NaN, Inf, or squares too large for it
         if (!(v2 <= 1e38f && w2 <= 1e38f) && !(norm2_exact<R>(v) <= 1e300 && norm2_exact<R>(w) <= 1e300)) bad = true;
-        if (scene_of) {   // per-scene max |v|^2 (v_ref); the filter only saves FP64 squares and atomics
-            unsigned long long* dst = scene_vmax + scene_of[i];
-            if (!((float)__longlong_as_double((long long)*(volatile unsigned long long*)dst) > v2 * (1.f + 1e-6f) + 1e-30f)) {
+        if (scene_of) {   // per-scene max |v|^2 (v_ref); the filters only save FP64 squares and atomics
+            const uint32_t sc = scene_of[i], act = __activemask();
+            // a warp's bodies are mostly of one scene: only its fastest can count
+            // (all of them asked for an atomic while the maxima were still low)
+            bool asks = true;
+            if (__match_any_sync(act, sc) == act)
+                asks = v2 >= __uint_as_float(__reduce_max_sync(act, __float_as_uint(v2))) * (1.f - 1e-6f) - 1e-30f;
+            unsigned long long* dst = scene_vmax + sc;
+            if (asks &&
+                !((float)__longlong_as_double((long long)*(volatile unsigned long long*)dst) > v2 * (1.f + 1e-6f) + 1e-30f)) {
                 const unsigned long long bits = (unsigned long long)__double_as_longlong(norm2_exact<R>(v));
                 if (bits > *(volatile unsigned long long*)dst) atomicMax(dst, bits);
             }
