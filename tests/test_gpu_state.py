@@ -54,3 +54,32 @@ def test_state_round_trip(n, precision, off):
     a = np.frombuffer(both[off:off + 24 * (n + 1)].cpu().numpy().tobytes()).reshape(n + 1, 3)
     assert np.array_equal(a[0], want["pos"][0]) and np.array_equal(a[1:], want["vel"])
     g.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("lo", [0.0, -3.0])
+def test_integrate_at_the_edges_of_formats_and_boxes(precision, lo):
+    """Conversions of numbers that FP32 holds exactly, rounded or not at all,
+    and the wrap of positions on, next to and beyond the faces."""
+    from paper_1501_05810_gb300 import nbgs
+    R = np.float32 if precision == "fp32" else np.float64
+    hi = lo + 10.0
+    a = np.array([1.0, -2.5, 0.1, 1.0 / 3.0, -1e-18, 1.17549435e-38 * 2.0 ** 70, 2.0 ** 60, 1.0 + 2.0 ** -23, 1.0 + 2.0 ** -24])
+    x = np.array([lo, hi, np.nextafter(hi, lo), np.nextafter(lo, -10.0), lo + 5.0, hi + 12.3, lo - 1e-300, -0.0, 1e-310])
+    n = len(a)
+    pos = np.stack([x, np.roll(x, 3), np.roll(x, 5)], -1)
+    prm = scenes.default_params(box_lo=(lo,) * 3, box_hi=(hi,) * 3, periodic=(1, 1, 1), precision=precision)
+    g = nbgs.Scene(scenes._scene("edges", prm, pos, np.zeros((n, 3)), np.zeros((n, 3)), np.full(n, 0.1), np.ones(n), []))
+    quat = np.zeros((n, 4))
+    quat[np.arange(n), np.arange(n) % 4] = a
+    g.set_bodies(pos, quat, np.zeros((n, 3)), np.zeros((n, 3)))
+    g.integrate()
+    b = g.get_bodies()
+    f = a.astype(R)
+    want = np.zeros((n, 4))
+    want[np.arange(n), np.arange(n) % 4] = (f * (R(1) / np.sqrt(f * f))).astype(np.float64)
+    assert np.array_equal(b["quat"], want)
+    s = np.fmod(pos - lo, 10.0)
+    wrapped = np.where((pos >= lo) & (pos < lo + 10.0), pos, lo + np.where(s < 0.0, s + 10.0, s))
+    assert np.array_equal(b["pos"], wrapped)
+    g.close()
