@@ -288,7 +288,33 @@ template <> struct FlowShape<float, 1> {
     static constexpr int threads = 128, blocks = 6;
 };
 
-template <class R, int L, bool Batch, bool Sub = false>
+// Records R_k = x v_ref for a warp and votes on the tolerance: 1 go on, 0 every
+// one of the n voters is below it, -1 a wait gave up.
+__device__ __noinline__ int warp_vote(DevInfo* info, int k, double x, bool below, uint32_t n)
+{
+    if (!(x <= 1e300)) x = __longlong_as_double(0x7FF0000000000000LL);
+    atomicMax(&info->rk_bits[rk_slot(k)], (unsigned long long)__double_as_longlong(x));
+    volatile uint32_t* flag = info->votes + 2 * k;
+    if (!below) {
+        flag[0] = 1u;
+        return 1;
+    }
+    atomicAdd(info->votes + 2 * k + 1, 1u);
+    const long long t0 = clock64();
+    for (;;) {
+        if (flag[0] != 0u) return 1;
+        if (flag[1] == n) return 0;
+        if ((((volatile uint32_t*)&info->err)[0] & kErrTimeout) || clock64() - t0 > (1LL << 31)) {
+            atomicOr(&info->err, kErrTimeout);
+            return -1;
+        }
+    }
+}
+
+// Vote: the tolerance test without a block waiting for its warps.  A warp with
+// a contact above the tolerance says so at once, one without waits at the end
+// of its sweep until another has or all are done.
+template <class R, int L, bool Batch, bool Sub = false, bool Vote = false>
 __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::blocks)) k_solve_flow(FlowArgs<R> A)
 {
     __shared__ uint32_t s_tile[kMaxColours + 1];   // first tile of every colour
@@ -387,6 +413,11 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         scene = nscene;
     }
     if (Sub) at.T = w0;
+    if (Vote && !work) return;
+    // the tolerance as a residual in R, and where the FP64 division is not needed to tell
+    const R near = Vote ? (R)(A.tol * vref) : R(0), slack = sizeof(R) == 4 ? R(1e-5) : R(1e-12);
+    const bool clear = near > R(1e-15) && near < R(1e15);
+    const R far2 = near * near * (R(1) + R(4) * slack);
     int k = 0;
     for (int pass = 0; pass < npass; ++pass) {
         const bool apply = pass < warm;
@@ -402,6 +433,7 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         }
         R rmax = R(0);
         bool over = false;   // a scene's contact above its tolerance
+        bool said = false;   // this warp's is known to the others
         if (Batch) ask(apply ? 0 : k);
         const uint32_t base = (uint32_t)pass << 9;
         for (bool more = work; more && ok;) {
@@ -482,6 +514,10 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
                     scene_max(A.scene_rk + scene_slot(k) * A.nscene, scene, live, lane % L == 0, bits_of(r2));
                 } else {
                     rmax = live && above(r2, rmax) ? r2 : rmax;
+                    if (Vote && !said && clear && __any_sync(kFull, rmax > far2)) {
+                        said = true;
+                        if (lane == 0) ((volatile uint32_t*)A.info->votes)[2 * k] = 1u;
+                    }
                 }
             }
             __syncwarp();   // the lanes of a unit read back what one of them saved
@@ -498,6 +534,19 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         }
         if (apply) continue;
         if (!Batch) rmax = sqrt(rmax);
+        if (Vote) {
+            if (!ok) break;
+            for (int o = 16; o > 0; o >>= 1) rmax = fmax(rmax, __shfl_xor_sync(kFull, rmax, o));
+            const double x = (double)rmax;
+            bool below = false;
+            if (!said && !(clear && rmax > near * (R(1) + slack)))
+                below = (clear && rmax < near * (R(1) - slack)) || x / vref <= A.tol;
+            const int v = lane == 0 ? warp_vote(A.info, k, x, below, min(W, ntot)) : 0;
+            const int all = __shfl_sync(kFull, v, 0);
+            if (all < 0) ok = false;
+            if (all <= 0) break;
+            continue;
+        }
         // R_k is recorded by every warp; a test of it needs the whole block, and
         // every block near the rotating residual slots or for batched scenes
         const bool vote = !Batch && ncol > 0 && A.tol > 0.0 && k + 2 < kHistKept;
@@ -610,14 +659,25 @@ const void* flow_kernel(bool batch, bool sub)
                    : (const void*)k_solve_flow<R, L, false>;
 }
 
+// A tolerance is voted on by warps (vote) where the chain of contacts bounds a
+// sweep and by blocks where their number does: with the tolerance, ms,
+//   bodies              1k FP64    2k     30k    250k   500k     1M
+//   by blocks             1.55    6.81   1.90   2.00    5.18   8.40
+//   by warps              1.42    6.00   1.77   2.19    6.74  10.03
 template <class R>
-FlowPlan flow_plan(int64_t n, int64_t C, bool batch, bool sub)
+FlowPlan flow_plan(int64_t n, int64_t C, bool batch, bool sub, bool vote)
 {
+    vote = vote && !batch && !sub;
     if (sizeof(R) == 4) {
-        if (C < 950000) return {flow_kernel<float, 2>(batch, sub), 16, 8, C < 245000 ? 1 : 2};
+        if (C < 245000)
+            return {vote ? (const void*)k_solve_flow<float, 2, false, false, true> : flow_kernel<float, 2>(batch, sub),
+                    16, 8, 1};
+        if (C < 950000) return {flow_kernel<float, 2>(batch, sub), 16, 8, 2};
         return {flow_kernel<float, 1>(batch, sub), 32, 4, 6};
     }
-    if (n < 64000) return {flow_kernel<double, 4>(batch, sub), 8, 8, 1};
+    if (n < 64000)
+        return {vote ? (const void*)k_solve_flow<double, 4, false, false, true> : flow_kernel<double, 4>(batch, sub),
+                8, 8, 1};
     return {flow_kernel<double, 1>(batch, sub), 32, n < 250000 ? 4 : 8, 1};
 }
 
@@ -662,7 +722,9 @@ nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm)
     A.scene_rk = s->scene_rk;
     A.scene_done = s->scene_done;
     A.scene_res = s->scene_res;
-    const FlowPlan P = flow_plan<R>(s->n, known_contacts(s), s->batch, sub);
+    // (near the rotating residual slots blocks meet at a barrier: they vote as blocks then)
+    const bool vote = tol > 0.0 && max_sweeps + 2 < kHistKept && s->n_contacts > 0;
+    const FlowPlan P = flow_plan<R>(s->n, known_contacts(s), s->batch, sub, vote);
     A.tile = P.tile;
     const void* fn = P.fn;
     const int threads = 32 * P.warps;

@@ -45,7 +45,9 @@ def _run(sc, flags, tol, sweeps, fixed):
 
 
 @pytest.mark.parametrize("shape,precision,tol,omega,fixed", [
-    ((5, 6, 2), "fp32", 0.0, 1.0, False), ((5, 6, 4), "fp32", 1e-3, 1.0, True), ((9, 10, 9), "fp32", 0.0, 0.8, True),
+    ((5, 6, 2), "fp32", 0.0, 1.0, False), ((5, 6, 4), "fp32", 1e-3, 1.0, True),
+    ((5, 6, 2), "fp32", 1e30, 1.0, False), ((30, 30, 30), "fp32", 2e-2, 1.0, False), ((5, 6, 4), "fp32", 1e-30, 1.0, True),
+    ((12, 12, 12), "fp64", 1e-2, 1.0, False), ((44, 46, 44), "fp32", 2e-2, 1.0, False), ((9, 10, 9), "fp32", 0.0, 0.8, True),
     ((44, 46, 44), "fp32", 0.0, 1.0, False), ((45, 46, 46), "fp32", 0.0, 1.0, False),
     ((70, 72, 70), "fp32", 0.0, 1.0, True), ((5, 6, 2), "fp64", 0.0, 1.0, True), ((7, 8, 6), "fp64", 1e-6, 0.9, True),
     ((40, 40, 39), "fp64", 0.0, 1.0, False), ((40, 42, 40), "fp64", 0.0, 1.0, True)])
