@@ -326,8 +326,17 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
     const uint32_t tw = (uint32_t)A.tile;
     tile_offsets(A.col_off, ncol, tw, s_off, s_tile);
     const uint32_t ntile = s_tile[ncol];
-    // warp w of the grid: warps 0 of all blocks first, so that few tiles spread over the SMs
-    const uint32_t W = nb * (blockDim.x >> 5), w0 = (threadIdx.x >> 5) * nb + blockIdx.x;
+    // Warp w0 of the grid.  FP32, every warp with tiles: the warps of a block take
+    // consecutive ones, whose bodies and records share lines.  Few tiles spread
+    // over the SMs, warps 0 of all blocks first; so do FP64 ones, whose
+    // arithmetic would pile up on the SMs a chain of contacts passes.  Sweeps,
+    // ms, spread -> consecutive: FP32 8k 1.52 -> 1.36, 60k 2.05 -> 1.79, 250k
+    // 1.52 -> 1.38, 500k 5.18 -> 4.94, 1M 8.43 -> 8.37, numbered z first 18.1 ->
+    // 17.0; FP64 12k 1.07 -> 1.40, 40k 1.66 -> 1.90, 120k 3.16 -> 3.19.
+    const uint32_t W = nb * (blockDim.x >> 5);
+    const bool near_by = sizeof(R) == 4 && ntile > W;
+    const uint32_t w0 = near_by ? blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)
+                                : (threadIdx.x >> 5) * nb + blockIdx.x;
     // with subdomains the tiles of the shared bodies' sums follow the contacts'
     const uint32_t n_shared = Sub ? A.info->n_shared : 0u, ntot = ntile + (Sub ? (n_shared + 31u) / 32u : 0u);
     const bool work = w0 < ntot;
