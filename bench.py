@@ -593,11 +593,15 @@ def main():
     per_launch_ms = phase_ms["sweep_kernel"] / n_launch
     sweep_rate = phase_updates / (phase_ms["sweep_kernel"] / 1e3) if phase_ms["sweep_kernel"] > 0 else None
     peak, peak_src = read_peaks()
+    # the kernel of the schedule asked for (no flags: the dataflow sweeps)
+    flags = tuned["sweep_flags"] if tuned else (args.sweep_flags or 0)
+    kernel = ("k_solve_comp" if flags & 1 else "k_flow_comp") if comp else \
+        ("k_solve_flow" if flags == 0 else "k_solve_persistent")
     # with subdomains the traffic depends on the grid: a capture of the same
     # workload and grid only
     traffic = measured_traffic(prec, n_ss + n_sw, sweeps_launch,
                                "" if args.subdomains is None else f" subdomains {args.subdomains}",
-                               "k_solve_comp" if comp else "k_solve_persistent", args.workload)
+                               kernel, args.workload)
     achieved = alg_bytes_per_launch / (per_launch_ms / 1e3) / 1e9 if per_launch_ms > 0 else None
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": steps,
@@ -622,7 +626,7 @@ def main():
         "gpu_launches": int(round(sum(v for k, v in launches.items() if k != "sweep_kernel") * steps / n_phase)),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": (achieved / peak) if achieved else None, "traffic": traffic,
-                     "kernel": f"{'k_solve_comp' if comp else 'k_solve_persistent'}<{'float' if prec == 'fp32' else 'double'}>",
+                     "kernel": f"{kernel}<{'float' if prec == 'fp32' else 'double'}>",
                      "peak_source": f"{peak_src} (MEASURED_PEAKS.json hbm_gbs)",
                      "alg_bytes_per_launch": alg_bytes_per_launch, "launch_ms": per_launch_ms},
         "clocks": ck,

@@ -62,11 +62,17 @@ enum {                                           /* initial impulses of a solve 
     NBGS_WARM_MLP = 2    /* previous-step impulse; the network of nbgs_mlp_load for new contacts */
 };
 enum {                                           /* scheduling of the colour sweeps */
-    NBGS_SOLVER_PERSISTENT = 0,  /* one cooperative launch per solve, grid barrier between colours */
+    NBGS_SOLVER_PERSISTENT = 0,  /* one cooperative launch per solve                              */
     NBGS_SOLVER_PER_COLOUR = 1   /* one launch per colour and sweep                              */
 };
 
-enum {                                           /* nbgs_params.sweep_flags bits (persistent solver) */
+/* nbgs_params.sweep_flags bits (persistent solver).  Without any the sweeps run
+ * as a dataflow: every contact waits for the versions of its bodies that the
+ * contacts before it in colour order leave, whatever the colour, the sweep or
+ * the subdomain others are at.  The flags choose the schedules of blocks of a
+ * colour, which wait for the blocks that share bodies with them: all give the
+ * same results (composites have the dataflow and NBGS_SWEEP_GLOBAL_SYNC). */
+enum {
     NBGS_SWEEP_GLOBAL_SYNC = 1,  /* grid barrier after every colour instead of waiting only for the
                                     blocks whose contacts share bodies with this block's contacts      */
     NBGS_SWEEP_TMA_STAGE = 2,    /* stage each block's chunk of the next colour (records, impulses)
@@ -262,7 +268,7 @@ nbgs_status nbgs_batch_step(nbgs_scene* scene, int32_t max_sweeps, double tol, i
 
 /* n_steps time steps captured as CUDA graphs and replayed on the scene
  * stream, with no host synchronisation inside or between the steps (the
- * batched extension: thousands of scenes in one persistent sweep launch
+ * batched extension: thousands of scenes in one cooperative sweep launch
  * under a captured graph).  Every step does what nbgs_step(max_sweeps, tol)
  * does, with device-sized launches: the contact count stays on the device,
  * the colouring needs no host in any case, and the buffers keep
@@ -285,9 +291,9 @@ nbgs_status nbgs_graph_step(nbgs_scene* scene, int32_t max_sweeps, double tol, i
 nbgs_status nbgs_get_scene_stats(nbgs_scene* scene, int32_t* sweeps_done, double* residual);
 
 /* Autotuner: times the solve of the current contacts (state saved and
- * restored) under every sweep schedule (point-to-point or grid-barrier
- * synchronisation, with or without shared-memory staging, warp-level units,
- * two contacts gathered per thread) and 1 to the maximum resident blocks
+ * restored) under every sweep schedule (the dataflow; point-to-point or
+ * grid-barrier synchronisation, with or without shared-memory staging,
+ * warp-level units, two contacts gathered per thread) and 1 to the maximum resident blocks
  * per SM, keeps the fastest, and returns its
  * sweep_flags and blocks per SM.  Call after nbgs_detect_contacts and
  * nbgs_colour_contacts.  Synchronises. */

@@ -1,6 +1,5 @@
 // mlp_tc.cuh -- the warm-start network on the 5th-generation tensor cores
-// (tcgen05), shared by its own kernels (mlp.cu) and by the prologue of the
-// persistent sweep kernel (solve.cu): operand layouts, descriptors, the
+// (tcgen05) for the kernels of mlp.cu: operand layouts, descriptors, the
 // forward pass of a 128-row tile, and the 12 features of a contact.
 #pragma once
 #include <cuda_bf16.h>

@@ -1082,7 +1082,7 @@ static nbgs_status solve_impl(nbgs_scene* s, int max_sweeps, double tol)
             if (!(s->prm.sweep_flags & NBGS_SWEEP_GLOBAL_SYNC)) {
                 // scratch free during the solve: the colouring's body degrees and the
                 // detection's per-body counts (the body offsets adj_off stay: the
-                // network's features read them in the kernel's prologue)
+                // network's features read them)
                 int* dmin = (int*)s->deg;
                 int* dmax = (int*)s->wall_mask;
                 cudaMemsetAsync(dmin, 0x7F, s->n * sizeof(int), st);   // large positive

@@ -13,7 +13,8 @@
 // records after the n bodies.  The sweep records name instances instead of
 // bodies, so the sweep kernels run unchanged -- contacts of one colour share
 // no body, hence no instance.  After each sweep the solver adds up the
-// instances of every body that has extras (solve.cu, inst_reduce_pass):
+// instances of every body that has extras (flow.cu, reduce_tile; with other
+// schedules solve.cu, inst_reduce_pass):
 // v <- v_acc + sum_p (instance_p - v_acc) in increasing p, and every
 // instance restarts from v -- the two message exchanges of Sect. 6.3.
 //

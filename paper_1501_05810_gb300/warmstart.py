@@ -130,7 +130,7 @@ def sweeps_to_tolerance(scene_dict, mode: str, theta=None, steps: int = 5, tol: 
     given warm start ('none', 'prev', 'mlp'), after `warm_steps` steps run
     with the previous-step warm start to reach a state with contact history.
     times: also the device time of each solve (CUDA events around
-    nbgs_solve_nbgs: the network's prologue, fused into the sweep kernel, and
+    nbgs_solve_nbgs: the network's kernel before the sweeps, and
     the sweeps), in ms."""
     import torch
     sc = dict(scene_dict)
@@ -249,7 +249,7 @@ def hopper_evaluation(n: int = 2_000_000, settle_steps: int = 600, settle_sweeps
             nnew.append(int(np.count_nonzero(np.all(f[:, 3:6] == 0.0, axis=1))) if len(f) else 0)
             ncon.append(int(len(f)))
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            e0.record(s.stream)   # the solve: the network's prologue (fused into the sweep kernel) and the sweeps
+            e0.record(s.stream)   # the solve: the network's prologue and the sweeps
             k, r = s.solve_nbgs(max_sweeps, tol)
             e1.record(s.stream)
             s.integrate()
