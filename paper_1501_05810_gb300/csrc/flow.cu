@@ -702,8 +702,10 @@ nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm)
     A.n = n;
     // the state-transfer staging buffer (13 doubles per body) holds the
     // versioned records and the masses during a solve; with subdomains the
-    // velocity records, which have room for the instances, are versioned in place
-    const bool sub = s->prm.subdomain_mode != NBGS_SUB_NONE && !s->batch;
+    // velocity records, which have room for the instances, are versioned in
+    // place.  Without contacts no instances are assigned (run_colour), and the
+    // subdomain arrays hold an earlier step's or do not exist yet.
+    const bool sub = s->prm.subdomain_mode != NBGS_SUB_NONE && !s->batch && s->n_contacts > 0;
     A.nrec = (uint32_t)(sub ? n + s->icap : n);
     A.tv = sub ? (uint4*)s->vel : (uint4*)s->stage;
     typename Mass2<R>::T* mass =
