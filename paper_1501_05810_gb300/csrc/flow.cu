@@ -422,7 +422,11 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         scene = nscene;
     }
     if (Sub) at.T = w0;
-    if (Vote && !work) return;
+    if (Vote && !work) {
+        // no tile at all: nobody else says that every sweep has run
+        if (w0 == 0u && lane == 0) A.info->sweeps_done = (uint32_t)A.max_sweeps;
+        return;
+    }
     // the tolerance as a residual in R, and where the FP64 division is not needed to tell
     const R near = Vote ? (R)(A.tol * vref) : R(0), slack = sizeof(R) == 4 ? R(1e-5) : R(1e-12);
     const bool clear = near > R(1e-15) && near < R(1e15);

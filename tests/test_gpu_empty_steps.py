@@ -39,3 +39,31 @@ def test_subdomain_steps_without_contacts(oracle_mod, sub, precision, rel):
         for k in ("vel", "angvel"):
             assert np.abs(x[k] - y[k]).max() <= rel * np.abs(y[k]).max()
     g.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("tol", [0.0, 1e-6])
+def test_graph_step_without_contacts_has_its_own_outcome(precision, tol):
+    """A replayed step that loses every contact reports what an ordinary step
+    does: all sweeps, residual 0, not the outcome of the step before."""
+    import ctypes
+    from paper_1501_05810_gb300 import nbgs
+
+    def outcome(g):
+        k, r = ctypes.c_int32(), ctypes.c_double()
+        nbgs._call(g.h, "nbgs_get_scene_stats", ctypes.byref(k), ctypes.byref(r))
+        return k.value, r.value, g.residual_history().tolist()
+    sc = _scene(precision=precision)
+    a, b = nbgs.Scene(sc), nbgs.Scene(sc)
+    for spacing, sweeps in ((0.999, 30), (0.999, 30), (3.0, 30), (0.999, 30), (3.0, 7)):
+        for g in (a, b):
+            g.update_bodies(_cube(spacing), None, sc["vel"], sc["angvel"])
+        sa = a.step(sweeps, tol)
+        if b.get_contacts()["j1"].size == 0 and sa["n_contacts"] > 0:
+            b.step(sweeps, tol)      # sizes the buffers, or finds the contacts again
+        else:
+            b.graph_step(sweeps, tol, 1)
+        assert (sa["n_contacts"] > 0) == (spacing < 1.0)
+        assert outcome(a) == outcome(b)
+    a.close()
+    b.close()
