@@ -133,13 +133,23 @@ __device__ __forceinline__ void scene_max(unsigned long long* rk, uint32_t scene
     }
 }
 
+// What the sweeps start from.  The sweep count is theirs to write, but where
+// there is no contact a kernel with votes by warps has nobody to do it.
+__device__ __forceinline__ void flow_begin(DevInfo* info, int max_sweeps)
+{
+    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+    info->sweeps_done = (uint32_t)max_sweeps;
+}
+
 // Gravity, versions 0 and the mass array; of batched scenes (nscene > 0) also
 // what their contacts ask for.
 template <class R>
 __global__ void k_flow_init(int64_t n, const R4<R>* __restrict__ vel, R gx, R gy, R gz, uint4* __restrict__ tv,
                             typename Mass2<R>::T* __restrict__ mass, int64_t nscene, const double* __restrict__ mu,
-                            const double* __restrict__ vref, double tol, R4<R>* __restrict__ par)
+                            const double* __restrict__ vref, double tol, R4<R>* __restrict__ par, DevInfo* info,
+                            int max_sweeps)
 {
+    flow_begin(info, max_sweeps);
     for (int64_t sc = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; sc < nscene; sc += (int64_t)gridDim.x * blockDim.x) {
         R4<R> q;
         q.x = (R)mu[sc];
@@ -170,6 +180,7 @@ __global__ void k_flow_init(int64_t n, const R4<R>* __restrict__ vel, R gx, R gy
 template <class R>
 __global__ void k_flow_init_sub(FlowArgs<R> A, R4<R>* vel, R gx, R gy, R gz, typename Mass2<R>::T* __restrict__ mass)
 {
+    flow_begin(A.info, A.max_sweeps);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < A.n; i += (int64_t)gridDim.x * blockDim.x) {
         R4<R> v = vel[2 * i], w = vel[2 * i + 1];
         typename Mass2<R>::T m;
@@ -422,11 +433,7 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         scene = nscene;
     }
     if (Sub) at.T = w0;
-    if (Vote && !work) {
-        // no tile at all: nobody else says that every sweep has run
-        if (w0 == 0u && lane == 0) A.info->sweeps_done = (uint32_t)A.max_sweeps;
-        return;
-    }
+    if (Vote && !work) return;
     // the tolerance as a residual in R, and where the FP64 division is not needed to tell
     const R near = Vote ? (R)(A.tol * vref) : R(0), slack = sizeof(R) == 4 ? R(1e-5) : R(1e-12);
     const bool clear = near > R(1e-15) && near < R(1e15);
@@ -752,7 +759,7 @@ nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm)
         k_flow_init_sub<R><<<gb, T, 0, st>>>(A, (R4<R>*)s->vel, gx, gy, gz, mass);
     else
         k_flow_init<R><<<gb, T, 0, st>>>(n, (const R4<R>*)s->vel, gx, gy, gz, A.tv, mass, A.nscene, s->scene_mu,
-                                         s->scene_vref, tol, (R4<R>*)s->scene_par);
+                                         s->scene_vref, tol, (R4<R>*)s->scene_par, s->info, max_sweeps);
     void* args[] = {&A};
     if (s->timing) cudaEventRecord(s->ev[8], st);
     const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(nblocks), dim3(threads), args, 0, st);
