@@ -559,8 +559,10 @@ __global__ void k_comp_records(int64_t C, int64_t nm, const uint32_t* __restrict
 template <class R>
 __global__ void k_comp_velinit(int64_t nb, const double4_32a* __restrict__ bquat, const double* __restrict__ bI0,
                                const double* __restrict__ bIinv, const double* __restrict__ binvm, double3 gdt,
-                               double dt, R4<R>* __restrict__ bvel, uint4* __restrict__ tv)
+                               double dt, R4<R>* __restrict__ bvel, uint4* __restrict__ tv, DevInfo* info)
 {
+    // more colours needed than there are: the dataflow relaxes nothing (flow_begin of flow.cu)
+    if (tv && blockIdx.x == 0 && threadIdx.x == 0 && (info->err & kErrColours) != 0u) info->n_colours = 0u;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nb; i += (int64_t)gridDim.x * blockDim.x) {
         R4<R> v = bvel[4 * i], w = bvel[4 * i + 1];
         if (!(binvm[i] > 0.0)) {
@@ -1133,7 +1135,7 @@ nbgs_status solve_comp_impl(nbgs_scene* s, int max_sweeps, double tol)
     const bool flow = s->n_contacts > 0 && !(s->prm.sweep_flags & NBGS_SWEEP_GLOBAL_SYNC);
     uint4* tv = flow ? (uint4*)s->stage : nullptr;
     k_comp_velinit<R><<<grid_for(s->nb, T, 8, s->num_sms), T, 0, st>>>(s->nb, s->bquat, s->bI0, s->bIinv, s->binvm, gdt,
-                                                                       s->prm.dt, (R4<R>*)s->bvel, tv);
+                                                                       s->prm.dt, (R4<R>*)s->bvel, tv, s->info);
     CompArgs<R> A;
     A.tv = tv;
     A.C = s->n_contacts;

@@ -135,10 +135,14 @@ __device__ __forceinline__ void scene_max(unsigned long long* rk, uint32_t scene
 
 // What the sweeps start from.  The sweep count is theirs to write, but where
 // there is no contact a kernel with votes by warps has nobody to do it.
+// Contacts that found no colour of their own (kErrColours) share the last one:
+// no order of versions holds for them, and the solve is an error already, so
+// nothing is relaxed.  (Both here: in k_solve_flow they cost box-sized scenes 1 %.)
 __device__ __forceinline__ void flow_begin(DevInfo* info, int max_sweeps)
 {
     if (blockIdx.x != 0 || threadIdx.x != 0) return;
     info->sweeps_done = (uint32_t)max_sweeps;
+    if ((info->err & kErrColours) != 0u) info->n_colours = info->n_shared = 0u;
 }
 
 // Gravity, versions 0 and the mass array; of batched scenes (nscene > 0) also

@@ -1,0 +1,49 @@
+"""States that a step must refuse: what the solve does when the colouring or
+the detection has reached a limit, and what the caller is told."""
+import numpy as np
+import pytest
+
+from paper_1501_05810_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def _hub(n, r_shell=2.05, **params):
+    """A sphere of radius 2 (the last body) in a shell of n small ones at r_shell."""
+    d = np.random.default_rng(n).normal(size=(n, 3))
+    pos = np.concatenate([d / np.linalg.norm(d, axis=1, keepdims=True) * r_shell, np.zeros((1, 3))]) + 5.0
+    prm = scenes.default_params(dt=1e-4, tau=5e-3, gravity=(0, 0, 0), box_lo=(0.0,) * 3, box_hi=(10.0,) * 3, **params)
+    return scenes._scene("hub", prm, pos, np.zeros_like(pos), np.zeros_like(pos), np.r_[np.full(n, 0.05), 2.0],
+                         np.ones(n + 1), [])
+
+
+@pytest.mark.parametrize("kind,precision,tol", [
+    ("spheres", "fp32", 0.0), ("spheres", "fp32", 1e-3), ("spheres", "fp64", 0.0), ("spheres", "fp64", 1e-3),
+    ("grid", "fp32", 0.0), ("grid", "fp64", 1e-3), ("composite", "fp32", 0.0), ("composite", "fp64", 1e-3)])
+def test_more_colours_than_there_are(kind, precision, tol):
+    """300 contacts of one body need 300 colours: a capacity error, at once
+    (the wait for a version that never comes takes a second)."""
+    import time
+    from paper_1501_05810_gb300 import nbgs
+    sc = _hub(300, precision=precision, omega=0.5 if kind == "grid" else 1.0,
+              subdomains=(2, 2, 2) if kind == "grid" else None)
+    g = nbgs.Scene(scenes.as_composites(sc) if kind == "composite" else sc)
+    g.sync()
+    t = time.perf_counter()
+    with pytest.raises(nbgs.NBGSError, match="256 colours") as e:
+        g.step(20, tol)
+    assert time.perf_counter() - t < 0.5
+    assert e.value.status == nbgs.NBGS_ECAPACITY
+    g.close()
+
+
+def test_as_many_colours_as_there_are():
+    """256 contacts of one body, all colours in use, are solved."""
+    from paper_1501_05810_gb300 import nbgs
+    ks = []
+    for n in (230, 256):
+        g = nbgs.Scene(_hub(n, precision="fp64"))
+        st = g.step(20, 0.0)
+        ks.append((st["n_colours"], st["sweeps_done"]))
+        g.close()
+    assert ks[0][0] >= 230 and ks[0][1] == ks[1][1] == 20 and ks[1][0] == 256
