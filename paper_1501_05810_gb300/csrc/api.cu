@@ -150,6 +150,8 @@ static nbgs_status check_device_errors(nbgs_scene* s)
     const uint32_t e = s->hinfo->err;
     // causes before what may come of them
     if (e & kErrNaN) return fail(s, NBGS_ENAN, "NaN or Inf in the body state");
+    rc = check_detect_limits(s);
+    if (rc != NBGS_OK) return rc;
     if (e & kErrContacts) return fail(s, NBGS_ECAPACITY, "a graph step found more contacts than its buffers hold");
     if (e & kErrColours) return fail(s, NBGS_ECAPACITY, "more than 256 colours needed");
     if (e & kErrTimeout) return fail(s, NBGS_ETIMEOUT, "a wait on the device timed out");

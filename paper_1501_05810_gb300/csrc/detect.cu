@@ -1031,6 +1031,19 @@ static nbgs_status write_contacts(nbgs_scene* s, const GridArgs& g, DCount C)
     return cuda_check(s, cudaGetLastError(), "detect");
 }
 
+// The limits of the detection, from the host's copy of the device's error
+// bits: an ordinary step asks before it goes on, replayed ones when the host
+// next looks.
+nbgs_status check_detect_limits(nbgs_scene* s)
+{
+    const DevInfo& hi = *s->hinfo;
+    if (hi.err & kErrGrid) return fail(s, NBGS_EINVAL, "detect: a periodic axis holds fewer than 3 grid cells");
+    if (hi.err & kErrCand)
+        return fail(s, NBGS_ECAPACITY, "detect: a body has " + std::to_string(hi.cand_need) +
+                                           " hull neighbours above it (limit " + std::to_string(kCandCap) + ")");
+    return NBGS_OK;
+}
+
 nbgs_status run_detect(nbgs_scene* s)
 {
     const int64_t n = s->n;
@@ -1115,10 +1128,8 @@ nbgs_status run_detect(nbgs_scene* s)
     if (rc != NBGS_OK) return rc;
     const DevInfo& hi = *s->hinfo;
     if (hi.err & kErrNaN) return fail(s, NBGS_ENAN, "detect: NaN or Inf in the velocities");
-    if (hi.err & kErrGrid) return fail(s, NBGS_EINVAL, "detect: a periodic axis holds fewer than 3 grid cells");
-    if (hi.err & kErrCand)
-        return fail(s, NBGS_ECAPACITY, "detect: a body has " + std::to_string(hi.cand_need) +
-                                           " hull neighbours above it (limit " + std::to_string(kCandCap) + ")");
+    rc = check_detect_limits(s);
+    if (rc != NBGS_OK) return rc;
     const int64_t nc = hi.n_contacts;
     if (nc > s->ccap) {
         rc = grow_contacts(s, nc);

@@ -564,6 +564,7 @@ void dev_free(nbgs_scene* s, void* p);
 
 // phases (detect.cu / colour.cu / solve.cu / integrate.cu)
 nbgs_status run_detect(nbgs_scene* s);
+nbgs_status check_detect_limits(nbgs_scene* s);
 nbgs_status run_colour(nbgs_scene* s);
 nbgs_status run_solve(nbgs_scene* s, int max_sweeps, double tol);
 template <class R>

@@ -47,3 +47,31 @@ def test_as_many_colours_as_there_are():
         ks.append((st["n_colours"], st["sweeps_done"]))
         g.close()
     assert ks[0][0] >= 230 and ks[0][1] == ks[1][1] == 20 and ks[1][0] == 256
+
+
+@pytest.mark.parametrize("limit", ["neighbours", "cells"])
+def test_graph_steps_report_the_limits_of_the_detection(limit):
+    """Replayed steps that drive a body past 32 neighbours of higher index, or
+    the hulls past a third of a periodic box: reported like an ordinary step's."""
+    from paper_1501_05810_gb300 import nbgs
+    if limit == "neighbours":
+        sc = _hub(40, r_shell=2.2)
+        sc["params"]["dt"] = 1e-2
+        sc["vel"][:-1] = (5.0 - sc["pos"][:-1]) / 2.2   # inwards at 1
+        for k in ("pos", "vel", "angvel", "radius", "density"):
+            sc[k] = np.ascontiguousarray(sc[k][::-1])   # the big sphere first: every pair is in its list
+        status, text = nbgs.NBGS_ECAPACITY, "hull neighbours"
+    else:
+        sc = scenes.periodic_cloud(seed=1, per_side=6, gravity=(0.0, 0.0, -981.0))
+        status, text = nbgs.NBGS_EINVAL, "fewer than 3 grid cells"
+    a, b = nbgs.Scene(sc), nbgs.Scene(sc)
+    with pytest.raises(nbgs.NBGSError, match=text):
+        for _ in range(21):
+            a.step(5, 0.0)
+    b.step(5, 0.0)
+    b.graph_step(5, 0.0, 20)
+    with pytest.raises(nbgs.NBGSError, match=text) as e:
+        b.sync()
+    assert e.value.status == status
+    a.close()
+    b.close()
