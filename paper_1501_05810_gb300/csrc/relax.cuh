@@ -173,6 +173,12 @@ __device__ __forceinline__ bool recip_ok(double wn, double wt) { return wn > 1e-
 // a few).
 __device__ __forceinline__ bool above(float a, float b) { return a > b; }
 __device__ __forceinline__ bool above(double a, double b) { return __double_as_longlong(a) > __double_as_longlong(b); }
+// a > b for a >= 0 and b >= 0 or NaN, of either sign: nothing is above a NaN (the
+// limit of a separating contact under an infinite friction coefficient).
+__device__ __forceinline__ bool beyond(double a, double b)
+{
+    return (unsigned long long)__double_as_longlong(a) > (unsigned long long)__double_as_longlong(b);
+}
 // max(0, y), 0 for NaN
 __device__ __forceinline__ float clamp0(float y) { return y > 0.f ? y : 0.f; }
 __device__ __forceinline__ double clamp0(double y)

@@ -552,7 +552,7 @@ template <> struct Unit<double, 1> {
             }
             yn = clamp0(yn);
             const double lim = mu * yn, len2 = yt * yt + yo * yo;
-            if (above(len2, lim * lim)) {
+            if (beyond(len2, lim * lim)) {
                 const double sc = slide_scale(lim, len2);
                 yt *= sc;
                 yo *= sc;
@@ -704,7 +704,7 @@ template <> struct Unit<double, 4> {
             if (j == 0u) z = clamp0(z);
             const double lim = mu * from(z, 0), z2 = z * z;
             const double len2 = from(z2, 1) + from(z2, 2);
-            if (above(len2, lim * lim)) {
+            if (beyond(len2, lim * lim)) {
                 const double sc = slide_scale(lim, len2);
                 if (j != 0u) z *= sc;
             }
