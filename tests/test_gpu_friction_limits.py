@@ -53,3 +53,21 @@ def test_infinite_friction_in_every_kernel(precision, n_side):
     for u, v in ((x["vel"], y["vel"]), (x["angvel"], y["angvel"]), (p, q)):
         assert np.isfinite(v).all()
         assert np.abs(u - v).max() <= (1e-12 * np.abs(v).max() if precision == "fp64" else 0.0)
+
+
+@pytest.mark.parametrize("density", [1e-152, 1e-118, 1e-112, 1e-77, 1.0, 1e77, 1e112, 1e118, 1e140])
+def test_sliding_over_the_exponents(oracle_mod, density):
+    """Sliding impulses whose squares reach from the first subnormals to 1e280:
+    FP64 sweeps against the oracle's square root and division."""
+    from paper_1501_05810_gb300 import nbgs
+    sc = _floor(9, 0.3, "fp64")
+    sc["density"] = np.full(81, density)
+    g, o = nbgs.Scene(sc), oracle_mod.OracleScene(sc)
+    a, b = g.step(5, 0.0), o.step(5, 0.0)
+    assert a["n_contacts"] == b["n_contacts"] == 81
+    x, y, p, q = g.get_bodies(), o.get_bodies(), g.get_contacts(), o.get_contacts()
+    for u, v in ((x["vel"], y["vel"]), (x["angvel"], y["angvel"]), (p["impulse"], q["impulse"])):
+        assert np.isfinite(v).all() and np.abs(u - v).max() <= 1e-12 * np.abs(v).max()
+    slides = np.hypot(q["impulse"][:, 1], q["impulse"][:, 2]) > 0.299 * q["impulse"][:, 0]
+    assert slides.sum() > 10
+    g.close()
