@@ -219,9 +219,11 @@ __device__ __forceinline__ bool tr_step(TrainTcSmem& S, int g, uint32_t& phase)
     return __all_sync(0xffffffffu, ok) != 0;   // a warp stays together
 }
 
-// 1 / (1 + e^-z): the hardware's reciprocal and a Newton step (no error beyond
-// the last place).  z from -80 on: the step wants a finite denominator, and
-// what is below is 1e-35 either way.
+// 1 / (1 + e^-z): the hardware's approximate reciprocal (within one unit in the
+// last place) and one step of the Newton-Raphson iteration y (2 - d y), after
+// which the error is that of the last rounding (tests/test_reciprocal_method.py).
+// z from -80 on: the step wants a finite denominator, and what is below is 1e-35
+// either way.  The library's __frcp_rn, with its branch: 1M samples 543 us, 342 this way.
 __device__ __forceinline__ float sigmoid_f(float z)
 {
     const float d = 1.f + __expf(-fmaxf(z, -80.f));
