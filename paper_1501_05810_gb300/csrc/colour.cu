@@ -284,12 +284,10 @@ constexpr uint32_t kChaseRing = 2048, kChaseRoom = 2 * kChaseThreads;   // a pas
 __device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 template <bool Wide>
-__global__ void __launch_bounds__(kChaseThreads)
-k_colour_chase(DCount Cc, const uint4* __restrict__ cpack, uint32_t* mask, uint32_t* cstate,
-               unsigned long long* meet, const uint32_t* from, const uint32_t* from_count, uint32_t* to,
-               uint32_t* to_count, int passes, DevInfo* info)
+__device__ __forceinline__ void chase(DCount Cc, const uint4* __restrict__ cpack, uint32_t* mask, uint32_t* cstate,
+                                      unsigned long long* meet, const uint32_t* from, const uint32_t* from_count,
+                                      uint32_t* to, uint32_t* to_count, int passes, DevInfo* info)
 {
-    if (Wide != (info->n_long != 0u)) return;
     extern __shared__ uint4 s_q[];                                         // kChaseRing contacts:
     uint32_t* const s_c = reinterpret_cast<uint32_t*>(s_q + kChaseRing);   // what they are, words and indices,
     uint2* const s_m = reinterpret_cast<uint2*>(s_c + kChaseRing);         // and the masks of their lists
@@ -438,6 +436,15 @@ k_colour_chase(DCount Cc, const uint4* __restrict__ cpack, uint32_t* mask, uint3
         }
         __syncthreads();
     }
+}
+
+__global__ void __launch_bounds__(kChaseThreads)
+k_colour_chase(DCount Cc, const uint4* __restrict__ cpack, uint32_t* mask, uint32_t* cstate, unsigned long long* meet,
+               const uint32_t* from, const uint32_t* from_count, uint32_t* to, uint32_t* to_count, int passes,
+               DevInfo* info)
+{
+    if (info->n_long != 0u) chase<true>(Cc, cpack, mask, cstate, meet, from, from_count, to, to_count, passes, info);
+    else chase<false>(Cc, cpack, mask, cstate, meet, from, from_count, to, to_count, passes, info);
 }
 
 // Stable counting sort of the contacts by colour, in tiles: contacts of a
@@ -700,21 +707,6 @@ __global__ void k_build_sweep(DCount Cc, int64_t n, const uint32_t* __restrict__
     }
 }
 
-template <bool Wide>
-static nbgs_status chase(nbgs_scene* s, int blocks, DCount C, const uint32_t* from, const uint32_t* from_count,
-                         uint32_t* to, uint32_t* to_count, int passes)
-{
-    const size_t smem = kChaseRing * (sizeof(uint4) + sizeof(uint32_t) + (Wide ? 0 : sizeof(uint2)));
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_colour_chase<Wide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e == cudaSuccess) {
-        k_colour_chase<Wide><<<blocks, kChaseThreads, smem, s->stream>>>(C, s->cpack, s->cmask, s->cstate, s->cmeet, from,
-                                                                         from_count, to, to_count, passes, s->info);
-        e = cudaGetLastError();
-    }
-    return cuda_check(s, e, "colour: rounds");
-}
-
 nbgs_status run_colour(nbgs_scene* s)
 {
     if (!s->detected) return fail(s, NBGS_EINVAL, "colour_contacts: call detect_contacts first");
@@ -764,22 +756,30 @@ nbgs_status run_colour(nbgs_scene* s)
                                                                               &s->info->n_long);
             k_adj_sort_long<<<8 * s->num_sms, T, 0, st>>>(s->clist[0], &s->info->n_long, s->adj_off, s->adj, s->cprio,
                                                            s->cpack);
-            // the kernel that the lists' lengths call for does the work, in
-            // turns of several passes where a block would fall far behind:
-            // colouring phase, us, 18 colours     117k  474k  717k  1.01M contacts
+            // in turns of several passes where a block would fall far behind:
+            // colouring phase, us, 18 colours     117k  474k  717k  1.01M  5.99M  18.0M contacts
             //   one turn                           171   229   280   610
-            //   7 turns of 9 passes                238   303   340   397
-            // (2.75M, 17 colours, the launches alone: 700 and 217; 5.99M: 4549 and 620)
-            const int turns = known_contacts(s) < 800000 ? 1 : kChaseTurns, passes = 9;
+            //   7 turns of 9 passes                238   303   340   397   1628   6902
+            //   12 turns of 9 passes                                       1690   5775
+            // (16 colours, 8.28M: 2345 with 7 turns, 2480 with 12; 18.0M by rounds of a
+            // launch each 5745).  Lists beyond 16 contacts, 3.16M / 8.69M: one turn 1233 /
+            // 5019, 7 turns 1048 / 3120; 1.96M of composites 1303 / 1338.
+            const int64_t known = known_contacts(s);
+            const int turns = known < 800000 ? 1 : known < 12000000 ? 7 : kChaseTurns, passes = 9;
             const int gc = grid_for(C, kChaseThreads, 3, s->num_sms);
             uint32_t* cnt = s->info->chase_count;
             cudaMemsetAsync(cnt, 0, kChaseTurns * sizeof(uint32_t), st);
-            for (int k = 0; k < turns && rc == NBGS_OK; ++k)
-                rc = chase<false>(s, gc, Cn, k ? s->clist[(k + 1) & 1] : nullptr, k ? cnt + k - 1 : nullptr,
-                                  s->clist[k & 1], k + 1 < turns ? cnt + k : nullptr, passes);
-            if (rc == NBGS_OK) rc = chase<true>(s, gc, Cn, nullptr, nullptr, s->clist[0], nullptr, 0);
+            const size_t smem = kChaseRing * (sizeof(uint4) + sizeof(uint32_t) + sizeof(uint2));
+            rc = cuda_check(s, cudaFuncSetAttribute((const void*)k_colour_chase, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    (int)smem), "colour: queues");
+            for (int k = 0; k < turns && rc == NBGS_OK; ++k) {
+                k_colour_chase<<<gc, kChaseThreads, smem, st>>>(
+                    Cn, s->cpack, s->cmask, s->cstate, s->cmeet, k ? s->clist[(k + 1) & 1] : nullptr,
+                    k ? cnt + k - 1 : nullptr, s->clist[k & 1], k + 1 < turns ? cnt + k : nullptr, passes, s->info);
+                rc = cuda_check(s, cudaGetLastError(), "colour: turns");
+            }
             if (rc != NBGS_OK) return rc;
-            if (s->timing) s->phase_launches[1] += 3 + turns;
+            if (s->timing) s->phase_launches[1] += 2 + turns;
         }
         const int64_t nbs = (C + kSortTile - 1) / kSortTile;
         if (kMaxColours * nbs > s->sort_hist_len) return fail(s, NBGS_EINVAL, "colour: histogram buffer too small");

@@ -24,7 +24,7 @@ namespace nbgs {
 constexpr int kMaxPlanes = 16;
 constexpr int kMaxColours = 256;       // a colour is 8 bits of the colouring state
 constexpr int kCandCap = 32;           // sphere candidates per body with j > i
-constexpr int kChaseTurns = 7;         // launches of the colouring at most
+constexpr int kChaseTurns = 12;        // launches of the colouring at most
 constexpr uint32_t kUncoloured = 0xFFFFFFFFu;
 constexpr uint32_t kNoList = 0xFFFFFFFFu;   // a contact end without an incidence list (wall, infinite mass)
 constexpr int kMaxSweepsHist = 4096;   // residual slots: history, 3 rotating, 4 final
