@@ -66,6 +66,16 @@ template <class R> struct Bodies {
     R4<R> va, wa, vb, wb;
 };
 
+// omega y + (1 - omega) p.  FP32: the operations fused one way, written out,
+// because the compiler fuses a plain expression differently from one kernel to
+// the next, and every schedule of the sweeps gives the same bits.
+__device__ __forceinline__ float blend(float omega, float y, float om1, float p)
+{
+    return fmaf(om1, p, __fmul_rn(omega, y));
+}
+__device__ __forceinline__ double blend(double omega, double y, double om1, double p) { return omega * y + om1 * p; }
+
+
 // Relax one contact (apply_only: add its stored impulse instead) on loaded
 // bodies: the impulse p (xyz) and the velocities in B are updated, and r_j^2
 // = |W (p_new - p_old)|^2 is returned.  False in `moves` when both masses are
@@ -118,7 +128,7 @@ __device__ __forceinline__ R relax_bodies(const SweepRec<R>& rr, R mu, R omega, 
             }
         }
         const R om1 = R(1) - omega;
-        const R pn = omega * yn + om1 * pp.x, pt = omega * yt + om1 * pp.y, po = omega * yo + om1 * pp.z;
+        const R pn = blend(omega, yn, om1, pp.x), pt = blend(omega, yt, om1, pp.y), po = blend(omega, yo, om1, pp.z);
         dn = pn - pp.x;
         dt_ = pt - pp.y;
         do_ = po - pp.z;
