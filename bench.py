@@ -593,10 +593,10 @@ def main():
     per_launch_ms = phase_ms["sweep_kernel"] / n_launch
     sweep_rate = phase_updates / (phase_ms["sweep_kernel"] / 1e3) if phase_ms["sweep_kernel"] > 0 else None
     peak, peak_src = read_peaks()
-    # the kernel of the schedule asked for (no flags: the dataflow sweeps)
+    # the kernel of the schedule asked for (no flags: the dataflow sweeps, but large FP32 Jacobi solves)
     flags = tuned["sweep_flags"] if tuned else (args.sweep_flags or 0)
     kernel = ("k_solve_comp" if flags & 1 else "k_flow_comp") if comp else \
-        ("k_solve_flow" if flags == 0 else "k_solve_persistent")
+        ("k_solve_flow" if flags == 0 and not (args.subdomains == "jacobi" and prec == "fp32") else "k_solve_persistent")
     # with subdomains the traffic depends on the grid: a capture of the same
     # workload and grid only
     traffic = measured_traffic(prec, n_ss + n_sw, sweeps_launch,

@@ -71,7 +71,9 @@ enum {                                           /* scheduling of the colour swe
  * contacts before it in colour order leave, whatever the colour, the sweep or
  * the subdomain others are at.  The flags choose the schedules of blocks of a
  * colour, which wait for the blocks that share bodies with them: all give the
- * same results (composites have the dataflow and NBGS_SWEEP_GLOBAL_SYNC). */
+ * same results (composites have the dataflow and NBGS_SWEEP_GLOBAL_SYNC).
+ * Larger FP32 solves of non-linear block Jacobi take the blocks without a flag
+ * too, which suit them better. */
 enum {
     NBGS_SWEEP_GLOBAL_SYNC = 1,  /* grid barrier after every colour instead of waiting only for the
                                     blocks whose contacts share bodies with this block's contacts      */
