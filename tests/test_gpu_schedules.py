@@ -56,3 +56,41 @@ def test_jacobi_schedules_by_size_give_the_same(shape, sweeps, tol):
     (sa, ra, ha, ba, pa), (sb, rb, hb, bb, pb) = out
     assert sa == sb and ra == rb and np.array_equal(ha, hb) and np.array_equal(pa, pb)
     assert all(np.array_equal(ba[k], bb[k]) for k in ("pos", "quat", "vel", "angvel"))
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("kind", ["single", "graph", "batch"])
+def test_bodies_without_contacts(precision, kind):
+    """Few contacts among many bodies, some without linear or any mobility: the
+    bodies that nothing touches move as under the other schedule."""
+    from paper_1501_05810_gb300 import nbgs
+    out = []
+    for flags in (0, nbgs.NBGS_SWEEP_GLOBAL_SYNC):
+        if kind == "batch":
+            g = nbgs.BatchScene(scenes.batch_scenes(9, seed=3, n_lo=50, n_hi=900, precision=precision, sweep_flags=flags,
+                                                    warm_start="prev"))
+        else:
+            g = nbgs.Scene(scenes.periodic_cloud(seed=4, per_side=16, spacing=1.1, dt=1e-2, gravity=(0.1, 0.2, -9.81),
+                                                 precision=precision, sweep_flags=flags, warm_start="prev"))
+        i, m = np.arange(g.n), 0.5
+        im, iI = np.full(g.n, 1.0 / m), np.full(g.n, 10.0 / m)
+        im[i % 5 == 0] = 0.0
+        iI[(i % 7 == 0) | (i % 10 == 0)] = 0.0
+        g.set_mass_properties(im, iI)
+        g.step(12, 1e-6)
+        if kind == "graph":
+            g.graph_step(12, 1e-6, 3)
+        else:
+            for _ in range(3):
+                g.step(12, 1e-6)
+        b, c = g.get_bodies(), g.get_contacts()
+        out.append((b, c["impulse"]))
+        hit = np.zeros(g.n, bool)
+        hit[c["j1"]] = hit[c["j2"][c["j2"] < g.n]] = True
+        assert hit.any() and (~hit).sum() > g.n // 4
+        g.close()
+    (x, p), (y, q) = out
+    rel = 0.0 if precision == "fp32" else 1e-11   # some 50 relaxations of a body, a few roundings each
+    for k in ("pos", "quat", "vel", "angvel"):
+        assert np.abs(x[k] - y[k]).max() <= rel * np.abs(y[k]).max()
+    assert np.abs(p - q).max() <= rel * np.abs(q).max()
