@@ -398,7 +398,10 @@ __global__ void k_hull(int64_t n, const R4<R>* __restrict__ vel, const double4_3
     bool bad = false;
     const float dtf = (float)dt, tauf = (float)tau;
     const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = first; i < n; i += stride) {
+    // by warps, so that the lanes with a body are known (the votes below)
+    for (int64_t i0 = first - (threadIdx.x & 31); i0 < n; i0 += stride) {
+        const int64_t i = i0 + (threadIdx.x & 31);
+        if (i >= n) break;
         R4<R> v, w;
         ld_body(vel + 2 * i, v, w);
         const double4_32a x = ld_d4(pos_r + i);
@@ -409,12 +412,14 @@ __global__ void k_hull(int64_t n, const R4<R>* __restrict__ vel, const double4_3
         // beyond FP32: NaN, Inf, or squares too large for it
         if (!(v2 <= 1e38f && w2 <= 1e38f) && !(norm2_exact<R>(v) <= 1e300 && norm2_exact<R>(w) <= 1e300)) bad = true;
         if (scene_of) {   // per-scene max |v|^2 (v_ref); the filters only save FP64 squares and atomics
-            const uint32_t sc = scene_of[i], act = __activemask();
+            const uint32_t sc = scene_of[i], act = n - i0 < 32 ? (1u << (int)(n - i0)) - 1u : 0xffffffffu;
             // a warp's bodies are mostly of one scene: only its fastest can count
-            // (all of them asked for an atomic while the maxima were still low)
+            // (all of them asked for an atomic while the maxima were still low);
+            // a NaN is nobody's maximum
             bool asks = true;
             if (__match_any_sync(act, sc) == act)
-                asks = v2 >= __uint_as_float(__reduce_max_sync(act, __float_as_uint(v2))) * (1.f - 1e-6f) - 1e-30f;
+                asks = v2 >= __uint_as_float(__reduce_max_sync(act, v2 == v2 ? __float_as_uint(v2) : 0u)) * (1.f - 1e-6f) -
+                                 1e-30f;
             unsigned long long* dst = scene_vmax + sc;
             if (asks &&
                 !((float)__longlong_as_double((long long)*(volatile unsigned long long*)dst) > v2 * (1.f + 1e-6f) + 1e-30f)) {
