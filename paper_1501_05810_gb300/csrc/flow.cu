@@ -31,7 +31,6 @@
 // launch) the earliest unfinished tile can always run.  Every wait is bounded.
 #include <algorithm>
 #include <mutex>
-#include <utility>
 #include <vector>
 
 #include "units.cuh"
@@ -654,18 +653,22 @@ __global__ void __launch_bounds__((FlowShape<R, L>::threads), (FlowShape<R, L>::
         A.info->sweeps_done = (uint32_t)(A.max_sweeps == 0 ? 0 : min(k + 1, A.max_sweeps));
 }
 
-// Resident blocks per SM of a flow kernel at a block size, looked up once.
-int flow_occ(const void* fn, int threads)
+// Resident blocks per SM of a flow kernel at a block size, looked up once per device.
+int flow_occ(int device, const void* fn, int threads)
 {
+    struct Known {
+        int device, threads, blocks;
+        const void* fn;
+    };
     static std::mutex mu;
-    static std::vector<std::pair<std::pair<const void*, int>, int>> known;
+    static std::vector<Known> known;
     std::lock_guard<std::mutex> lock(mu);
-    for (const auto& kv : known)
-        if (kv.first.first == fn && kv.first.second == threads) return kv.second;
+    for (const Known& k : known)
+        if (k.fn == fn && k.threads == threads && k.device == device) return k.blocks;
     int o = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, threads, 0);
     cudaGetLastError();
-    known.push_back({{fn, threads}, o});
+    known.push_back({device, threads, o, fn});
     return o;
 }
 
@@ -773,7 +776,7 @@ nbgs_status run_flow(nbgs_scene* s, int max_sweeps, double tol, int warm)
     A.tile = P.tile;
     const void* fn = P.fn;
     const int threads = 32 * P.warps;
-    int nblocks = std::min(flow_occ(fn, threads), P.blocks_per_sm) * s->num_sms;
+    int nblocks = std::min(flow_occ(s->device, fn, threads), P.blocks_per_sm) * s->num_sms;
     if (s->coop_blocks < s->max_coop_blocks) nblocks = std::min(nblocks, s->coop_blocks);   // set by nbgs_autotune
     if (nblocks < 1) return fail(s, NBGS_ECUDA, "solve: sweep kernel does not fit");
     const int T = 256, gb = grid_for(std::max<int64_t>(n, 1), T, 8, s->num_sms);

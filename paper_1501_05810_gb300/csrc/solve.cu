@@ -1011,21 +1011,25 @@ static SolveArgs<R> make_args(nbgs_scene* s, int max_sweeps, double tol)
 static int gather_k(int flags) { return (flags & NBGS_SWEEP_GATHER2) ? 2 : 1; }
 
 // Resident blocks per SM of one persistent sweep variant (with the shared
-// memory of the TMA stage reserved), looked up once per variant.
+// memory of the TMA stage reserved), looked up once per variant and device.
 template <class R>
-static int persist_occ(const void* fn)
+static int persist_occ(int device, const void* fn)
 {
+    struct Known {
+        int device, blocks;
+        const void* fn;
+    };
     static std::mutex mu;
-    static std::vector<std::pair<const void*, int>> known;
+    static std::vector<Known> known;
     std::lock_guard<std::mutex> lock(mu);
-    for (const auto& kv : known)
-        if (kv.first == fn) return kv.second;
+    for (const Known& k : known)
+        if (k.fn == fn && k.device == device) return k.blocks;
     int o = 0;
     const int dyn = (int)Stage<R>::BYTES;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, fn, kPersistThreads, dyn);
     cudaGetLastError();
-    known.emplace_back(fn, o);
+    known.push_back({device, o, fn});
     return o;
 }
 
@@ -1087,7 +1091,7 @@ static nbgs_status solve_impl(nbgs_scene* s, int max_sweeps, double tol)
                                                : (const void*)k_solve_persistent<R, false, false, false>);
         // every block of a cooperative launch must be resident: variants that
         // hold more contacts per thread fit fewer blocks per SM
-        const int nblocks = std::min(s->coop_blocks, persist_occ<R>(fn) * s->num_sms);
+        const int nblocks = std::min(s->coop_blocks, persist_occ<R>(s->device, fn) * s->num_sms);
         if (nblocks < 1) return fail(s, NBGS_ECUDA, "solve: persistent kernel does not fit");
         const DCount Cn = contact_count(s);
         if (A.C > 0) {
