@@ -74,9 +74,10 @@ static bool alloc_contact_arrays(nbgs_scene* s, int64_t cap)
 
 static void free_contact_arrays(nbgs_scene* s)
 {
-    void* ps[] = {s->cj1, s->cj2, s->cgeo, s->clev, s->cimp, s->cworld, s->prev_j2, s->prev_P, s->adj, s->cstate,
-                  s->cprio, s->clist[0], s->clist[1], s->cmeet, s->perm, s->inv, s->srec, s->sp, s->spre, s->cpack};
-    for (void* p : ps) dev_free(s, p);
+    // (cleared: an allocation that fails leaves the arrays after it as they are)
+    auto drop = [s](auto*&... ps) { ((dev_free(s, ps), ps = nullptr), ...); };
+    drop(s->cj1, s->cj2, s->cgeo, s->clev, s->cimp, s->cworld, s->prev_j2, s->prev_P, s->adj, s->cstate, s->cprio,
+         s->clist[0], s->clist[1], s->cmeet, s->perm, s->inv, s->srec, s->sp, s->spre, s->cpack);
 }
 
 static bool alloc_sort_temps(nbgs_scene* s)
@@ -103,6 +104,7 @@ nbgs_status grow_contacts(nbgs_scene* s, int64_t need)
     free_contact_arrays(s);
     dev_free(s, s->sort_hist);
     dev_free(s, s->scan_tmp);
+    s->sort_hist = s->scan_tmp = nullptr;
     s->ccap = cap;
     if (!alloc_contact_arrays(s, cap) || !alloc_sort_temps(s)) {
         dev_free(s, old_j2);

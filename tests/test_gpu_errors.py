@@ -75,3 +75,44 @@ def test_graph_steps_report_the_limits_of_the_detection(limit):
     assert e.value.status == status
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("refuse", [0, 1, 7, 15, 20, 21])
+def test_no_memory_for_more_contacts(refuse):
+    """The allocation that fails while the contact buffers grow: an error, and
+    every buffer is given back once."""
+    import torch
+    from paper_1501_05810_gb300 import nbgs
+    sc = scenes.hcp_packing(16, 16, 16, dt=5e-4, precision="fp32", contacts_per_body=1)
+    sc["pos"][:, :2] += 0.25
+    live, twice, left = set(), [], [None]
+    proto_a, proto_f = nbgs.nbgs_allocator._fields_[1][1], nbgs.nbgs_allocator._fields_[2][1]
+
+    def alloc(ctx, nbytes, stream):
+        if left[0] is not None:
+            left[0] -= 1
+            if left[0] < 0:
+                return None
+        p = torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0))
+        live.add(p)
+        return p
+
+    def free(ctx, p, stream):
+        if p in live:
+            live.remove(p)
+            torch.cuda.caching_allocator_delete(int(p))
+        else:
+            twice.append(p)
+
+    a = nbgs.nbgs_allocator(None, proto_a(alloc), proto_f(free))
+    arrs = [np.ascontiguousarray(sc[k], dtype=np.float64) for k in ("pos", "vel", "angvel", "radius", "density")]
+    params = nbgs.make_params(sc["params"])
+    st, h = nbgs.nbgs_create_scene(params, len(sc["radius"]), *[nbgs._ptr(x) for x in arrs], a,
+                                   torch.cuda.current_stream().cuda_stream)
+    assert st == nbgs.NBGS_OK
+    left[0] = refuse
+    with pytest.raises(nbgs.NBGSError) as e:
+        nbgs._call(h, "nbgs_detect_contacts", None)
+    assert e.value.status == nbgs.NBGS_ENOMEM
+    nbgs.library().nbgs_destroy_scene(h)
+    assert not twice and not live
