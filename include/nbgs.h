@@ -52,7 +52,7 @@ typedef enum nbgs_status {
     NBGS_ECAPACITY = 4,  /* more contacts / colours than the buffers hold        */
     NBGS_ENOTCONV = 5,   /* tolerance not reached in max_sweeps; results valid   */
     NBGS_ENAN = 6,       /* a NaN or Inf appeared in the state                   */
-    NBGS_ETIMEOUT = 7    /* a device-side wait gave up (grid barrier)            */
+    NBGS_ETIMEOUT = 7    /* a device-side wait gave up                           */
 } nbgs_status;
 
 enum { NBGS_FP64 = 0, NBGS_FP32 = 1 };           /* arithmetic of the sweeps      */

@@ -274,9 +274,10 @@ __global__ void k_adj_sort_long(const uint32_t* __restrict__ longs, const uint32
 // orders them; a pass is two memory latencies (the successors' words, the
 // swaps).  Otherwise (Wide) the masks are kept in memory, 256 colours each,
 // ordered by fences around a count of the arrivals.
+// One kernel serves both, so that no launch is there for nothing.
 //   us (ncu, cold)                            81k contacts   2.75M
 //   rounds over a list, a launch per round        326         618
-//   this, masks in memory and fences               98        1174
+//   this, masks in memory and fences, one turn     98        1174
 //   this, masks with the arrivals                  44         217
 constexpr int kChaseThreads = 512;
 constexpr uint32_t kChaseRing = 2048, kChaseRoom = 2 * kChaseThreads;   // a pass adds at most kChaseRoom

@@ -626,7 +626,7 @@ __device__ __forceinline__ bool wall_kept(const double nrm[3], double c, double4
 // Hull-intersecting pairs.  Every body (in cell order) looks at the bodies
 // behind it in its own cell and at the 13 neighbour cells ahead (after it in
 // z, y, x), so that each pair is tested once; the pair joins the list of its
-// lower body through that body's counter, and k_write_contacts puts each list
+// lower body through that body's counter, and k_write_ends puts each list
 // into ascending order.  cs[c] is the first slot of cell c for every cell
 // (cs[ncells] = n), so the cells x - 1 .. x + 1 of a (y, z) row are one
 // contiguous range; a periodic image adds one constant shift to a whole

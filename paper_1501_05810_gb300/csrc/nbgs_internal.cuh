@@ -40,7 +40,7 @@ enum : uint32_t {
     kErrCand = 1u,        // more than kCandCap neighbours above i
     kErrContacts = 2u,    // contact buffer too small
     kErrColours = 4u,     // more than kMaxColours colours
-    kErrTimeout = 8u,     // a grid barrier wait gave up
+    kErrTimeout = 8u,     // a bounded wait gave up (versions, sums, votes, barriers, windows, tensor cores)
     kErrNaN = 16u,        // NaN / Inf in velocities or positions
     kErrGrid = 32u        // periodic axis with fewer than 3 cells
 };
@@ -202,7 +202,7 @@ template <> struct __align__(16) SweepRec<double> {
     double2 ids_bias;  // (j1 | j2 << 32 bits, bias)
     double2 lev;       // (la, lb)
     double2 nxy;       // (nx, ny)
-    double2 nz_;       // (nz, unused)
+    double2 nz_;       // (nz, factor of the tangent basis -1 / (sign(nz) + nz))
 };
 
 // What the dataflow sweeps need of a contact besides its record: the masses of
@@ -472,9 +472,9 @@ struct nbgs_scene {
     uint32_t* deg = nullptr;       // n + 1
     uint32_t* adj_off = nullptr;   // n + 1
     uint32_t* adj = nullptr;       // 2 ccap
-    uint32_t* cstate = nullptr;    // (round << 8) | colour, kUncoloured before
+    uint32_t* cstate = nullptr;    // colour, kUncoloured before
     uint64_t* cprio = nullptr;
-    uint4* cpack = nullptr;        // colouring: per contact (body 1, body 2 or none, its positions in their lists)
+    uint4* cpack = nullptr;        // colouring: per contact (body 1, body 2 or none, the contact after it in the list of either)
     uint32_t* cmask = nullptr;     // colouring: 8 x 32 colour bits per body (its coloured prefix)
     unsigned long long* cmeet = nullptr;   // contacts: what the first of two arrivals leaves for the second
     uint32_t* clist[2] = {nullptr, nullptr};   // contacts: bodies with long lists, then contacts that queues give away
