@@ -871,18 +871,32 @@ nbgs_status nbgs_graph_step(nbgs_scene* s, int32_t max_sweeps, double tol, int32
             drop_graphs(s);
             return rc;
         }
-        // each capture swapped the warm-start pointers once: back where they were
+        // with a warm start each capture swapped its pointers once: back where they were
         s->g_sweeps = max_sweeps;
         s->g_tol = tol;
         s->g_ccap = s->ccap;
-        s->g_next = 0;
-        s->last_sweeps = max_sweeps;
+        s->g_row = s->row_off;
+    }
+    s->last_sweeps = max_sweeps;
+    const bool warm = s->prm.warm_start != NBGS_WARM_NONE;
+    if (warm && !s->solved && !s->counts_stale) {
+        // a replay takes its history from the contacts of the last solve; here
+        // it lies one step back (a restored checkpoint, contacts detected but
+        // not solved), or nbgs_set_bodies has ended it
+        if (s->have_prev) {
+            swap_warm_buffers(s);
+        } else {
+            nbgs_status rc = cuda_check(s, cudaMemsetAsync(s->row_off, 0, (size_t)(s->n + 1) * sizeof(uint32_t), s->stream),
+                                        "graph_step: history");
+            if (rc != NBGS_OK) return rc;
+        }
     }
     for (int32_t k = 0; k < n_steps; ++k) {
-        nbgs_status rc = cuda_check(s, cudaGraphLaunch(s->gexec[s->g_next], s->stream), "graph_step: launch");
+        // the graph that reads the history where the last step, replayed or not, has left it
+        nbgs_status rc = cuda_check(s, cudaGraphLaunch(s->gexec[s->row_off == s->g_row ? 0 : 1], s->stream),
+                                    "graph_step: launch");
         if (rc != NBGS_OK) return rc;
-        swap_warm_buffers(s);
-        s->g_next ^= 1;
+        if (warm) swap_warm_buffers(s);
     }
     s->counts_stale = true;
     return NBGS_OK;

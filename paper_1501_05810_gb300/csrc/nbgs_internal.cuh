@@ -541,7 +541,7 @@ struct nbgs_scene {
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
     int32_t g_sweeps = -1;
     double g_tol = -1.0;
-    int g_next = 0;                // graph of the next replay
+    const uint32_t* g_row = nullptr;   // row_off where graph 0 starts from (graph 1: the other of the two)
     int64_t g_ccap = -1;   // contact capacity the graphs were captured with
     bool counts_stale = false;     // graphs ran since the host last read the counts
     // timing

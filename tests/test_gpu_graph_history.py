@@ -1,0 +1,63 @@
+"""Replayed steps among other calls: a scene that replays does exactly what its
+twin does with ordinary steps, whatever was called in between."""
+import numpy as np
+import pytest
+
+from paper_1501_05810_gb300 import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def _pour(precision, warm):
+    sc = scenes.loose_pour(seed=4, n=1500, precision=precision, warm_start=warm)
+    sc["vel"] = np.random.default_rng(3).normal(0.0, 2.0, sc["vel"].shape)
+    sc["params"]["dt"] = 0.02
+    return sc
+
+
+def _same(a, b, what):
+    x, y, p, q = a.get_bodies(), b.get_bodies(), a.get_contacts(), b.get_contacts()
+    for k in ("pos", "quat", "vel", "angvel"):
+        assert np.array_equal(x[k], y[k]), (what, k)
+    for k in ("j1", "j2", "colour", "normal", "xi", "impulse"):
+        assert np.array_equal(p[k], q[k]), (what, k)
+
+
+@pytest.mark.parametrize("precision,warm", [("fp32", "prev"), ("fp64", "prev"), ("fp32", "none"), ("fp64", "none")])
+def test_replays_among_other_calls(precision, warm, tmp_path):
+    from paper_1501_05810_gb300 import nbgs
+    sc = _pour(precision, warm)
+    a, b = nbgs.Scene(sc), nbgs.Scene(sc)
+    start = a.get_bodies()
+    ops = ["graph1", "graph2", "step", "graph1", "step", "step", "graph3", "update", "graph1", "set", "graph2", "step",
+           "set", "graph1", "detect", "graph1", "graph1", "save", "step", "load", "step", "graph1", "step", "load", "graph2",
+           "zero", "graph1"]
+    for g in (a, b):
+        g.step(20, 0.0)
+    for k, op in enumerate(ops):
+        if op.startswith("graph"):
+            b.graph_step(20, 0.0, int(op[5:]))
+            for _ in range(int(op[5:])):
+                a.step(20, 0.0)
+        for i, g in enumerate((a, b)):
+            if op == "step":
+                g.step(20, 0.0)
+            elif op == "zero":
+                g.step(0, 0.0)
+            elif op == "update":
+                s = g.get_bodies()
+                g.update_bodies(s["pos"], s["quat"], 0.5 * s["vel"], s["angvel"])
+            elif op == "set":
+                g.set_bodies(start["pos"], start["quat"], start["vel"], start["angvel"])
+            elif op == "detect":
+                g.detect_contacts()
+            elif op == "save":
+                g.save_state(str(tmp_path / f"{i}.ckpt"))
+            elif op == "load":
+                g.load_state(str(tmp_path / f"{i}.ckpt"))
+        if op not in ("set", "update", "detect", "load"):
+            assert len(a.get_contacts()["j1"]) > 300
+            _same(a, b, (k, op))
+            assert np.array_equal(a.residual_history(), b.residual_history())
+    a.close()
+    b.close()
