@@ -162,7 +162,7 @@ static nbgs_status check_device_errors(nbgs_scene* s)
 
 // After graph steps the host does not know the contact counts: read them
 // (and the device's error bits) before anything else uses them.
-static nbgs_status refresh_after_graphs(nbgs_scene* s)
+nbgs_status refresh_after_graphs(nbgs_scene* s)
 {
     if (!s->counts_stale) return NBGS_OK;
     s->counts_stale = false;
@@ -206,16 +206,6 @@ bool params_valid(const nbgs_params* p)
 }  // namespace nbgs
 
 using namespace nbgs;
-
-#define NBGS_GUARD(s)                                         \
-    do {                                                      \
-        if (!(s)) return NBGS_EINVAL;                         \
-        if ((s)->status != NBGS_OK) return (s)->status;       \
-        if ((s)->counts_stale) {                              \
-            const nbgs_status guard_rc_ = refresh_after_graphs(s); \
-            if (guard_rc_ != NBGS_OK) return guard_rc_;       \
-        }                                                     \
-    } while (0)
 
 extern "C" {
 

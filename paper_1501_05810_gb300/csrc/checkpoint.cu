@@ -217,15 +217,13 @@ extern "C" {
 
 nbgs_status nbgs_save_state(nbgs_scene* s, const char* path)
 {
-    if (!s) return NBGS_EINVAL;
-    if (s->status != NBGS_OK) return s->status;
+    NBGS_GUARD(s);
     return nbgs::run_save_state(s, path);
 }
 
 nbgs_status nbgs_load_state(nbgs_scene* s, const char* path)
 {
-    if (!s) return NBGS_EINVAL;
-    if (s->status != NBGS_OK) return s->status;
+    NBGS_GUARD(s);
     return nbgs::run_load_state(s, path);
 }
 

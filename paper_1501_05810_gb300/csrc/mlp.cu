@@ -580,8 +580,7 @@ nbgs_status nbgs_mlp_adam(float* theta, const float* grad, float* m, float* v, i
 
 nbgs_status nbgs_mlp_load(nbgs_scene* s, const float* theta, int64_t count)
 {
-    if (!s) return NBGS_EINVAL;
-    if (s->status != NBGS_OK) return s->status;
+    NBGS_GUARD(s);
     if (!theta || count != kNParams) return fail(s, NBGS_EINVAL, "mlp_load: expected 9347 parameters");
     if (!s->mlp_theta) {
         s->mlp_theta = (float*)dev_alloc(s, kNParams * sizeof(float));
@@ -593,8 +592,7 @@ nbgs_status nbgs_mlp_load(nbgs_scene* s, const float* theta, int64_t count)
 
 nbgs_status nbgs_mlp_features(nbgs_scene* s, float* out, int64_t cap, int64_t* n_out)
 {
-    if (!s) return NBGS_EINVAL;
-    if (s->status != NBGS_OK) return s->status;
+    NBGS_GUARD(s);
     if (!s->coloured) return fail(s, NBGS_EINVAL, "mlp_features: detect and colour the contacts first");
     if (n_out) *n_out = s->n_contacts;
     if (!out || cap < s->n_contacts || s->n_contacts == 0) return NBGS_OK;

@@ -615,4 +615,19 @@ inline DCount contact_count(const nbgs_scene* s)
 }
 SceneView scene_view(const nbgs_scene* s);
 
+nbgs_status refresh_after_graphs(nbgs_scene* s);   // api.cu
+
 }  // namespace nbgs
+
+// Every entry point on a scene: no null scene, no scene that has failed, and the
+// counts that replayed steps left on the device (n_contacts is the buffers'
+// capacity until then).
+#define NBGS_GUARD(s)                                         \
+    do {                                                      \
+        if (!(s)) return NBGS_EINVAL;                         \
+        if ((s)->status != NBGS_OK) return (s)->status;       \
+        if ((s)->counts_stale) {                              \
+            const nbgs_status guard_rc_ = nbgs::refresh_after_graphs(s); \
+            if (guard_rc_ != NBGS_OK) return guard_rc_;       \
+        }                                                     \
+    } while (0)

@@ -273,8 +273,7 @@ nbgs_status run_get_subdomains(nbgs_scene* s, int64_t cap, uint32_t* out)
 
 extern "C" nbgs_status nbgs_get_subdomains(nbgs_scene* s, int64_t cap, uint32_t* out, int64_t* n_out)
 {
-    if (!s) return NBGS_EINVAL;
-    if (s->status != NBGS_OK) return s->status;
+    NBGS_GUARD(s);
     if (cap < 0 || (cap > 0 && !out)) return nbgs::fail(s, NBGS_EINVAL, "get_subdomains: bad arguments");
     if (n_out) *n_out = s->n_contacts;
     return nbgs::run_get_subdomains(s, cap, out);

@@ -61,3 +61,33 @@ def test_replays_among_other_calls(precision, warm, tmp_path):
             assert np.array_equal(a.residual_history(), b.residual_history())
     a.close()
     b.close()
+
+
+def test_calls_straight_after_replays(tmp_path):
+    """Calls that read the contact count, with nothing in between that has
+    brought it from the device."""
+    from paper_1501_05810_gb300 import nbgs
+    sc = _pour("fp32", "prev")
+    a, b, c = nbgs.Scene(sc), nbgs.Scene(sc), nbgs.Scene(sc)
+    for g in (a, b, c):
+        g.step(20, 0.0)
+    path = str(tmp_path / "replayed.ckpt")
+    a.step(20, 0.0)
+    b.graph_step(20, 0.0, 1)
+    b.save_state(path)                    # the contacts there are, not the capacity
+    c.graph_step(20, 0.0, 2)
+    c.load_state(path)                    # its own replays end here
+    for _ in range(2):
+        for g in (a, b, c):
+            g.step(20, 0.0)
+        _same(a, b, "saved")
+        _same(a, c, "loaded")
+    b.graph_step(20, 0.0, 1)
+    a.step(20, 0.0)
+    assert len(b.get_subdomains()) == len(a.get_contacts()["j1"])
+    b.graph_step(20, 0.0, 1)
+    for g in (a, b):                      # after a step there are no coloured contacts to compute features of
+        with pytest.raises(nbgs.NBGSError, match="detect and colour"):
+            g.mlp_features()
+        g.close()
+    c.close()
