@@ -279,7 +279,8 @@ nbgs_status nbgs_batch_step(nbgs_scene* scene, int32_t max_sweeps, double tol, i
  * more sets an error
  * bit and the next synchronising call returns NBGS_ECAPACITY (take ordinary
  * nbgs_step calls then, which grow the buffers).  The first call, and any
- * call with other max_sweeps or tol or after the buffers grew, captures the
+ * call with other max_sweeps or tol, after the buffers grew or after walls,
+ * warm start, schedule or (by a checkpoint) parameters changed, captures the
  * step first (two graphs, one for each parity of the warm-start buffers).
  * Needs one ordinary nbgs_step before (it sizes the buffers and starts the
  * warm-start history); sphere scenes or batches, the persistent solver, no

@@ -846,7 +846,11 @@ nbgs_status nbgs_graph_step(nbgs_scene* s, int32_t max_sweeps, double tol, int32
                                     "no network warm start");
     if (s->timing) return fail(s, NBGS_EINVAL, "graph_step: disable timing first");
     if (n_steps == 0) return NBGS_OK;
-    const bool fresh = s->gexec[0] && max_sweeps == s->g_sweeps && tol == s->g_tol && s->ccap == s->g_ccap;
+    // what the launches were recorded with
+    const bool fresh = s->gexec[0] && max_sweeps == s->g_sweeps && tol == s->g_tol && s->ccap == s->g_ccap &&
+                       s->coop_blocks == s->g_coop && s->r_max == s->g_rmax &&
+                       std::memcmp(&s->prm, &s->g_prm, sizeof(s->prm)) == 0 &&
+                       std::memcmp(&s->planes, &s->g_planes, sizeof(s->planes)) == 0;
     if (!fresh) {
         nbgs_status rc = refresh_after_graphs(s);
         if (rc != NBGS_OK) return rc;
@@ -865,6 +869,10 @@ nbgs_status nbgs_graph_step(nbgs_scene* s, int32_t max_sweeps, double tol, int32
         s->g_sweeps = max_sweeps;
         s->g_tol = tol;
         s->g_ccap = s->ccap;
+        s->g_coop = s->coop_blocks;
+        s->g_rmax = s->r_max;
+        std::memcpy(&s->g_prm, &s->prm, sizeof(s->prm));
+        std::memcpy(&s->g_planes, &s->planes, sizeof(s->planes));
         s->g_row = s->row_off;
     }
     s->last_sweeps = max_sweeps;

@@ -542,7 +542,11 @@ struct nbgs_scene {
     int32_t g_sweeps = -1;
     double g_tol = -1.0;
     const uint32_t* g_row = nullptr;   // row_off where graph 0 starts from (graph 1: the other of the two)
-    int64_t g_ccap = -1;   // contact capacity the graphs were captured with
+    int64_t g_ccap = -1;   // contact capacity the graphs were captured with,
+    int g_coop = 0;        // and the rest of what their launches hold by value
+    double g_rmax = 0.0;
+    nbgs_params g_prm;
+    nbgs::Planes g_planes{};
     bool counts_stale = false;     // graphs ran since the host last read the counts
     // timing
     bool timing = false;

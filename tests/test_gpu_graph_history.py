@@ -91,3 +91,40 @@ def test_calls_straight_after_replays(tmp_path):
             g.mlp_features()
         g.close()
     c.close()
+
+
+def test_replays_after_changes_of_the_scene(tmp_path):
+    """Walls, masses, warm start and parameters that change between replays."""
+    from paper_1501_05810_gb300 import nbgs
+    sc = _pour("fp32", "prev")
+    a, b = nbgs.Scene(sc), nbgs.Scene(sc)
+    other = nbgs.Scene(dict(sc, params=dict(sc["params"], mu=0.1, dt=5e-3, gravity=(3.0, 0.0, -4.0))))
+    other.step(20, 0.0)
+    other.save_state(str(tmp_path / "other.ckpt"))
+    other.close()
+    mass = 4.0 / 3.0 * np.pi * sc["radius"] ** 3
+    hi = sc["params"]["box_hi"]
+    changes = [lambda g: nbgs._call(g.h, "nbgs_add_plane", (nbgs.C.c_double * 3)(-1.0, 0.0, 0.0), 0.05 - float(hi[0])),
+               lambda g: nbgs._call(g.h, "nbgs_set_warm_start", nbgs.NBGS_WARM_NONE),
+               lambda g: g.set_mass_properties(0.5 / mass, 2.5 / (mass * sc["radius"] ** 2)),
+               lambda g: nbgs._call(g.h, "nbgs_add_plane", (nbgs.C.c_double * 3)(0.0, -1.0, 0.0), 0.05 - float(hi[1])),
+               lambda g: nbgs._call(g.h, "nbgs_set_warm_start", nbgs.NBGS_WARM_PREV),
+               lambda g: g.load_state(str(tmp_path / "other.ckpt"))]
+    for g in (a, b):
+        g.step(20, 0.0)
+    for k, change in enumerate(changes):
+        b.graph_step(20, 0.0, 2)
+        for _ in range(2):
+            a.step(20, 0.0)
+        for g in (a, b):
+            change(g)
+        if k == len(changes) - 1:   # other parameters and no solve since: an ordinary step first
+            with pytest.raises(nbgs.NBGSError):
+                b.graph_step(20, 0.0, 1)
+            break
+        a.step(20, 0.0)
+        b.graph_step(20, 0.0, 1)
+        assert len(a.get_contacts()["j1"]) > 100
+        _same(a, b, k)
+    a.close()
+    b.close()
