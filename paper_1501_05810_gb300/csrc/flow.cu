@@ -688,6 +688,7 @@ int flow_occ(int device, const void* fn, int threads)
 //   FP64, 4 lanes, 8 warps/SM    1.44    1.74    2.23    3.67    7.09
 //   FP64, 1 lane,  4 warps/SM    3.14    4.20    4.43    4.43    5.31
 //   FP64, 1 lane,  8 warps/SM    3.14    4.91    5.55    5.73    5.83
+// (FP64 since the sliding scale is rsqrt(): 2 to 4 % less up to 30k, the same above.)
 // The FP32 kernels give the same bits, so their line is drawn by what decides,
 // the contacts (256 loose scenes, 1.1M bodies with 0.6M contacts, two steps:
 // 17.1 ms with two lanes, 19.2 with one); the FP64 ones by the bodies, which

