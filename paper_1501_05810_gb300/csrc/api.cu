@@ -455,6 +455,7 @@ static nbgs_status create_common(const nbgs_params* params, const nbgs_batch_des
         nbgs_destroy_scene(s);
         return NBGS_ENOMEM;
     }
+    std::memset(s->hinfo, 0, sizeof(DevInfo));
     cudaMemsetAsync(s->info, 0, sizeof(DevInfo), s->stream);
     cudaMemsetAsync(s->vel, 0, 2 * nn * vec4_bytes(s), s->stream);
     cudaMemsetAsync(s->pos_r, 0, nn * sizeof(double4_32a), s->stream);
