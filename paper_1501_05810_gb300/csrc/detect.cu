@@ -636,7 +636,8 @@ __device__ __forceinline__ bool wall_kept(const double nrm[3], double c, double4
 // searched for both bodies of a pair, nested loops and the list in the
 // thread, 4M gas bodies took 574 us and 1M packed ones 145 (ncu, cold), this
 // way 368 and 213; the packed scene's solve takes 8 ms.  A late pile of 1M
-// composites, 16.4M pairs, 1.74 ms before and 3.74 now, of a step of 97.
+// composites, 16.4M pairs: 1.74 ms before and 1.69 now (3.74 with each lane's
+// queue worked off alone, see below).
 //
 // The search is a loop of FP32 screens over the rows' slots, run together
 // (the lanes of a warp differ in the lengths of the rows by more than in
